@@ -40,8 +40,6 @@ unsigned long long now_ns() {
       .count();
 }
 
-constexpr long kJacSplitItemsHost = 65536;  // as the single-problem Jacobian launcher
-
 // Items of one colour pass (the largest over the colours of the schedule),
 // as the kernels enumerate them.
 long sor_items_host(int Nx, int Ny, int st, int Kc) {
@@ -58,7 +56,7 @@ template <typename T>
 struct TaskPool {
   struct Group {
     std::vector<BTask2<T>> tasks;
-    size_t first = 0;
+    size_t first = 0, smem = 0;
     int blocks = 0;
   };
   std::vector<Group> groups;
@@ -66,6 +64,12 @@ struct TaskPool {
   int begin() {
     groups.emplace_back();
     return (int)groups.size() - 1;
+  }
+  void add_tiles(int g, BTask2<T> t, const Tile2Shape &sh) {
+    t.TX = sh.TX;
+    t.TY = sh.TY;
+    groups[g].smem = std::max(groups[g].smem, sh.smem);
+    add(g, t, sh.blocks);
   }
   void add(int g, BTask2<T> t, int nb) {
     t.b0 = groups[g].blocks;
@@ -86,7 +90,7 @@ template <typename T>
 struct StageData {
   TaskPool<T> pool;
   TaskPool<double> pool64;  // residual tasks (FP64 arrays whatever T)
-  int g_res = -1, g_jac[2][2] = {{-1, -1}, {-1, -1}}, g_f32 = -1, g_upd = -1;
+  int g_res = -1, g_jac[2] = {-1, -1}, g_f32 = -1, g_upd = -1;
   int g_direct_zero = -1, g_direct_scatter = -1, g_direct = -1;
   int g_vc_zero = -1, g_vc_scatter = -1, g_vc_lu = -1, g_zero_du = -1;
   std::vector<int> g_cop, g_dinv, g_sor, g_restrict, g_prolong;  // per depth
@@ -97,14 +101,14 @@ struct StageData {
   BTask2<double> *dev64 = nullptr;
   Tail2<T> *dev_tails = nullptr;
   Batch2Launch<T> launch(int g) const {
-    if (g < 0) return Batch2Launch<T>{nullptr, 0, 0};
+    if (g < 0) return Batch2Launch<T>{nullptr, 0, 0, 0};
     const auto &G = pool.groups[g];
-    return Batch2Launch<T>{dev + G.first, (int)G.tasks.size(), G.blocks};
+    return Batch2Launch<T>{dev + G.first, (int)G.tasks.size(), G.blocks, G.smem};
   }
   Batch2Launch<double> launch64(int g) const {
-    if (g < 0) return Batch2Launch<double>{nullptr, 0, 0};
+    if (g < 0) return Batch2Launch<double>{nullptr, 0, 0, 0};
     const auto &G = pool64.groups[g];
-    return Batch2Launch<double>{dev64 + G.first, (int)G.tasks.size(), G.blocks};
+    return Batch2Launch<double>{dev64 + G.first, (int)G.tasks.size(), G.blocks, G.smem};
   }
   ~StageData() {
     cudaFree(dev);
@@ -199,8 +203,7 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
     StageData<T> sd;
     // ---- the tasks of this stage
     sd.g_res = sd.pool64.begin();
-    for (int g = 0; g < 2; ++g)
-      for (int f = 0; f < 2; ++f) sd.g_jac[g][f] = sd.pool.begin();
+    for (int f = 0; f < 2; ++f) sd.g_jac[f] = sd.pool.begin();
     if (kMixed) sd.g_f32 = sd.pool.begin();
     sd.g_upd = sd.pool.begin();
     sd.g_direct_zero = sd.pool.begin();
@@ -252,7 +255,7 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
       t.A = reinterpret_cast<T *>(p->dense);
       t.x = reinterpret_cast<T *>(p->xbuf);
       t.piv = p->piv;
-      {  // residual (the block count of launch2_residual)
+      {  // residual (the tiles and block count of launch2_residual)
         BTask2<double> r;
         std::memset(&r, 0, sizeof(r));
         r.prob = i;
@@ -263,23 +266,9 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
         r.U = Lv.U;
         r.R64 = Lv.R;
         r.partials = p->partials2;
-        const int g = b2_grid(n);
-        sd.pool64.add(sd.g_res, r, g > 1024 ? 1024 : g);
+        sd.pool64.add_tiles(sd.g_res, r, tile2_residual_shape(Lv.Nx, Lv.Ny));
       }
-      {  // Jacobian: one cell per thread on large levels, else one (cell, block) item
-        const bool cells = ctx->jac2d_cell_min >= 0 && n >= ctx->jac2d_cell_min;
-        BTask2<T> j = t;
-        int nb;
-        if (cells) {
-          const int th = b2_jacobian_cell_threads();
-          nb = (n + th - 1) / th;
-        } else {
-          const long items = (long)n * K;
-          j.msplit = 3 * items <= kJacSplitItemsHost ? 1 : 0;
-          nb = b2_grid(items * (j.msplit ? 3 : 1));
-        }
-        sd.pool.add(sd.g_jac[cells ? 1 : 0][t.frozen ? 1 : 0], j, nb);
-      }
+      sd.pool.add_tiles(sd.g_jac[t.frozen ? 1 : 0], t, tile2_jacobian_shape(Lv.Nx, Lv.Ny, st0));
       if (kMixed) sd.pool.add(sd.g_f32, t, b2_grid(3L * n));
       sd.pool.add(sd.g_upd, t, b2_grid(n));
       if (l == L) {  // Newton on the coarsest grid: dense LU of the regularized system
@@ -440,10 +429,8 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
       cudaError_t e;
       if ((e = cudaMemcpyAsync(done, done_h, sizeof(int) * count, cudaMemcpyHostToDevice, q))) return e;
       if ((e = cudaMemsetAsync(flags, 0, sizeof(int) * count, q))) return e;
-      for (int g = 0; g < 2; ++g)
-        for (int f = 0; f < 2; ++f)
-          if ((e = launchb2_jacobian<T>(sd.launch(sd.g_jac[g][f]), done, g ? kB2JacCells : kB2JacItems, f == 1, q)))
-            return e;
+      for (int f = 0; f < 2; ++f)
+        if ((e = launchb2_jacobian<T>(sd.launch(sd.g_jac[f]), done, f == 1, q))) return e;
       if constexpr (kMixed) {
         if ((e = launchb2_to_f32(sd.launch(sd.g_f32), done, q))) return e;
       }

@@ -349,7 +349,7 @@ nswe_status solve2d_t(nswe_prob_s *p, const double *U0, double *U, const nswe_pa
     if (l < s0 && launch2_interp(p->dev2, l + 1, p->host2.lev[l + 1].Nx * p->host2.lev[l + 1].Ny,
                                  p->host2.lev[l + 1].U, Lv.U, s))
       return NSWE_ECUDA;
-    if (launch2_residual(p->dev2, l, n, Lv.U, Lv.R, p->res_dev, p->partials2, s)) return NSWE_ECUDA;
+    if (launch2_residual(p->dev2, l, Lv.Nx, Lv.Ny, Lv.U, Lv.R, p->res_dev, p->partials2, s)) return NSWE_ECUDA;
     // One Newton step of this level (Eq. 12-14 with Algorithm 2): the same
     // launches every iteration, so they are captured once into a CUDA graph
     // and replayed; the host only waits for the residual and the flag.
@@ -364,8 +364,7 @@ nswe_status solve2d_t(nswe_prob_s *p, const double *U0, double *U, const nswe_pa
     T *const Rs = kMixed ? J + (size_t)K * 9 * blk_stride(cm, Lv.Nx, Lv.Ny) : reinterpret_cast<T *>(Lv.R);
     auto step = [&](cudaStream_t q) -> cudaError_t {
       cudaError_t e;
-      if ((e = launch2_jacobian<T>(p->dev2, l, n, st0, Lv.U, prm.eps[l], prm.alpha, Lv.R, J, frozen, cm,
-                                   p->ctx->jac2d_cell_min, q)))
+      if ((e = launch2_jacobian<T>(p->dev2, l, Lv.Nx, Lv.Ny, st0, Lv.U, prm.eps[l], prm.alpha, Lv.R, J, frozen, cm, q)))
         return e;
       if constexpr (kMixed) {
         if ((e = launch2_to_f32(3L * n, Lv.R, reinterpret_cast<float *>(Rs), q))) return e;
@@ -384,7 +383,7 @@ nswe_status solve2d_t(nswe_prob_s *p, const double *U0, double *U, const nswe_pa
           if ((e = mg2_vcycle<T>(p, m, prm, q, tail))) return e;
       }
       if ((e = launch2_update<T>(n, Lv.U, dU, prm.tau, p->flag, q))) return e;
-      if ((e = launch2_residual(p->dev2, l, n, Lv.U, Lv.R, p->res_dev, p->partials2, q))) return e;
+      if ((e = launch2_residual(p->dev2, l, Lv.Nx, Lv.Ny, Lv.U, Lv.R, p->res_dev, p->partials2, q))) return e;
       if ((e = cudaMemcpyAsync(p->res_host, p->res_dev, sizeof(double), cudaMemcpyDeviceToHost, q))) return e;
       return cudaMemcpyAsync(p->flag_host, p->flag, sizeof(int), cudaMemcpyDeviceToHost, q);
     };
@@ -629,9 +628,8 @@ nswe_status nswe_ctx_set_batch_2d(nswe_ctx ctx, int mode) {
 }
 
 nswe_status nswe_ctx_set_jacobian_cells_2d(nswe_ctx ctx, int min_cells) {
-  if (!ctx) return NSWE_EINVAL;
-  ctx->jac2d_cell_min = min_cells;
-  return NSWE_OK;
+  (void)min_cells;  // one kernel serves every level size
+  return ctx ? NSWE_OK : NSWE_EINVAL;
 }
 
 nswe_status nswe_ctx_set_stream(nswe_ctx ctx, void *stream) {
@@ -944,7 +942,7 @@ nswe_status nswe_residual(nswe_ctx ctx, nswe_prob prob, int level, const double 
   if (!ctx || !prob || prob->ctx != ctx || !U || !R || level < 0 || level >= prob->levels) return NSWE_EINVAL;
   DeviceGuard dg(ctx->device);
   if (prob->dim == 2)
-    return launch2_residual(prob->dev2, level, nswe_prob_cells(prob, level), U, R, res_l1, ctx->partials,
+    return launch2_residual(prob->dev2, level, prob->Nx >> level, prob->Ny >> level, U, R, res_l1, ctx->partials,
                             ctx->stream) == cudaSuccess
                ? NSWE_OK
                : NSWE_ECUDA;
@@ -960,10 +958,10 @@ static nswe_status jacobian_common(nswe_ctx ctx, nswe_prob prob, int level, int 
   if (!(eps > 0.0) || !std::isfinite(eps) || !(alpha >= 0.0) || !std::isfinite(alpha)) return NSWE_EINVAL;
   DeviceGuard dg(ctx->device);
   if (prob->dim == 2) {
-    const int n = nswe_prob_cells(prob, level);
-    if (launch2_residual(prob->dev2, level, n, U, R, res, ctx->partials, ctx->stream) ||
-        launch2_jacobian<double>(prob->dev2, level, n, nb == 5 ? ST_J21 : ST_J9, U, eps, alpha, R, J, frozen, 0,
-                                 ctx->jac2d_cell_min, ctx->stream))
+    const int Nx = prob->Nx >> level, Ny = prob->Ny >> level;
+    if (launch2_residual(prob->dev2, level, Nx, Ny, U, R, res, ctx->partials, ctx->stream) ||
+        launch2_jacobian<double>(prob->dev2, level, Nx, Ny, nb == 5 ? ST_J21 : ST_J9, U, eps, alpha, R, J, frozen, 0,
+                                 ctx->stream))
       return NSWE_ECUDA;
     return NSWE_OK;
   }
@@ -997,10 +995,10 @@ nswe_status nswe_jacobian_f32(nswe_ctx ctx, nswe_prob prob, int level, int nb, c
   DeviceGuard dg(ctx->device);
   if (prob->dim == 2) {
     if (nb != 9 && nb != 21) return NSWE_EINVAL;
-    const int n = nswe_prob_cells(prob, level);
-    return (launch2_residual(prob->dev2, level, n, U, R, res_l1, ctx->partials, ctx->stream) ||
-            launch2_jacobian<float>(prob->dev2, level, n, nb == 21 ? ST_J21 : ST_J9, U, eps, alpha, R, J, false, 0,
-                                    ctx->jac2d_cell_min, ctx->stream))
+    const int Nx = prob->Nx >> level, Ny = prob->Ny >> level;
+    return (launch2_residual(prob->dev2, level, Nx, Ny, U, R, res_l1, ctx->partials, ctx->stream) ||
+            launch2_jacobian<float>(prob->dev2, level, Nx, Ny, nb == 21 ? ST_J21 : ST_J9, U, eps, alpha, R, J, false, 0,
+                                    ctx->stream))
                ? NSWE_ECUDA
                : NSWE_OK;
   }
@@ -1115,8 +1113,8 @@ nswe_status autotune2d_t(nswe_ctx ctx, nswe_prob prob, const double *U, const ns
       cudaEventCreate(&e1))
     status = NSWE_ENOMEM;
   if (status == NSWE_OK &&
-      (launch2_residual(prob->dev2, 0, n, U, R64, nullptr, prob->partials2, s) ||
-       launch2_jacobian<T>(prob->dev2, 0, n, st, U, prm.eps[0], prm.alpha, R64, J, frozen, 0, ctx->jac2d_cell_min, s)))
+      (launch2_residual(prob->dev2, 0, prob->Nx, prob->Ny, U, R64, nullptr, prob->partials2, s) ||
+       launch2_jacobian<T>(prob->dev2, 0, prob->Nx, prob->Ny, st, U, prm.eps[0], prm.alpha, R64, J, frozen, 0, s)))
     status = NSWE_ECUDA;
   if (status == NSWE_OK) {
     if constexpr (std::is_same<T, float>::value) {

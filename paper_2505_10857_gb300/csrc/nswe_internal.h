@@ -92,7 +92,17 @@ struct ProbDev2 {
   Level2Dev lev[NSWE_MAX_LEVELS];
 };
 
-cudaError_t launch2_residual(const ProbDev2 *p, int level, int n, const double *U, double *R, double *res,
+// Tiles of the residual and the Jacobian of a level (nswe_tile2d.cuh): cells
+// per tile, blocks of the launch and their dynamic shared memory.
+struct Tile2Shape {
+  int TX, TY, blocks;
+  size_t smem;
+};
+constexpr int kTile2MaxSmem = 225 * 1024;
+constexpr int kSmCount = 152;  // SMs of a GB300
+Tile2Shape tile2_residual_shape(int Nx, int Ny);
+Tile2Shape tile2_jacobian_shape(int Nx, int Ny, int st);
+cudaError_t launch2_residual(const ProbDev2 *p, int level, int Nx, int Ny, const double *U, double *R, double *res,
                              double *partials, cudaStream_t s);
 // Multigrid launchers for T = double (FP64 path) and T = float (the multigrid
 // of a mixed-precision step); the Jacobian may be stored in either.
@@ -110,13 +120,10 @@ __host__ __device__ __forceinline__ size_t blk_pos(int cm, int Nx, int Ny, int i
 }
 
 // frozen: the frozen linearisation (weights and eigenvectors from U); cm:
-// the storage of J (blk_pos); levels of at least cell_min cells (>= 0) take
-// the one-cell-per-thread kernel, the others one (cell, block) item per
-// thread (the same bits either way).
-constexpr int kJac2CellMinDefault = 32768;
+// the storage of J (blk_pos).
 template <typename TJ>
-cudaError_t launch2_jacobian(const ProbDev2 *p, int level, int n, int st, const double *U, double eps, double alpha,
-                             const double *R, TJ *J, bool frozen, int cm, int cell_min, cudaStream_t s);
+cudaError_t launch2_jacobian(const ProbDev2 *p, int level, int Nx, int Ny, int st, const double *U, double eps,
+                             double alpha, const double *R, TJ *J, bool frozen, int cm, cudaStream_t s);
 template <typename T>
 cudaError_t launch2_coarse_op(int Nx, int Ny, int st, const T *Jf, T *Jc, int cm, cudaStream_t s);
 template <typename T>
@@ -186,7 +193,7 @@ struct BTask2 {
   T *J, *Dinv, *R, *dU;  // its multigrid arrays (R: the right-hand side in T)
   T *Jc, *Rc, *dUc;      // the next coarser level's: Galerkin operator, restriction, prolongation
   const ProbDev2 *P;     // residual / Jacobian / update: the problem and its nested level
-  int level, frozen, msplit;
+  int level, frozen, TX, TY;  // TX x TY: the tile of a residual or Jacobian task
   double *U, *R64;       // state and FP64 residual of the Newton level
   double *partials;      // residual partial sums (nb of them)
   float *R32;            // FP32 copy of R64 (mixed precision)
@@ -201,12 +208,11 @@ template <typename T>
 struct Batch2Launch {
   const BTask2<T> *tasks;
   int ntask, blocks;
+  size_t smem;  // residual and Jacobian: dynamic shared memory, the largest of the tasks' tiles
 };
 cudaError_t launchb2_residual(const Batch2Launch<double> &b, const int *done, double *res, cudaStream_t s);
 template <typename TJ>
-cudaError_t launchb2_jacobian(const Batch2Launch<TJ> &b, const int *done, int kind, bool frozen, cudaStream_t s);
-constexpr int kB2JacItems = 0, kB2JacCells = 1;  // launchb2_jacobian kinds
-int b2_jacobian_cell_threads();
+cudaError_t launchb2_jacobian(const Batch2Launch<TJ> &b, const int *done, bool frozen, cudaStream_t s);
 cudaError_t launchb2_to_f32(const Batch2Launch<float> &b, const int *done, cudaStream_t s);
 template <typename T>
 cudaError_t launchb2_zero_du(const Batch2Launch<T> &b, const int *done, cudaStream_t s);
@@ -329,7 +335,6 @@ struct nswe_ctx_s {
   int team_cells = 1024; // cluster form: multigrid levels with at least this many cells on every CTA
   int batch2d_lockstep = 1;  // 2D batches: 1 lockstep batched launches (default), 0 concurrent solves
   int cm2d_min_cells = 131072;  // 2D Newton levels of at least this many cells store J9 colour-major
-  int jac2d_cell_min = nswe::kJac2CellMinDefault;  // 2D levels from which the per-cell Jacobian kernel runs
   // 2D V-cycles: levels of at most tail2[precision] cells run in the one-block tail (0 FP64, 1 mixed)
   int tail2[2] = {nswe::tail2_cells<double>(), nswe::tail2_cells<float>()};
   std::vector<nswe_tuned2d> tuned2;  // nswe_autotune_2d's choices per size and precision

@@ -13,6 +13,7 @@
 #include <type_traits>
 #include <utility>
 
+#include "nswe_fp64.cuh"
 #include "nswe_internal.h"
 
 namespace nswe {
@@ -90,280 +91,6 @@ __device__ __forceinline__ Geo2 make_geo2(const ProbDev2 &P, int l) {
 #define NSWE_SOR_UNROLL 1
 #endif
 constexpr long kSorSplitF64 = NSWE_SOR_SPLIT_F64, kSorSplitF32 = NSWE_SOR_SPLIT_F32;
-// Largest number of (cell, block, component) items for which the Jacobian
-// takes one component per item.
-#ifndef NSWE_JAC_SPLIT_ITEMS
-#define NSWE_JAC_SPLIT_ITEMS 65536
-#endif
-constexpr long kJacSplitItems = NSWE_JAC_SPLIT_ITEMS;
-
-// Perturbation of one interior cell in one component (cp < 0: none).
-struct Pert {
-  int cp, m;
-  double eps;
-};
-
-__device__ __forceinline__ void bc_post(int kind, const double *st, double o[3], int normal) {
-  if (kind == NSWE_BC2_REFLECT) {
-    o[normal] = -o[normal];
-  } else if (kind == NSWE_BC2_DISCHARGE) {
-    o[1] = st[1];
-    o[2] = st[2];
-  } else if (kind == NSWE_BC2_DEPTH) {
-    o[0] = st[0];
-  }
-}
-
-// Cell value with two ghost layers (x rule, then y rule at corners).
-__device__ __forceinline__ void cellv(const Geo2 &G, const double *U, int i, int j, const Pert &p, double o[3]) {
-  const int Nx = G.Nx, Ny = G.Ny, n = Nx * Ny;
-  int xk = 0, xs = 0;
-  if (i < 0 || i >= Nx) {
-    xs = i < 0 ? 0 : 1;
-    xk = G.bck[xs * Ny + min(max(j, 0), Ny - 1)];
-    if (xk == NSWE_BC2_INFLOW) {
-      o[0] = G.bcs[xs * 3];
-      o[1] = G.bcs[xs * 3 + 1];
-      o[2] = G.bcs[xs * 3 + 2];
-      return;
-    }
-    i = (xk == NSWE_BC2_REFLECT) ? (i < 0 ? -1 - i : 2 * Nx - 1 - i) : (i < 0 ? 0 : Nx - 1);
-  }
-  if (j < 0 || j >= Ny) {
-    const int ys = j < 0 ? 2 : 3;
-    const int yk = G.bck[2 * Ny + (ys - 2) * Nx + i];
-    if (yk == NSWE_BC2_INFLOW) {
-      o[0] = G.bcs[ys * 3];
-      o[1] = G.bcs[ys * 3 + 1];
-      o[2] = G.bcs[ys * 3 + 2];
-    } else {
-      const int jj = (yk == NSWE_BC2_REFLECT) ? (j < 0 ? -1 - j : 2 * Ny - 1 - j) : (j < 0 ? 0 : Ny - 1);
-      const int c = jj * Nx + i;
-#pragma unroll
-      for (int m = 0; m < 3; ++m) o[m] = (c == p.cp && m == p.m) ? U[m * n + c] + p.eps : U[m * n + c];
-      bc_post(yk, G.bcs + ys * 3, o, 2);
-    }
-  } else {
-    const int c = j * Nx + i;
-#pragma unroll
-    for (int m = 0; m < 3; ++m) o[m] = (c == p.cp && m == p.m) ? U[m * n + c] + p.eps : U[m * n + c];
-  }
-  if (xk) bc_post(xk, G.bcs + xs * 3, o, 1);
-}
-
-__device__ __forceinline__ void weno3_both(double a, double b, double c, double &up, double &um) {
-  double d0 = c - b, d1 = b - a;
-  double e0 = kZeta2 + d0 * d0, e1 = kZeta2 + d1 * d1;
-  double s0 = e0 * e0, s1 = e1 * e1;
-  double p0 = 1.5 * b - 0.5 * c, p1 = 0.5 * a + 0.5 * b;
-  double q0 = 0.5 * b + 0.5 * c, q1 = -0.5 * a + 1.5 * b;
-  double D1 = s1 + 2.0 * s0, D2 = 2.0 * s1 + s0;
-  double inv = 1.0 / (D1 * D2);
-  up = (s1 * p0 + 2.0 * s0 * p1) * (D2 * inv);
-  um = (2.0 * s1 * q0 + s0 * q1) * (D1 * inv);
-}
-
-// WENO3 of the values (a, b, c) with the nonlinear weights of (a0, b0, c0):
-// the frozen linearisation's reconstruction (weights as in weno3_both).
-__device__ __forceinline__ void weno3_fixed(double a0, double b0, double c0, double a, double b, double c,
-                                            double &up, double &um) {
-  double d0 = c0 - b0, d1 = b0 - a0;
-  double e0 = kZeta2 + d0 * d0, e1 = kZeta2 + d1 * d1;
-  double s0 = e0 * e0, s1 = e1 * e1;
-  double p0 = 1.5 * b - 0.5 * c, p1 = 0.5 * a + 0.5 * b;
-  double q0 = 0.5 * b + 0.5 * c, q1 = -0.5 * a + 1.5 * b;
-  double D1 = s1 + 2.0 * s0, D2 = 2.0 * s1 + s0;
-  double inv = 1.0 / (D1 * D2);
-  up = (s1 * p0 + 2.0 * s0 * p1) * (D2 * inv);
-  um = (2.0 * s1 * q0 + s0 * q1) * (D1 * inv);
-}
-
-// One-sided characteristic WENO3 at the interface between line cells a and
-// a+1; v[0..3] = cells a-1..a+2; side 0: U^-, side 1: U^+. FROZEN: the
-// eigenvectors and the nonlinear weights come from b, the unperturbed values
-// of the same cells (b is not read otherwise).
-template <bool FROZEN>
-__device__ __forceinline__ void char_rec(int dir, const double v[4][3], const double b[4][3], double g, int side,
-                                         double out[3]) {
-  const int in = dir == 0 ? 1 : 2, it = dir == 0 ? 2 : 1;
-  const double(*r)[3] = FROZEN ? b : v;
-  const double h = 0.5 * (r[1][0] + r[2][0]);
-  const double ih = 1.0 / h;
-  const double un = 0.5 * (r[1][in] + r[2][in]) * ih, ut = 0.5 * (r[1][it] + r[2][it]) * ih;
-  const double c = sqrt(g * h), i2c = 0.5 / c;
-  double W[3][3], Wb[3][3];
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    const double *u = v[side + s];
-    W[s][0] = (un + c) * i2c * u[0] - i2c * u[in];
-    W[s][1] = -ut * u[0] + u[it];
-    W[s][2] = -(un - c) * i2c * u[0] + i2c * u[in];
-    if (FROZEN) {
-      const double *w = b[side + s];
-      Wb[s][0] = (un + c) * i2c * w[0] - i2c * w[in];
-      Wb[s][1] = -ut * w[0] + w[it];
-      Wb[s][2] = -(un - c) * i2c * w[0] + i2c * w[in];
-    }
-  }
-  double Wr[3];
-#pragma unroll
-  for (int f = 0; f < 3; ++f) {
-    double up, um;
-    if (FROZEN)
-      weno3_fixed(Wb[0][f], Wb[1][f], Wb[2][f], W[0][f], W[1][f], W[2][f], up, um);
-    else
-      weno3_both(W[0][f], W[1][f], W[2][f], up, um);
-    Wr[f] = side == 0 ? um : up;
-  }
-  out[0] = Wr[0] + Wr[2];
-  out[in] = (un - c) * Wr[0] + (un + c) * Wr[2];
-  out[it] = ut * Wr[0] + Wr[1] + ut * Wr[2];
-}
-
-__device__ __forceinline__ void llf(int dir, const double L[3], const double R[3], double g, double F[3]) {
-  const int in = dir == 0 ? 1 : 2;
-  const double iL = 1.0 / L[0], iR = 1.0 / R[0];
-  const double uL = L[1] * iL, vL = L[2] * iL, uR = R[1] * iR, vR = R[2] * iR;
-  const double pL = 0.5 * g * L[0] * L[0], pR = 0.5 * g * R[0] * R[0];
-  double FL[3], FR[3];
-  if (dir == 0) {
-    FL[0] = L[1]; FL[1] = L[1] * uL + pL; FL[2] = L[1] * vL;
-    FR[0] = R[1]; FR[1] = R[1] * uR + pR; FR[2] = R[1] * vR;
-  } else {
-    FL[0] = L[2]; FL[1] = L[2] * uL; FL[2] = L[2] * vL + pL;
-    FR[0] = R[2]; FR[1] = R[2] * uR; FR[2] = R[2] * vR + pR;
-  }
-  const double a = fmax(fabs(L[in] * iL) + sqrt(g * L[0]), fabs(R[in] * iR) + sqrt(g * R[0]));
-#pragma unroll
-  for (int m = 0; m < 3; ++m) F[m] = 0.5 * (FL[m] + FR[m]) - 0.5 * a * (R[m] - L[m]);
-}
-
-// Interface values of one line of direction dir (dir 0: row r, positions
-// a-3..a+3 along x; dir 1: column r, positions a-3..a+3 along y) at the
-// interfaces a-3/2 .. a+3/2 (f = 0..3), sides U^- (0) and U^+ (1), of the
-// (possibly perturbed) state; FROZEN: weights and eigenvectors from U itself.
-template <bool FROZEN>
-__device__ __forceinline__ void line_values2(const Geo2 &G, const double *U, int dir, int a, int r, const Pert &p,
-                                             double out[4][2][3]) {
-  double v[7][3];                 // line cells a-3 .. a+3
-  double v0[FROZEN ? 7 : 1][3];   // the same cells unperturbed (FROZEN)
-#pragma unroll
-  for (int s = 0; s < 7; ++s) {
-    if (dir == 0) cellv(G, U, a - 3 + s, r, p, v[s]);
-    else cellv(G, U, r, a - 3 + s, p, v[s]);
-  }
-  if (FROZEN) {
-    const Pert none{-1, 0, 0.0};
-#pragma unroll
-    for (int s = 0; s < 7; ++s) {
-      if (dir == 0) cellv(G, U, a - 3 + s, r, none, v0[FROZEN ? s : 0]);
-      else cellv(G, U, r, a - 3 + s, none, v0[FROZEN ? s : 0]);
-    }
-  }
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    // interface between cells k = a-2+f and k+1: v index of cell k-1 is f
-    const double(*w)[3] = &v[f];
-    const double(*w0)[3] = FROZEN ? &v0[FROZEN ? f : 0] : w;
-    if (f > 0) char_rec<FROZEN>(dir, w, w0, G.g, 0, out[f][0]);
-    if (f < 3) char_rec<FROZEN>(dir, w, w0, G.g, 1, out[f][1]);
-  }
-}
-
-// The direction-dir part of R_ij from the interface values of its three
-// lines (transverse positions r0-1, r0, r0+1): the edge fluxes at the two
-// Gauss points of the faces a-1/2, a+1/2 (flux = right minus left) and the
-// source component 1 + dir, -(1/4) sum g h b_dir (S / (dx dy)).
-__device__ __forceinline__ void dir_part2(const Geo2 &G, int dir, int c, const double (*l0)[2][3],
-                                          const double (*l1)[2][3], const double (*l2)[2][3], double flux[3],
-                                          double &S) {
-  const double(*ifv[3])[2][3] = {l0, l1, l2};
-  const int n = G.Nx * G.Ny;
-  double fl[2][3] = {{0, 0, 0}, {0, 0, 0}};
-  double hq[2][4];
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const double sg = q == 0 ? -kTq : kTq;
-    double gv[4][2][3];
-#pragma unroll
-    for (int f = 0; f < 4; ++f)
-#pragma unroll
-      for (int sd = 0; sd < 2; ++sd) {
-        if ((f == 0 && sd == 0) || (f == 3 && sd == 1)) continue;
-#pragma unroll
-        for (int m = 0; m < 3; ++m) gv[f][sd][m] = ifv[1][f][sd][m] + sg * (ifv[2][f][sd][m] - ifv[0][f][sd][m]);
-      }
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      double F[3];
-      llf(dir, gv[1 + e][0], gv[1 + e][1], G.g, F);
-#pragma unroll
-      for (int m = 0; m < 3; ++m) fl[e][m] += 0.5 * F[m];
-    }
-    hq[q][0] = gv[0][1][0];
-    hq[q][1] = gv[1][1][0];
-    hq[q][2] = gv[2][0][0];
-    hq[q][3] = gv[3][0][0];
-  }
-#pragma unroll
-  for (int m = 0; m < 3; ++m) flux[m] = fl[1][m] - fl[0][m];
-  double acc = 0.0;
-#pragma unroll
-  for (int q = 0; q < 2; ++q)
-#pragma unroll
-    for (int pp = 0; pp < 2; ++pp) {
-      const double hv = kLag2[pp][0] * hq[q][0] + kLag2[pp][1] * hq[q][1] + kLag2[pp][2] * hq[q][2] +
-                        kLag2[pp][3] * hq[q][3];
-      const int beta = dir == 0 ? q : pp, gamma = dir == 0 ? pp : q;
-      acc += G.g * hv * G.gq[(dir * 4 + 2 * beta + gamma) * n + c];
-    }
-  S = -0.25 * acc;
-}
-
-// Local residual R_ij (Eq. 20) of the (possibly perturbed) state; FROZEN:
-// the reconstructions take their weights and eigenvectors from U itself.
-template <bool FROZEN>
-__device__ void local_residual2(const Geo2 &G, const double *U, int i, int j, const Pert &p, double R[3]) {
-  const int c = j * G.Nx + i;
-  double flux[2][3], S[3] = {0.0, 0.0, 0.0};
-#pragma unroll 1
-  for (int dir = 0; dir < 2; ++dir) {
-    const int a = dir == 0 ? i : j, r0 = dir == 0 ? j : i;
-    double ifv[3][4][2][3];
-#pragma unroll 1
-    for (int t = 0; t < 3; ++t) line_values2<FROZEN>(G, U, dir, a, r0 - 1 + t, p, ifv[t]);
-    dir_part2(G, dir, c, ifv[0], ifv[1], ifv[2], flux[dir], S[1 + dir]);
-  }
-#pragma unroll
-  for (int m = 0; m < 3; ++m) R[m] = flux[0][m] / G.dx + flux[1][m] / G.dy - S[m];
-}
-
-// Interior cell whose state the (possibly ghost) position (i, j) reads, as in
-// cellv, or -1 where it reads boundary data only (inflow ghosts).
-__device__ __forceinline__ int cell_src(const Geo2 &G, int i, int j) {
-  const int Nx = G.Nx, Ny = G.Ny;
-  if (i < 0 || i >= Nx) {
-    const int xs = i < 0 ? 0 : 1;
-    const int xk = G.bck[xs * Ny + min(max(j, 0), Ny - 1)];
-    if (xk == NSWE_BC2_INFLOW) return -1;
-    i = (xk == NSWE_BC2_REFLECT) ? (i < 0 ? -1 - i : 2 * Nx - 1 - i) : (i < 0 ? 0 : Nx - 1);
-  }
-  if (j < 0 || j >= Ny) {
-    const int ys = j < 0 ? 2 : 3;
-    const int yk = G.bck[2 * Ny + (ys - 2) * Nx + i];
-    if (yk == NSWE_BC2_INFLOW) return -1;
-    j = (yk == NSWE_BC2_REFLECT) ? (j < 0 ? -1 - j : 2 * Ny - 1 - j) : (j < 0 ? 0 : Ny - 1);
-  }
-  return j * Nx + i;
-}
-
-// Whether the line (dir, a, r) of line_values2 reads interior cell cp.
-__device__ __forceinline__ bool line_reads(const Geo2 &G, int dir, int a, int r, int cp) {
-  bool hit = false;
-#pragma unroll
-  for (int s = 0; s < 7; ++s) hit |= (dir == 0 ? cell_src(G, a - 3 + s, r) : cell_src(G, r, a - 3 + s)) == cp;
-  return hit;
-}
 __device__ double block_sum2(double v, double *red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -378,126 +105,43 @@ __device__ double block_sum2(double v, double *red) {
   return red[32];
 }
 
+}  // namespace
+}  // namespace nswe
+
+#include "nswe_tile2d.cuh"
+
+namespace nswe {
+namespace {
+
 // ---------------------------------------------------------------------------- kernels
 
-// The residual of Eq. 20 by block `bid` of `nblk` (grid-stride over cells),
-// its l1 partial sum stored in partials[bid].
-__device__ __forceinline__ void residual_blocks2(const ProbDev2 *P, int level, const double *U, double *R,
-                                                 double *partials, int bid, int nblk) {
+__global__ void __launch_bounds__(kTile2Threads, 1) k2_residual(const ProbDev2 *P, int level, const double *U,
+                                                                double *R, double *partials, int TX, int TY) {
+  pdl_enter();
+  residual_tiles2(P, level, U, R, partials, TX, TY, blockIdx.x, gridDim.x);
+}
+
+// res = the sum of the partials / cells: strided over the block, then the
+// block's fixed-order sum (one thread adding 512 partials took 36 us).
+__device__ __forceinline__ void finish_block2(const double *partials, int nparts, int n, double *res) {
   __shared__ double red[33];
-  const Geo2 G = make_geo2(*P, level);
-  const int n = G.Nx * G.Ny;
-  const Pert np{-1, 0, 0.0};
-  double acc = 0.0;
-  for (int c = bid * blockDim.x + threadIdx.x; c < n; c += nblk * blockDim.x) {
-    double r[3];
-    local_residual2<false>(G, U, c % G.Nx, c / G.Nx, np, r);
-    R[c] = r[0];
-    R[n + c] = r[1];
-    R[2 * n + c] = r[2];
-    acc += fabs(r[0]) + fabs(r[1]) + fabs(r[2]);
-  }
-  const double s = block_sum2(acc, red);
-  if (threadIdx.x == 0) partials[bid] = s;
+  double v = 0.0;
+  for (int i = threadIdx.x; i < nparts; i += blockDim.x) v += partials[i];
+  const double s = block_sum2(v, red);
+  if (threadIdx.x == 0) *res = s / n;
 }
 
-__global__ void __launch_bounds__(kThreads) k2_residual(const ProbDev2 *P, int level, const double *U, double *R,
-                                                        double *partials) {
+__global__ void __launch_bounds__(kThreads) k2_finish(const double *partials, int nparts, int n, double *res) {
   pdl_enter();
-  residual_blocks2(P, level, U, R, partials, blockIdx.x, gridDim.x);
-}
-
-__global__ void k2_finish(const double *partials, int nparts, int n, double *res) {
-  pdl_enter();
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < nparts; ++i) s += partials[i];
-    *res = s / n;
-  }
-}
-
-// One item = (cell, stencil block k): three perturbed local residuals
-// (FROZEN: the frozen linearisation).
-// msplit: one item per (cell, block, component m) instead of per (cell,
-// block), for small grids where the kernel is bound by each thread's chain.
-template <typename TJ, bool FROZEN>
-__device__ __forceinline__ void jacobian_items2(const ProbDev2 *P, int level, int st, const double *U, double eps,
-                                                double alpha, const double *R, TJ *J, int msplit, int cm, int first,
-                                                int stride) {
-  const Geo2 G = make_geo2(*P, level);
-  const int n = G.Nx * G.Ny, K = st_size(st), kc = st_center(st);
-  const double ieps = 1.0 / eps;
-  const int items = n * K * (msplit ? 3 : 1);
-  for (int it = first; it < items; it += stride) {
-    const int c = it % n, kq = it / n, k = msplit ? kq % K : kq, i = c % G.Nx, j = c / G.Nx;
-    const int m0 = msplit ? kq / K : 0, m1 = msplit ? m0 + 1 : 3;
-    const size_t S = blk_stride(cm, G.Nx, G.Ny), pc = blk_pos(cm, G.Nx, G.Ny, i, j);
-    const int pi = i + st_off(st, k, 0), pj = j + st_off(st, k, 1);
-    if (pi < 0 || pi >= G.Nx || pj < 0 || pj >= G.Ny) {
-      for (int l = 0; l < 3; ++l)
-        for (int m = m0; m < m1; ++m) J[(size_t)(k * 9 + l * 3 + m) * S + pc] = TJ(0.0);
-      continue;
-    }
-    const double R0[3] = {R[c], R[n + c], R[2 * n + c]};
-    const double reg = (k == kc) ? alpha * (fabs(R0[0]) + fabs(R0[1]) + fabs(R0[2])) : 0.0;
-    // The perturbed local residuals of Eq. 12, built line by line: a line
-    // that does not read cell cp has the same interface values for the three
-    // perturbations and is reconstructed once; a direction none of whose
-    // lines read cp contributes the same flux and source to all three.
-    const int cp = pj * G.Nx + pi;
-    const Pert none{-1, 0, 0.0};
-    double fd[2][3][3], sd[2][3];  // [dir][m][component], [dir][m]
-#pragma unroll 1
-    for (int dir = 0; dir < 2; ++dir) {
-      const int a = dir == 0 ? i : j, r0 = dir == 0 ? j : i;
-      double ifv[3][4][2][3];
-      int reads = 0;
-#pragma unroll 1
-      for (int t = 0; t < 3; ++t) {
-        if (line_reads(G, dir, a, r0 - 1 + t, cp)) reads |= 1 << t;
-        else line_values2<FROZEN>(G, U, dir, a, r0 - 1 + t, none, ifv[t]);
-      }
-      if (!reads) {
-        double f[3], sv;
-        dir_part2(G, dir, c, ifv[0], ifv[1], ifv[2], f, sv);
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {  // the same for every m (m0..m1-1 are read)
-          fd[dir][m][0] = f[0];
-          fd[dir][m][1] = f[1];
-          fd[dir][m][2] = f[2];
-          sd[dir][m] = sv;
-        }
-        continue;
-      }
-#pragma unroll 1
-      for (int m = m0; m < m1; ++m) {
-        const Pert p{cp, m, eps};
-#pragma unroll 1
-        for (int t = 0; t < 3; ++t)
-          if (reads & (1 << t)) line_values2<FROZEN>(G, U, dir, a, r0 - 1 + t, p, ifv[t]);
-        dir_part2(G, dir, c, ifv[0], ifv[1], ifv[2], fd[dir][m], sd[dir][m]);
-      }
-    }
-    for (int m = m0; m < m1; ++m) {
-      const double Sm[3] = {0.0, sd[0][m], sd[1][m]};
-#pragma unroll
-      for (int l = 0; l < 3; ++l) {
-        const double Rp = fd[0][m][l] / G.dx + fd[1][m][l] / G.dy - Sm[l];
-        double v = (Rp - R0[l]) * ieps;
-        if (l == m) v += reg;
-        J[(size_t)(k * 9 + l * 3 + m) * S + pc] = TJ(v);
-      }
-    }
-  }
+  finish_block2(partials, nparts, n, res);
 }
 
 template <typename TJ, bool FROZEN>
-__global__ void __launch_bounds__(kThreads) k2_jacobian(const ProbDev2 *P, int level, int st, const double *U,
-                                                        double eps, double alpha, const double *R, TJ *J,
-                                                        int msplit, int cm) {
+__global__ void __launch_bounds__(kTile2Threads, 1) k2_jacobian(const ProbDev2 *P, int level, int st, const double *U,
+                                                                double eps, double alpha, const double *R, TJ *J,
+                                                                int cm, int TX, int TY) {
   pdl_enter();
-  jacobian_items2<TJ, FROZEN>(P, level, st, U, eps, alpha, R, J, msplit, cm, blockIdx.x * blockDim.x + threadIdx.x,
-                              gridDim.x * blockDim.x);
+  jacobian_tiles2<TJ, FROZEN>(P, level, st, U, eps, alpha, R, J, cm, TX, TY, blockIdx.x, gridDim.x);
 }
 
 template <typename T>
@@ -1039,12 +683,14 @@ __global__ void __launch_bounds__(kThreads) k2_interp(const ProbDev2 *P, int coa
   const Geo2 Gc = make_geo2(*P, coarse_level);
   const int Ncx = Gc.Nx, Ncy = Gc.Ny, Nfx = 2 * Ncx, nf = 4 * Ncx * Ncy;
   const double w[2][3] = {{0.125, 1.0, -0.125}, {-0.125, 1.0, 0.125}};
-  const Pert np{-1, 0, 0.0};
   for (int cc = blockIdx.x * blockDim.x + threadIdx.x; cc < Ncx * Ncy; cc += gridDim.x * blockDim.x) {
     const int I = cc % Ncx, Jc = cc / Ncx;
     double nb[3][3][3];
     for (int q = -1; q <= 1; ++q)
-      for (int p = -1; p <= 1; ++p) cellv(Gc, Uc, I + p, Jc + q, np, nb[q + 1][p + 1]);
+      for (int p = -1; p <= 1; ++p) {
+        int src, code;
+        cell_meta(Gc, Uc, I + p, Jc + q, nb[q + 1][p + 1], src, code);
+      }
     for (int b = 0; b < 2; ++b)
       for (int a = 0; a < 2; ++a) {
         const int cf = (2 * Jc + b) * Nfx + 2 * I + a;
@@ -1075,11 +721,11 @@ int grid2(long items) {
 // already short, the same edges made a nested solve 3 % slower, so launches
 // into a capture keep ordinary stream order.
 template <typename... KArgs, typename... Args>
-void launchk2(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Args &&...args) {
+void launchk2s(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args &&...args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1092,132 +738,91 @@ void launchk2(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Arg
   cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-}  // namespace
+template <typename... KArgs, typename... Args>
+void launchk2(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Args &&...args) {
+  launchk2s(kern, grid, block, 0, s, std::forward<Args>(args)...);
+}
 
-cudaError_t launch2_residual(const ProbDev2 *p, int level, int n, const double *U, double *R, double *res,
-                             double *partials, cudaStream_t s) {
-  const int grid = grid2(n) > 1024 ? 1024 : grid2(n);
-  launchk2(k2_residual, grid, kThreads, s, p, level, U, R, partials);
-  if (res) launchk2(k2_finish, 1, 32, s, partials, grid, n, res);
+// Launches a tile kernel with `smem` bytes of dynamic shared memory; the
+// kernel's limit is raised once per device (up to the 227 KB of an SM).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_tile2(std::atomic<unsigned> &raised, void (*kern)(KArgs...), int grid, size_t smem, cudaStream_t s,
+                         Args &&...args) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned bit = 1u << (dev & 31);
+  if (!(raised.load(std::memory_order_acquire) & bit)) {
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTile2MaxSmem))) return e;
+    raised.fetch_or(bit, std::memory_order_release);
+  }
+  launchk2s(kern, grid, kTile2Threads, smem, s, std::forward<Args>(args)...);
   return cudaGetLastError();
 }
 
-// The same Jacobian with one cell per thread (large grids): the six
-// unperturbed reconstruction lines of the cell and its two direction parts
-// are built once and serve all blocks and components; each perturbation
-// rebuilds only the lines that read the perturbed cell (for J9, 60 line
-// reconstructions per cell against 90 when each (cell, block) item builds
-// its own). The same expressions on the same inputs as k2_jacobian, so the
-// same bits. The lines live in local memory (about 1.9 KB a thread), which
-// costs less than the saved FP64 work from about 32,768 cells on; below
-// that the per-item kernel's nine- or 27-fold parallelism wins
-// (kJac2CellMinDefault).
-constexpr int kJacCellThreads = 128;
-template <typename TJ, bool FROZEN>
-__device__ __forceinline__ void jacobian_cells2(const ProbDev2 *P, int level, int st, const double *U, double eps,
-                                                double alpha, const double *R, TJ *J, int cm, int first,
-                                                int stride) {
-  const Geo2 G = make_geo2(*P, level);
-  const int n = G.Nx * G.Ny, K = st_size(st), kc = st_center(st);
-  const double ieps = 1.0 / eps;
-  const Pert none{-1, 0, 0.0};
-  for (int c = first; c < n; c += stride) {
-    const int i = c % G.Nx, j = c / G.Nx;
-    const size_t S = blk_stride(cm, G.Nx, G.Ny), pc = blk_pos(cm, G.Nx, G.Ny, i, j);
-    const double R0[3] = {R[c], R[n + c], R[2 * n + c]};
-    double base[2][3][4][2][3], fb[2][3], sb[2];
-#pragma unroll 1
-    for (int dir = 0; dir < 2; ++dir) {
-      const int a = dir == 0 ? i : j, r0 = dir == 0 ? j : i;
-#pragma unroll 1
-      for (int t = 0; t < 3; ++t) line_values2<FROZEN>(G, U, dir, a, r0 - 1 + t, none, base[dir][t]);
-      dir_part2(G, dir, c, base[dir][0], base[dir][1], base[dir][2], fb[dir], sb[dir]);
-    }
-#pragma unroll 1
-    for (int k = 0; k < K; ++k) {
-      const int pi = i + st_off(st, k, 0), pj = j + st_off(st, k, 1);
-      if (pi < 0 || pi >= G.Nx || pj < 0 || pj >= G.Ny) {
-        for (int e = 0; e < 9; ++e) J[(size_t)(k * 9 + e) * S + pc] = TJ(0.0);
-        continue;
-      }
-      const int cp = pj * G.Nx + pi;
-      const double reg = (k == kc) ? alpha * (fabs(R0[0]) + fabs(R0[1]) + fabs(R0[2])) : 0.0;
-      int reads[2];
-#pragma unroll 1
-      for (int dir = 0; dir < 2; ++dir) {
-        const int a = dir == 0 ? i : j, r0 = dir == 0 ? j : i;
-        reads[dir] = 0;
-        for (int t = 0; t < 3; ++t)
-          if (line_reads(G, dir, a, r0 - 1 + t, cp)) reads[dir] |= 1 << t;
-      }
-#pragma unroll 1
-      for (int m = 0; m < 3; ++m) {
-        const Pert p{cp, m, eps};
-        double fd[2][3], sdv[2];
-#pragma unroll 1
-        for (int dir = 0; dir < 2; ++dir) {
-          if (!reads[dir]) {
-            fd[dir][0] = fb[dir][0];
-            fd[dir][1] = fb[dir][1];
-            fd[dir][2] = fb[dir][2];
-            sdv[dir] = sb[dir];
-            continue;
-          }
-          const int a = dir == 0 ? i : j, r0 = dir == 0 ? j : i;
-          double tmp[3][4][2][3];
-          const double(*l[3])[2][3];
-#pragma unroll 1
-          for (int t = 0; t < 3; ++t) {
-            if (reads[dir] & (1 << t)) {
-              line_values2<FROZEN>(G, U, dir, a, r0 - 1 + t, p, tmp[t]);
-              l[t] = tmp[t];
-            } else {
-              l[t] = base[dir][t];
-            }
-          }
-          dir_part2(G, dir, c, l[0], l[1], l[2], fd[dir], sdv[dir]);
-        }
-        const double Sm[3] = {0.0, sdv[0], sdv[1]};
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          const double Rp = fd[0][q] / G.dx + fd[1][q] / G.dy - Sm[q];
-          double v = (Rp - R0[q]) * ieps;
-          if (q == m) v += reg;
-          J[(size_t)(k * 9 + q * 3 + m) * S + pc] = TJ(v);
-        }
+}  // namespace
+
+// The tile of a residual (NF = 1) or Jacobian (NF flux variants) of an Nx x Ny
+// level: the least estimated time over tiles that fit shared memory. A block
+// holds an SM; its time is the FP64 warp instructions of its largest sub-
+// partition, phase by phase (the halo's included), and the tiles run in
+// rounds of one per SM. So large grids take the largest tile that fills the
+// SMs evenly, small grids tiles of a few cells. Results do not depend on the
+// tile, the order of the partial sums of res does.
+static Tile2Shape tile2_choose(int Nx, int Ny, int NF, int K) {
+  const bool jac = NF > 1;
+  const int NV = jac ? 10 : 1;
+  Tile2Shape best{0, 0, 0, 0};
+  long best_cost = 0;
+  size_t off[8];
+  auto rounds4 = [](long items) { return (items + 127) / 128; };  // warps per sub-partition
+  static const int side[] = {3, 4, 6, 8, 10, 12, 16, 20, 24, 28, 32};
+  for (int cx : side)
+    for (int cy : side) {
+      // the same number of tiles, evenly sized
+      const int nx = (Nx + cx - 1) / cx, ny = (Ny + cy - 1) / cy, TX = (Nx + nx - 1) / nx, TY = (Ny + ny - 1) / ny;
+      const size_t smem = sizeof(double) * tile2_doubles(TX, TY, NV, NF, jac, off);
+      if (smem > (size_t)kTile2MaxSmem) continue;
+      const long nI = (long)(TX + 2) * (TY + 2), nP = (long)(TX + 3) * (TY + 2) + (long)(TY + 3) * (TX + 2);
+      const long nF = (long)(TX + 1) * TY + (long)(TY + 1) * TX, cells = (long)TX * TY;
+      long cost = 40 + 190 * rounds4(nP) + 130 * rounds4(NF * nF) + (jac ? 85 * rounds4(3L * K * cells) : 100 * rounds4(cells));
+      if (jac) cost += 60 * rounds4(36 * nI);
+      cost *= ((long)nx * ny + kSmCount - 1) / kSmCount;
+      if (!best.TX || cost < best_cost) {
+        best_cost = cost;
+        best = Tile2Shape{TX, TY, nx * ny, smem};
       }
     }
-  }
+  return best;
 }
 
-template <typename TJ, bool FROZEN>
-__global__ void __launch_bounds__(kJacCellThreads) k2_jacobian_cell(const ProbDev2 *P, int level, int st,
-                                                                  const double *U, double eps, double alpha,
-                                                                  const double *R, TJ *J, int cm) {
-  pdl_enter();
-  jacobian_cells2<TJ, FROZEN>(P, level, st, U, eps, alpha, R, J, cm, blockIdx.x * blockDim.x + threadIdx.x,
-                              gridDim.x * blockDim.x);
+Tile2Shape tile2_residual_shape(int Nx, int Ny) {
+  Tile2Shape t = tile2_choose(Nx, Ny, 1, 0);
+  if (t.blocks > 1024) t.blocks = 1024;  // partial sums; the blocks stride over the tiles
+  return t;
+}
+Tile2Shape tile2_jacobian_shape(int Nx, int Ny, int st) {
+  return st == ST_J21 ? tile2_choose(Nx, Ny, 37, 21) : tile2_choose(Nx, Ny, 25, 9);
+}
+
+cudaError_t launch2_residual(const ProbDev2 *p, int level, int Nx, int Ny, const double *U, double *R, double *res,
+                             double *partials, cudaStream_t s) {
+  static std::atomic<unsigned> raised{0};
+  const Tile2Shape t = tile2_residual_shape(Nx, Ny);
+  const cudaError_t e = launch_tile2(raised, k2_residual, t.blocks, t.smem, s, p, level, U, R, partials, t.TX, t.TY);
+  if (e != cudaSuccess) return e;
+  if (res) launchk2(k2_finish, 1, kThreads, s, partials, t.blocks, Nx * Ny, res);
+  return cudaGetLastError();
 }
 
 template <typename TJ>
-cudaError_t launch2_jacobian(const ProbDev2 *p, int level, int n, int st, const double *U, double eps, double alpha,
-                             const double *R, TJ *J, bool frozen, int cm, int cell_min, cudaStream_t s) {
-  if (cell_min >= 0 && n >= cell_min) {
-    const int grid = (int)((n + kJacCellThreads - 1) / kJacCellThreads);
-    if (frozen)
-      launchk2(k2_jacobian_cell<TJ, true>, grid, kJacCellThreads, s, p, level, st, U, eps, alpha, R, J, cm);
-    else
-      launchk2(k2_jacobian_cell<TJ, false>, grid, kJacCellThreads, s, p, level, st, U, eps, alpha, R, J, cm);
-    return cudaGetLastError();
-  }
-  const long items = (long)n * (st == ST_J21 ? 21 : 9);
-  const int msplit = 3 * items <= kJacSplitItems ? 1 : 0;
-  const int grid = grid2(items * (msplit ? 3 : 1));
-  if (frozen)
-    launchk2(k2_jacobian<TJ, true>, grid, kThreads, s, p, level, st, U, eps, alpha, R, J, msplit, cm);
-  else
-    launchk2(k2_jacobian<TJ, false>, grid, kThreads, s, p, level, st, U, eps, alpha, R, J, msplit, cm);
-  return cudaGetLastError();
+cudaError_t launch2_jacobian(const ProbDev2 *p, int level, int Nx, int Ny, int st, const double *U, double eps,
+                             double alpha, const double *R, TJ *J, bool frozen, int cm, cudaStream_t s) {
+  static std::atomic<unsigned> raised[2];
+  const Tile2Shape t = tile2_jacobian_shape(Nx, Ny, st);
+  auto kern = frozen ? k2_jacobian<TJ, true> : k2_jacobian<TJ, false>;
+  return launch_tile2(raised[frozen ? 1 : 0], kern, t.blocks, t.smem, s, p, level, st, U, eps, alpha, R, J, cm, t.TX,
+                      t.TY);
 }
 
 template <typename T>
@@ -1304,8 +909,8 @@ cudaError_t launch2_to_f32(long count, const double *src, float *dst, cudaStream
 }
 
 #define NSWE_2D_INSTANTIATE(T)                                                                                    \
-  template cudaError_t launch2_jacobian<T>(const ProbDev2 *, int, int, int, const double *, double, double,      \
-                                           const double *, T *, bool, int, int, cudaStream_t);                   \
+  template cudaError_t launch2_jacobian<T>(const ProbDev2 *, int, int, int, int, const double *, double, double, \
+                                           const double *, T *, bool, int, cudaStream_t);                        \
   template cudaError_t launch2_coarse_op<T>(int, int, int, const T *, T *, int, cudaStream_t);                   \
   template cudaError_t launch2_dinv<T>(int, int, int, const T *, T *, int, cudaStream_t);                        \
   template cudaError_t launch2_sor<T>(int, int, int, const T *, const T *, const T *, T *, double, int, int, int, \
@@ -1347,42 +952,31 @@ __device__ __forceinline__ const BTask2<T> *btask2(const BTask2<T> *tasks, int n
   return (done && done[t->prob]) ? nullptr : t;
 }
 
-__global__ void __launch_bounds__(kThreads) kb2_residual(const BTask2<double> *tasks, int ntask, const int *done) {
+__global__ void __launch_bounds__(kTile2Threads, 1) kb2_residual(const BTask2<double> *tasks, int ntask,
+                                                                 const int *done) {
   pdl_enter();
   int lb;
   const BTask2<double> *t = btask2(tasks, ntask, done, lb);
-  if (t) residual_blocks2(t->P, t->level, t->U, t->R64, t->partials, lb, t->nb);
+  if (t) residual_tiles2(t->P, t->level, t->U, t->R64, t->partials, t->TX, t->TY, lb, t->nb);
 }
 
-// One task per block: res[prob] = (sum of its partials, in order) / cells (as k2_finish).
-__global__ void kb2_finish(const BTask2<double> *tasks, int ntask, const int *done, double *res) {
+// One task per block: res[prob] = the sum of its partials / cells (as k2_finish).
+__global__ void __launch_bounds__(kThreads) kb2_finish(const BTask2<double> *tasks, int ntask, const int *done,
+                                                       double *res) {
   pdl_enter();
   const BTask2<double> &t = tasks[blockIdx.x];
-  if ((done && done[t.prob]) || threadIdx.x != 0) return;
-  double s = 0.0;
-  for (int i = 0; i < t.nb; ++i) s += t.partials[i];
-  res[t.prob] = s / (t.Nx * t.Ny);
+  if (done && done[t.prob]) return;
+  finish_block2(t.partials, t.nb, t.Nx * t.Ny, res + t.prob);
 }
 
 template <typename TJ, bool FROZEN>
-__global__ void __launch_bounds__(kThreads) kb2_jacobian(const BTask2<TJ> *tasks, int ntask, const int *done) {
+__global__ void __launch_bounds__(kTile2Threads, 1) kb2_jacobian(const BTask2<TJ> *tasks, int ntask, const int *done) {
   pdl_enter();
   int lb;
   const BTask2<TJ> *t = btask2(tasks, ntask, done, lb);
   if (t)
-    jacobian_items2<TJ, FROZEN>(t->P, t->level, t->st, t->U, t->eps, t->alpha, t->R64, t->J, t->msplit, t->cm,
-                                lb * blockDim.x + threadIdx.x, t->nb * blockDim.x);
-}
-
-template <typename TJ, bool FROZEN>
-__global__ void __launch_bounds__(kJacCellThreads) kb2_jacobian_cell(const BTask2<TJ> *tasks, int ntask,
-                                                                   const int *done) {
-  pdl_enter();
-  int lb;
-  const BTask2<TJ> *t = btask2(tasks, ntask, done, lb);
-  if (t)
-    jacobian_cells2<TJ, FROZEN>(t->P, t->level, t->st, t->U, t->eps, t->alpha, t->R64, t->J, t->cm,
-                                lb * blockDim.x + threadIdx.x, t->nb * blockDim.x);
+    jacobian_tiles2<TJ, FROZEN>(t->P, t->level, t->st, t->U, t->eps, t->alpha, t->R64, t->J, t->cm, t->TX, t->TY, lb,
+                                t->nb);
 }
 
 __global__ void __launch_bounds__(kThreads) kb2_to_f32(const BTask2<float> *tasks, int ntask, const int *done) {
@@ -1508,26 +1102,22 @@ __global__ void __launch_bounds__(kThreads) kb2_update(const BTask2<T> *tasks, i
 }  // namespace
 
 int b2_grid(long items) { return grid2(items); }
-int b2_jacobian_cell_threads() { return kJacCellThreads; }
 
 cudaError_t launchb2_residual(const Batch2Launch<double> &b, const int *done, double *res, cudaStream_t s) {
   if (b.ntask == 0) return cudaSuccess;
-  launchk2(kb2_residual, b.blocks, kThreads, s, b.tasks, b.ntask, done);
-  launchk2(kb2_finish, b.ntask, 32, s, b.tasks, b.ntask, done, res);
+  static std::atomic<unsigned> raised{0};
+  const cudaError_t e = launch_tile2(raised, kb2_residual, b.blocks, b.smem, s, b.tasks, b.ntask, done);
+  if (e != cudaSuccess) return e;
+  launchk2(kb2_finish, b.ntask, kThreads, s, b.tasks, b.ntask, done, res);
   return cudaGetLastError();
 }
 
 template <typename TJ>
-cudaError_t launchb2_jacobian(const Batch2Launch<TJ> &b, const int *done, int kind, bool frozen, cudaStream_t s) {
+cudaError_t launchb2_jacobian(const Batch2Launch<TJ> &b, const int *done, bool frozen, cudaStream_t s) {
   if (b.ntask == 0) return cudaSuccess;
-  if (kind == kB2JacCells) {
-    if (frozen) launchk2(kb2_jacobian_cell<TJ, true>, b.blocks, kJacCellThreads, s, b.tasks, b.ntask, done);
-    else launchk2(kb2_jacobian_cell<TJ, false>, b.blocks, kJacCellThreads, s, b.tasks, b.ntask, done);
-  } else {
-    if (frozen) launchk2(kb2_jacobian<TJ, true>, b.blocks, kThreads, s, b.tasks, b.ntask, done);
-    else launchk2(kb2_jacobian<TJ, false>, b.blocks, kThreads, s, b.tasks, b.ntask, done);
-  }
-  return cudaGetLastError();
+  static std::atomic<unsigned> raised[2];
+  auto kern = frozen ? kb2_jacobian<TJ, true> : kb2_jacobian<TJ, false>;
+  return launch_tile2(raised[frozen ? 1 : 0], kern, b.blocks, b.smem, s, b.tasks, b.ntask, done);
 }
 
 cudaError_t launchb2_to_f32(const Batch2Launch<float> &b, const int *done, cudaStream_t s) {
@@ -1617,7 +1207,7 @@ cudaError_t launchb2_update(const Batch2Launch<T> &b, const int *done, int *flag
 }
 
 #define NSWE_B2_INSTANTIATE(T)                                                                                     \
-  template cudaError_t launchb2_jacobian<T>(const Batch2Launch<T> &, const int *, int, bool, cudaStream_t);       \
+  template cudaError_t launchb2_jacobian<T>(const Batch2Launch<T> &, const int *, bool, cudaStream_t);            \
   template cudaError_t launchb2_zero_du<T>(const Batch2Launch<T> &, const int *, cudaStream_t);                   \
   template cudaError_t launchb2_coarse_op<T>(const Batch2Launch<T> &, const int *, cudaStream_t);                 \
   template cudaError_t launchb2_dinv<T>(const Batch2Launch<T> &, const int *, cudaStream_t);                      \

@@ -470,7 +470,7 @@ def nswe_ctx_get_tuned_2d(ctx, Nx, Ny, precision):
 
 
 def nswe_ctx_set_jacobian_cells_2d(ctx, min_cells):
-    """2D levels of at least min_cells cells take the per-cell Jacobian kernel (<0: never)."""
+    """Accepted and without effect: one Jacobian kernel serves every level size (see include/nswe.h)."""
     _check("nswe_ctx_set_jacobian_cells_2d", lib().nswe_ctx_set_jacobian_cells_2d(ctx.h, int(min_cells)))
 
 
