@@ -218,9 +218,11 @@ nswe_status nswe_set_launch_overlap_2d(int enable);
 
 /* Tail threshold of the 2D V-cycles (the paper has no counterpart; results
  * are the same bits whatever its value): from the first level of at most
- * max_cells cells down to the coarsest and back, a V-cycle runs as one
- * thread block per problem instead of one launch per colour pass. precision:
- * NSWE_PREC_FP64 (default 256 cells) or NSWE_PREC_MIXED (default 4096). */
+ * max_cells cells that fits down to the coarsest and back, a V-cycle runs as
+ * one launch, a thread-block cluster per problem whose CTAs keep the levels in
+ * shared memory, instead of one launch per colour pass. precision:
+ * NSWE_PREC_FP64 (default 4096 cells) or NSWE_PREC_MIXED (default: every
+ * level that fits). */
 nswe_status nswe_ctx_set_tail_2d(nswe_ctx ctx, int precision, int max_cells);
 
 /* Autotuner of the 2D V-cycle (the paper has no counterpart): forms the

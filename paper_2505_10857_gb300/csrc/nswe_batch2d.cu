@@ -148,7 +148,7 @@ void for_each_pass(int st, int steps, int Kc, F &&pass) {
 // tails[i]: the tail threshold (cells) of problem i's V-cycles.
 template <typename T>
 nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const double *const *U0s, double *const *Us,
-                       const nswe_params *prms, const int *tails, bool each, nswe_info *infos) {
+                       const nswe_params *prms, const long *tails, bool each, nswe_info *infos) {
   constexpr bool kMixed = std::is_same<T, float>::value;
   const nswe_params &P0 = prms[0];
   const int st0 = (P0.jacobian & ~NSWE_JAC_FROZEN) == NSWE_JAC_FULL ? ST_J21 : ST_J9;
@@ -215,10 +215,19 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
     sd.g_zero_du = sd.pool.begin();
     sd.g_tail = sd.pool.begin();
     int depths = 0;  // grid-wide V-cycle depths of the stage
+    int direct_cells = 0, lu_cells = 0;
     struct VC {
       int i, l, ls, L, cm;
     };
     std::vector<VC> vcs;
+    // CTAs per problem of the cluster launch: as many as let the stage's
+    // V-cycles run at once on nine clusters' worth of SMs
+    int nvc = 0;
+    for (size_t a = 0; a < act.size(); ++a) nvc += lev[a] < probs[act[a]]->levels - 1 ? 1 : 0;
+    int tail_ctas = kTail2MaxCtas;
+    while (tail_ctas > 2 && tail_ctas * nvc > 144) tail_ctas /= 2;
+    int used_ctas = 1, tail_threads = 0;
+    size_t tail_smem = 0;
     for (size_t a = 0; a < act.size(); ++a) {
       const int i = act[a], l = lev[a];
       nswe_prob_s *p = probs[i];
@@ -227,7 +236,10 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
       const Level2Dev &Lv = p->host2.lev[l];
       const int n = Lv.Nx * Lv.Ny;
       const int minc = ctx->cm2d_min_cells;
-      const int cm = (l < L && st0 == ST_J9 && minc >= 0 && n >= minc && n > tails[i]) ? 1 : 0;
+      const int cm = (l < L && st0 == ST_J9 && minc >= 0 && n >= minc &&
+                      tail2_first<T>(p, l, st0, tails[i], tail_ctas) > l)
+                         ? 1
+                         : 0;
       T *const J = reinterpret_cast<T *>(Lv.J);
       T *const dU = reinterpret_cast<T *>(Lv.dU);
       T *const Rs = kMixed ? J + (size_t)K * 9 * blk_stride(cm, Lv.Nx, Lv.Ny) : reinterpret_cast<T *>(Lv.R);
@@ -253,7 +265,6 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
       t.alpha = prm.alpha;
       t.tau = prm.tau;
       t.A = reinterpret_cast<T *>(p->dense);
-      t.x = reinterpret_cast<T *>(p->xbuf);
       t.piv = p->piv;
       {  // residual (the tiles and block count of launch2_residual)
         BTask2<double> r;
@@ -276,15 +287,28 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
         sd.pool.add(sd.g_direct_zero, t, b2_grid(N3 * N3));
         sd.pool.add(sd.g_direct_scatter, t, b2_grid((long)n * K));
         sd.pool.add(sd.g_direct, t, 1);
+        direct_cells = std::max(direct_cells, n);
         continue;
       }
-      // V-cycles: the first level of at most tails[i] cells starts the tail
-      int ls = L;
-      for (int m = l; m < L; ++m)
-        if (p->host2.lev[m].Nx * p->host2.lev[m].Ny <= tails[i]) {
-          ls = m;
-          break;
-        }
+      // V-cycles: the tail's levels, on a cluster per problem
+      Tail2<T> tl;
+      std::memset(&tl, 0, sizeof(tl));
+      tl.L = L;
+      for (int m = l, stl = st0; m <= L; ++m, stl = st_coarse_host(stl)) {
+        const Level2Dev &Lm = p->host2.lev[m];
+        tl.Nx[m] = Lm.Nx;
+        tl.Ny[m] = Lm.Ny;
+        tl.st[m] = stl;
+        tl.J[m] = m == l ? J : reinterpret_cast<T *>(Lm.J);
+        tl.R[m] = m == l ? Rs : reinterpret_cast<T *>(Lm.R);
+        tl.Dinv[m] = reinterpret_cast<T *>(Lm.Dinv);
+        tl.dU[m] = reinterpret_cast<T *>(Lm.dU);
+      }
+      tl.A = reinterpret_cast<const T *>(p->dense);
+      tl.piv = p->piv;
+      const int ls = plan_tail2<T>(tl, l, cm, tails[i], tail_ctas);
+      used_ctas = std::max(used_ctas, tl.ctas);
+      sd.tails.push_back(tl);
       vcs.push_back({i, l, ls, L, cm});
       depths = std::max(depths, ls - l);
     }
@@ -333,16 +357,16 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
           t.dUc = reinterpret_cast<T *>(Lc.dU);
         }
         t.A = reinterpret_cast<T *>(p->dense);
-        t.x = reinterpret_cast<T *>(p->xbuf);
         t.piv = p->piv;
         if (m < v.L) {
-          sd.pool.add(sd.g_cop[d], t, b2_grid((long)(Lm.Nx / 2) * (Lm.Ny / 2)));
+          sd.pool.add(sd.g_cop[d], t, b2_grid(9L * (Lm.Nx / 2) * (Lm.Ny / 2)));
           sd.pool.add(sd.g_dinv[d], t, b2_grid(n));
         } else {  // the coarsest: dense factors
           const long N3 = 3L * n;
           sd.pool.add(sd.g_vc_zero, t, b2_grid(N3 * N3));
           sd.pool.add(sd.g_vc_scatter, t, b2_grid((long)n * st_size_host(st)));
           sd.pool.add(sd.g_vc_lu, t, 1);
+          lu_cells = std::max(lu_cells, n);
         }
         if (d == 0) sd.pool.add(sd.g_zero_du, t, b2_grid(3L * n));
         if (m < v.ls) {
@@ -353,39 +377,17 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
         }
         st = st_coarse_host(st);
       }
-      // the tail of this problem's V-cycle (one block)
-      Tail2<T> tl;
-      std::memset(&tl, 0, sizeof(tl));
-      tl.ls = v.ls;
-      tl.L = v.L;
-      int stl = st0;
-      for (int m = v.l; m <= v.L; ++m) {
-        if (m >= v.ls) {
-          const Level2Dev &Lm = p->host2.lev[m];
-          tl.Nx[m] = Lm.Nx;
-          tl.Ny[m] = Lm.Ny;
-          tl.st[m] = stl;
-          if (m == v.l) {
-            const Level2Dev &Lv = p->host2.lev[v.l];
-            tl.J[m] = reinterpret_cast<T *>(Lv.J);
-            tl.R[m] = kMixed ? tl.J[m] + (size_t)K * 9 * blk_stride(v.cm, Lv.Nx, Lv.Ny) : reinterpret_cast<T *>(Lv.R);
-          } else {
-            tl.J[m] = reinterpret_cast<T *>(Lm.J);
-            tl.R[m] = reinterpret_cast<T *>(Lm.R);
-          }
-          tl.Dinv[m] = reinterpret_cast<T *>(Lm.Dinv);
-          tl.dU[m] = reinterpret_cast<T *>(Lm.dU);
-        }
-        stl = st_coarse_host(stl);
-      }
-      tl.A = reinterpret_cast<const T *>(p->dense);
-      tl.piv = p->piv;
-      tl.x = reinterpret_cast<T *>(p->xbuf);
       BTask2<T> tt;
       std::memset(&tt, 0, sizeof(tt));
       tt.prob = v.i;
       sd.pool.add(sd.g_tail, tt, 1);
-      sd.tails.push_back(tl);
+    }
+    // one cluster size for the launch: every problem's bands planned for it
+    for (size_t v = 0; v < vcs.size(); ++v) {
+      plan_tail2<T>(sd.tails[v], vcs[v].l, vcs[v].cm, tails[vcs[v].i], used_ctas);
+      sd.tails[v].ctas = used_ctas;
+      tail_threads = std::max(tail_threads, sd.tails[v].threads);
+      tail_smem = std::max(tail_smem, sd.tails[v].smem);
     }
     // ---- upload the task tables
     sd.pool.flatten();
@@ -437,8 +439,8 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
       // Newton on the coarsest grid
       const auto dz = sd.launch(sd.g_direct);
       if ((e = launchb2_dense_factor<T>(sd.launch(sd.g_direct_zero), sd.launch(sd.g_direct_scatter), dz.tasks,
-                                        dz.ntask, done, flags, q)) ||
-          (e = launchb2_dense_solve<T>(dz.tasks, dz.ntask, done, q)))
+                                        dz.ntask, direct_cells, done, flags, q)) ||
+          (e = launchb2_dense_solve<T>(dz.tasks, dz.ntask, direct_cells, done, q)))
         return e;
       // V-cycles: Galerkin operators and inverse diagonal blocks, coarsest factors, then nu3 cycles
       for (int d = 0; d < 16; ++d)
@@ -446,12 +448,11 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
       for (int d = 0; d < 16; ++d)
         if ((e = launchb2_dinv<T>(sd.launch(sd.g_dinv[d]), done, q))) return e;
       const auto lu = sd.launch(sd.g_vc_lu);
-      if ((e = launchb2_dense_factor<T>(sd.launch(sd.g_vc_zero), sd.launch(sd.g_vc_scatter), lu.tasks, lu.ntask,
-                                        done, flags, q)))
-        return e;
       if ((e = launchb2_zero_du<T>(sd.launch(sd.g_zero_du), done, q))) return e;
       const auto tail = sd.launch(sd.g_tail);
-      for (int v = 0; v < P0.nu3; ++v) {
+      // all levels of all problems on their clusters: the nu3 V-cycles are one launch
+      const int launches = depths == 0 ? 1 : P0.nu3, cycles = depths == 0 ? P0.nu3 : 1;
+      for (int v = 0; v < launches; ++v) {
         for (int d = 0; d < depths; ++d) {
           const auto b = sd.launch(sd.g_sor[d]);
           for_each_pass(sd.sor_st[d], P0.nu1, Kc, [&](int mode, int kc, int col, int reps) {
@@ -459,7 +460,13 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
           });
           if (e || (e = launchb2_restrict<T>(sd.launch(sd.g_restrict[d]), done, q))) return e;
         }
-        if ((e = launchb2_vcycle_tail<T>(sd.dev_tails, tail.tasks, tail.ntask, done, P0.nu1, P0.nu2, omega, Kc, q)))
+        // the coarsest factors, overlapped by the launch that uses them
+        if (v == 0 &&
+            (e = launchb2_dense_factor<T>(sd.launch(sd.g_vc_zero), sd.launch(sd.g_vc_scatter), lu.tasks, lu.ntask,
+                                          lu_cells, done, flags, q)))
+          return e;
+        if ((e = launchb2_vcycle_tail<T>(sd.dev_tails, tail.tasks, tail.ntask, used_ctas, tail_threads, tail_smem,
+                                         done, P0.nu1, P0.nu2, omega, Kc, cycles, v == 0, q)))
           return e;
         for (int d = depths - 1; d >= 0; --d) {
           if ((e = launchb2_prolong<T>(sd.launch(sd.g_prolong[d]), done, q))) return e;
@@ -567,7 +574,7 @@ nswe_status solve2d_lockstep(nswe_ctx ctx, int count, const nswe_prob *probs, co
   DevGuard dg(ctx->device);
   // each problem's schedule and tail threshold (colours2d = AUTO resolved per size)
   std::vector<nswe_params> res(count);
-  std::vector<int> tail(count);
+  std::vector<long> tail(count);
   for (int i = 0; i < count; ++i) resolve2d(probs[i], prms[each ? i : 0], res[i], tail[i]);
   std::vector<int> group(count, -1);
   int ngroups = 0;
@@ -586,7 +593,8 @@ nswe_status solve2d_lockstep(nswe_ctx ctx, int count, const nswe_prob *probs, co
     std::vector<const double *> u0g;
     std::vector<double *> ug;
     std::vector<nswe_params> prg;
-    std::vector<int> idx, tg;
+    std::vector<int> idx;
+    std::vector<long> tg;
     for (int i = 0; i < count; ++i)
       if (group[i] == g) {
         pg.push_back(probs[i]);

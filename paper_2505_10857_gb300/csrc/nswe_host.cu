@@ -269,40 +269,13 @@ MG2<T> mg2_bind(const nswe_prob_s *p, int l0, int st0, const T *J, const T *R, T
   return m;
 }
 
+// The hierarchy m as the cluster launch takes it, the tail's first level chosen.
 template <typename T>
-cudaError_t mg2_setup(nswe_prob_s *p, const MG2<T> &m, cudaStream_t s) {
-  cudaError_t e;
-  for (int l = m.l0 + 1; l <= m.L; ++l)
-    if ((e = launch2_coarse_op<T>(m.lv[l - 1].Nx, m.lv[l - 1].Ny, m.st[l - 1], m.lv[l - 1].J, m.lv[l].J,
-                                  m.lv[l - 1].cm, s)))
-      return e;
-  for (int l = m.l0; l < m.L; ++l)
-    if ((e = launch2_dinv<T>(m.lv[l].Nx, m.lv[l].Ny, m.st[l], m.lv[l].J, m.lv[l].Dinv, m.lv[l].cm, s))) return e;
-  return launch2_dense_factor<T>(m.lv[m.L].Nx, m.lv[m.L].Ny, m.st[m.L], m.lv[m.L].J,
-                                 reinterpret_cast<T *>(p->dense), p->piv, p->flag, s);
-}
-
-// Algorithm 2 from level l0: grid-wide kernels on the large levels; from the
-// first level of at most `tail` cells down to the coarsest and back up, one
-// block-persistent launch (the same bits either way).
-template <typename T>
-cudaError_t mg2_vcycle(nswe_prob_s *p, const MG2<T> &m, const nswe_params &prm, cudaStream_t s, int tail) {
-  cudaError_t e;
-  int ls = m.L;  // first level handled by the tail launch
-  for (int l = m.l0; l < m.L; ++l) {
-    if (m.lv[l].Nx * m.lv[l].Ny <= tail) {
-      ls = l;
-      break;
-    }
-    if ((e = smooth2<T>(m.lv[l], m.st[l], prm.nu1, prm.omega, prm.colours2d, s))) return e;
-    if ((e = launch2_restrict<T>(m.lv[l].Nx, m.lv[l].Ny, m.st[l], m.lv[l].J, m.lv[l].R, m.lv[l].dU, m.lv[l + 1].R,
-                                 m.lv[l + 1].dU, m.lv[l].cm, s)))
-      return e;
-  }
+Tail2<T> tail2_of(const nswe_prob_s *p, const MG2<T> &m, long tail) {
   Tail2<T> t;
-  t.ls = ls;
+  std::memset(&t, 0, sizeof(t));
   t.L = m.L;
-  for (int l = ls; l <= m.L; ++l) {
+  for (int l = m.l0; l <= m.L; ++l) {
     t.Nx[l] = m.lv[l].Nx;
     t.Ny[l] = m.lv[l].Ny;
     t.st[l] = m.st[l];
@@ -313,13 +286,52 @@ cudaError_t mg2_vcycle(nswe_prob_s *p, const MG2<T> &m, const nswe_params &prm, 
   }
   t.A = reinterpret_cast<const T *>(p->dense);
   t.piv = p->piv;
-  t.x = reinterpret_cast<T *>(p->xbuf);
-  if ((e = launch2_vcycle_tail<T>(t, prm.nu1, prm.nu2, prm.omega, prm.colours2d, s))) return e;
-  for (int l = ls - 1; l >= m.l0; --l) {
-    if ((e = launch2_prolong<T>(m.lv[l].Nx, m.lv[l].Ny, m.lv[l].dU, m.lv[l + 1].dU, s))) return e;
-    if ((e = smooth2<T>(m.lv[l], m.st[l], prm.nu2, prm.omega, prm.colours2d, s))) return e;
+  plan_tail2<T>(t, m.l0, m.lv[m.l0].cm, tail, kTail2MaxCtas);
+  return t;
+}
+
+// Galerkin operators and inverse diagonal blocks of every level; the coarsest
+// factorisation follows in the first V-cycle (mg2_vcycle).
+template <typename T>
+cudaError_t mg2_setup(nswe_prob_s *p, const MG2<T> &m, cudaStream_t s) {
+  cudaError_t e;
+  for (int l = m.l0 + 1; l <= m.L; ++l)
+    if ((e = launch2_coarse_op<T>(m.lv[l - 1].Nx, m.lv[l - 1].Ny, m.st[l - 1], m.lv[l - 1].J, m.lv[l].J,
+                                  m.lv[l - 1].cm, s)))
+      return e;
+  return launch2_dinv_levels<T>(tail2_of<T>(p, m, 0), m.l0, m.lv[m.l0].cm, s);
+}
+
+// Algorithm 2 from level l0, `cycles` times: grid-wide kernels on the large
+// levels; the levels from the tail's first one down to the coarsest and back
+// up as one cluster launch (the same bits either way). factor: the coarsest
+// system is factored first, right before the launch that uses it, which
+// overlaps it.
+template <typename T>
+cudaError_t mg2_vcycle(nswe_prob_s *p, const MG2<T> &m, const nswe_params &prm, cudaStream_t s, long tail, int cycles,
+                       bool factor) {
+  cudaError_t e = cudaSuccess;
+  const Tail2<T> t = tail2_of<T>(p, m, tail);
+  const Lev2<T> &C = m.lv[m.L];
+  const int launches = t.ls == m.l0 ? 1 : cycles, per = t.ls == m.l0 ? cycles : 1;
+  for (int v = 0; v < launches; ++v) {
+    for (int l = m.l0; l < t.ls; ++l) {
+      if ((e = smooth2<T>(m.lv[l], m.st[l], prm.nu1, prm.omega, prm.colours2d, s))) return e;
+      if ((e = launch2_restrict<T>(m.lv[l].Nx, m.lv[l].Ny, m.st[l], m.lv[l].J, m.lv[l].R, m.lv[l].dU, m.lv[l + 1].R,
+                                   m.lv[l + 1].dU, m.lv[l].cm, s)))
+        return e;
+    }
+    const bool f = factor && v == 0;
+    if (f && (e = launch2_dense_factor<T>(C.Nx, C.Ny, m.st[m.L], C.J, reinterpret_cast<T *>(p->dense), p->piv, p->flag,
+                                          s)))
+      return e;
+    if ((e = launch2_vcycle_tail<T>(t, prm.nu1, prm.nu2, prm.omega, prm.colours2d, per, f, s))) return e;
+    for (int l = t.ls - 1; l >= m.l0; --l) {
+      if ((e = launch2_prolong<T>(m.lv[l].Nx, m.lv[l].Ny, m.lv[l].dU, m.lv[l + 1].dU, s))) return e;
+      if ((e = smooth2<T>(m.lv[l], m.st[l], prm.nu2, prm.omega, prm.colours2d, s))) return e;
+    }
   }
-  return cudaSuccess;
+  return e;
 }
 
 // Algorithm 3 for one 2D problem, sequenced from the host (one synchronisation
@@ -332,7 +344,7 @@ template <typename T>
 nswe_status solve2d_t(nswe_prob_s *p, const double *U0, double *U, const nswe_params &prm_in, nswe_info *info,
                       cudaStream_t s) {
   nswe_params prm;
-  int tail;
+  long tail;
   resolve2d(p, prm_in, prm, tail);
   const int L = p->levels - 1;
   const int s0 = (prm.nest_start < 0 || prm.nest_start > L) ? L : prm.nest_start;
@@ -358,7 +370,10 @@ nswe_status solve2d_t(nswe_prob_s *p, const double *U0, double *U, const nswe_pa
     // Colour-major J9 and Dinv on large levels solved by V-cycles (not on
     // the tail's levels, nor on the coarsest, whose J the dense LU reads).
     const int minc = p->ctx->cm2d_min_cells;
-    const int cm = (l < L && st0 == ST_J9 && minc >= 0 && n >= minc && n > tail) ? 1 : 0;
+    const int cm = (l < L && st0 == ST_J9 && minc >= 0 && n >= minc &&
+                    tail2_first<T>(p, l, st0, tail, kTail2MaxCtas) > l)
+                       ? 1
+                       : 0;
     T *const J = reinterpret_cast<T *>(Lv.J);
     T *const dU = reinterpret_cast<T *>(Lv.dU);
     T *const Rs = kMixed ? J + (size_t)K * 9 * blk_stride(cm, Lv.Nx, Lv.Ny) : reinterpret_cast<T *>(Lv.R);
@@ -374,13 +389,12 @@ nswe_status solve2d_t(nswe_prob_s *p, const double *U0, double *U, const nswe_pa
       if (l == L) {
         if ((e = launch2_dense_factor<T>(Lv.Nx, Lv.Ny, st0, J, reinterpret_cast<T *>(p->dense), p->piv, p->flag, q)) ||
             (e = launch2_dense_solve<T>(n, reinterpret_cast<const T *>(p->dense), p->piv, Rs,
-                                        reinterpret_cast<T *>(p->xbuf), dU, q)))
+                                        dU, q)))
           return e;
       } else {
         if ((e = mg2_setup<T>(p, m, q))) return e;
         if ((e = cudaMemsetAsync(dU, 0, sizeof(T) * 3 * n, q))) return e;
-        for (int v = 0; v < prm.nu3; ++v)
-          if ((e = mg2_vcycle<T>(p, m, prm, q, tail))) return e;
+        if ((e = mg2_vcycle<T>(p, m, prm, q, tail, prm.nu3, true))) return e;
       }
       if ((e = launch2_update<T>(n, Lv.U, dU, prm.tau, p->flag, q))) return e;
       if ((e = launch2_residual(p->dev2, l, Lv.Nx, Lv.Ny, Lv.U, Lv.R, p->res_dev, p->partials2, q))) return e;
@@ -526,7 +540,7 @@ nswe_status vcycle2d_entry(nswe_ctx ctx, nswe_prob prob, int level, int nb, cons
                            const nswe_params &prm_in) {
   if (nb != 9 && nb != 21) return NSWE_EINVAL;
   nswe_params prm;
-  int tail;
+  long tail;
   resolve2d(prob, prm_in, prm, tail);
   tail = ctx->tail2[std::is_same<T, float>::value ? 1 : 0];  // the standalone call's own precision
   MG2<T> m = mg2_bind<T>(prob, level, nb == 21 ? ST_J21 : ST_J9, J, R, dU, 0);
@@ -535,18 +549,17 @@ nswe_status vcycle2d_entry(nswe_ctx ctx, nswe_prob prob, int level, int nb, cons
     const int n = nswe_prob_cells(prob, level);
     return (launch2_dense_factor<T>(m.lv[level].Nx, m.lv[level].Ny, m.st[level], J,
                                     reinterpret_cast<T *>(prob->dense), prob->piv, prob->flag, ctx->stream) ||
-            launch2_dense_solve<T>(n, reinterpret_cast<const T *>(prob->dense), prob->piv, R,
-                                   reinterpret_cast<T *>(prob->xbuf), dU, ctx->stream))
+            launch2_dense_solve<T>(n, reinterpret_cast<const T *>(prob->dense), prob->piv, R, dU, ctx->stream))
                ? NSWE_ECUDA
                : NSWE_OK;
   }
-  return (mg2_setup<T>(prob, m, ctx->stream) || mg2_vcycle<T>(prob, m, prm, ctx->stream, tail)) ? NSWE_ECUDA
-                                                                                                : NSWE_OK;
+  return (mg2_setup<T>(prob, m, ctx->stream) || mg2_vcycle<T>(prob, m, prm, ctx->stream, tail, 1, true)) ? NSWE_ECUDA
+                                                                                                         : NSWE_OK;
 }
 
 }  // namespace
 
-void nswe::resolve2d(const nswe_prob_s *p, const nswe_params &in, nswe_params &out, int &tail) {
+void nswe::resolve2d(const nswe_prob_s *p, const nswe_params &in, nswe_params &out, long &tail) {
   out = in;
   const int prec = in.precision == NSWE_PREC_MIXED ? 1 : 0;
   tail = p->ctx->tail2[prec];
@@ -926,7 +939,6 @@ nswe_status nswe_prob_create_2d(nswe_ctx ctx, nswe_prob *out, int Nx, int Ny, in
   }
   p->dense = a;
   a += round_up(N3 * N3);
-  p->xbuf = a;
   a += round_up(N3);
   if (cudaMemcpyAsync(kind_dev, kinds.data(), sizeof(int) * nk, cudaMemcpyHostToDevice, ctx->stream)) ok = false;
   if (cudaMemcpyAsync(p->dev2, &p->host2, sizeof(ProbDev2), cudaMemcpyHostToDevice, ctx->stream)) ok = false;
@@ -1054,7 +1066,7 @@ nswe_status nswe_mg_smooth(nswe_ctx ctx, nswe_prob prob, int level, int nb, cons
   const Level2Dev &L = prob->host2.lev[level];
   const int stc = nb == 21 ? ST_J21 : ST_J9;
   nswe_params prm;
-  int tail;
+  long tail;
   resolve2d(prob, *params, prm, tail);
   Lev2<double> Lv{L.Nx, L.Ny, const_cast<double *>(J), L.Dinv, const_cast<double *>(R), dU, colour_major};
   int count = 0;
@@ -1131,13 +1143,13 @@ nswe_status autotune2d_t(nswe_ctx ctx, nswe_prob prob, const double *U, const ns
       nswe_params q = prm;
       q.colours2d = schedules[a];
       float t = 0.f;
-      if (cudaMemsetAsync(dU, 0, sizeof(T) * 3 * n, s) || mg2_vcycle<T>(prob, m, q, s, tails[b]) ||  // untimed
+      if (cudaMemsetAsync(dU, 0, sizeof(T) * 3 * n, s) || mg2_vcycle<T>(prob, m, q, s, tails[b], 1, true) ||  // untimed
           cudaEventRecord(e0, s)) {
         status = NSWE_ECUDA;
         break;
       }
       for (int r = 0; r < reps && status == NSWE_OK; ++r)
-        if (mg2_vcycle<T>(prob, m, q, s, tails[b])) status = NSWE_ECUDA;
+        if (mg2_vcycle<T>(prob, m, q, s, tails[b], 1, false)) status = NSWE_ECUDA;
       if (status != NSWE_OK || cudaEventRecord(e1, s) || cudaEventSynchronize(e1) ||
           cudaEventElapsedTime(&t, e0, e1)) {
         status = NSWE_ECUDA;

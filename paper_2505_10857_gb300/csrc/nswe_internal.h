@@ -141,28 +141,23 @@ cudaError_t launch2_prolong(int Nx, int Ny, T *dU, const T *dUc, cudaStream_t s)
 template <typename T>
 cudaError_t launch2_dense_factor(int Nx, int Ny, int st, const T *J, T *A, int *piv, int *flag, cudaStream_t s);
 template <typename T>
-cudaError_t launch2_dense_solve(int n, const T *A, const int *piv, const T *R, T *x, T *dU, cudaStream_t s);
+cudaError_t launch2_dense_solve(int n, const T *A, const int *piv, const T *R, T *dU, cudaStream_t s);
 template <typename T>
 cudaError_t launch2_update(int n, double *U, const T *dU, double tau, int *flag, cudaStream_t s);
 cudaError_t launch2_to_f32(long count, const double *src, float *dst, cudaStream_t s);
 
 // The levels ls..L of a 2D V-cycle (down-leg, coarsest solve with the dense
-// factors A/piv, up-leg) run by one thread block: the levels of at most
-// tail2_cells<T>() cells, where one launch per colour pass would cost
-// more than the pass. One SM issues FP32 at 64x its FP64 rate, so the FP64
-// tail stops at far smaller levels.
+// factors A/piv, up-leg) run by one thread-block cluster (nswe_cluster2d.cuh).
+constexpr int kTail2Threads = 512, kTail2MaxCtas = 16;
+// Levels of at most this many cells go to the cluster unless a threshold was
+// set (and if their bands fit its shared memory). FP32 levels gain whatever
+// their size; in FP64 the arithmetic of a larger level wants more than the 16
+// SMs of a cluster (a V-cycle at 256 x 128: 4.30 ms with 64 x 32 as the
+// largest level on the cluster, 4.50 with 128 x 64, 4.68 with 32 x 16).
 template <typename T>
-#ifndef NSWE_TAIL_F64
-#define NSWE_TAIL_F64 256
-#endif
-#ifndef NSWE_TAIL_F32
-#define NSWE_TAIL_F32 4096
-#endif
-constexpr int tail2_cells() { return sizeof(T) == 4 ? NSWE_TAIL_F32 : NSWE_TAIL_F64; }
-#ifndef NSWE_TAIL_THREADS
-#define NSWE_TAIL_THREADS 1024
-#endif
-constexpr int kTail2Threads = NSWE_TAIL_THREADS;
+constexpr long tail2_cells() {
+  return sizeof(T) == 4 ? 1L << 30 : 4096;
+}
 template <typename T>
 struct Tail2 {
   int ls, L;
@@ -170,10 +165,27 @@ struct Tail2 {
   T *J[NSWE_MAX_LEVELS], *Dinv[NSWE_MAX_LEVELS], *R[NSWE_MAX_LEVELS], *dU[NSWE_MAX_LEVELS];
   const T *A;
   const int *piv;
-  T *x;
+  // filled by plan_tail2
+  int l0, cm;                // the V-cycle's first level and the storage of its J and Dinv (blk_pos)
+  int ctas, threads;         // CTAs of the cluster and their threads
+  int shared_from;           // levels from here on share one place in shared memory, the others keep theirs
+  int off[NSWE_MAX_LEVELS];  // each level's place there (values of T)
+  int lu_off, lu_smem;       // the direct solve's, and whether the factors fit too
+  size_t smem;               // bytes per CTA
 };
+// Chooses ls >= l0 (the first level of at most max_cells cells that fits) and
+// the cluster of at most max_ctas CTAs; Nx, Ny, st of l0 .. L given. Returns ls.
 template <typename T>
-cudaError_t launch2_vcycle_tail(const Tail2<T> &t, int nu1, int nu2, double omega, int Kc, cudaStream_t s);
+int plan_tail2(Tail2<T> &t, int l0, int cm0, long max_cells, int max_ctas);
+// `cycles` V-cycles of the levels ls .. L. after_factor: the launch before it
+// on the stream is the coarsest factorisation (launch2_dense_factor), which it
+// may overlap.
+template <typename T>
+cudaError_t launch2_vcycle_tail(const Tail2<T> &t, int nu1, int nu2, double omega, int Kc, int cycles,
+                                bool after_factor, cudaStream_t s);
+// Inverse diagonal blocks of the levels l0 .. L - 1 (Nx, Ny, st, J, Dinv of t).
+template <typename T>
+cudaError_t launch2_dinv_levels(Tail2<T> t, int l0, int cm0, cudaStream_t s);
 cudaError_t launch2_interp(const ProbDev2 *p, int coarse_level, int nc, const double *Uc, double *Uf,
                            cudaStream_t s);
 
@@ -198,7 +210,7 @@ struct BTask2 {
   double *partials;      // residual partial sums (nb of them)
   float *R32;            // FP32 copy of R64 (mixed precision)
   double eps, alpha, tau;
-  T *A, *x;              // dense coarsest system and its solve buffer
+  T *A;                  // dense coarsest system
   int *piv;
 };
 // Launchers: tasks is a DEVICE array of ntask tasks sorted by b0, blocks the
@@ -230,15 +242,17 @@ template <typename T>
 cudaError_t launchb2_restrict(const Batch2Launch<T> &b, const int *done, cudaStream_t s);
 template <typename T>
 cudaError_t launchb2_prolong(const Batch2Launch<T> &b, const int *done, cudaStream_t s);
-// one block per task: the tail of each task's V-cycle (tails[i] for tasks[i])
+// one cluster of `ctas` CTAs per task: the tail of each task's V-cycle (tails[i] for tasks[i])
 template <typename T>
-cudaError_t launchb2_vcycle_tail(const Tail2<T> *tails, const BTask2<T> *tasks, int ntask, const int *done, int nu1,
-                                 int nu2, double omega, int Kc, cudaStream_t s);
+cudaError_t launchb2_vcycle_tail(const Tail2<T> *tails, const BTask2<T> *tasks, int ntask, int ctas, int threads,
+                                 size_t smem, const int *done, int nu1, int nu2, double omega, int Kc, int cycles,
+                                 bool after_factor, cudaStream_t s);
+// max_cells: the largest of the tasks' coarsest levels
 template <typename T>
 cudaError_t launchb2_dense_factor(const Batch2Launch<T> &zero, const Batch2Launch<T> &scatter, const BTask2<T> *tasks,
-                                  int ntask, const int *done, int *flags, cudaStream_t s);
+                                  int ntask, int max_cells, const int *done, int *flags, cudaStream_t s);
 template <typename T>
-cudaError_t launchb2_dense_solve(const BTask2<T> *tasks, int ntask, const int *done, cudaStream_t s);
+cudaError_t launchb2_dense_solve(const BTask2<T> *tasks, int ntask, int max_cells, const int *done, cudaStream_t s);
 template <typename T>
 cudaError_t launchb2_update(const Batch2Launch<T> &b, const int *done, int *flags, cudaStream_t s);
 int b2_grid(long items);  // blocks of kThreads for `items` grid-stride items (as the single launches)
@@ -253,7 +267,7 @@ nswe_status solve2d_lockstep(nswe_ctx ctx, int count, const nswe_prob *probs, co
 // colours2d = NSWE_COLOURS2D_AUTO takes the schedule and tail that
 // nswe_autotune_2d recorded for p's size and precision (none recorded:
 // schedule 0 and the context's tail).
-void resolve2d(const nswe_prob_s *p, const nswe_params &in, nswe_params &out, int &tail);
+void resolve2d(const nswe_prob_s *p, const nswe_params &in, nswe_params &out, long &tail);
 
 // One solve of a batch.
 struct SolveTask {
@@ -335,8 +349,8 @@ struct nswe_ctx_s {
   int team_cells = 1024; // cluster form: multigrid levels with at least this many cells on every CTA
   int batch2d_lockstep = 1;  // 2D batches: 1 lockstep batched launches (default), 0 concurrent solves
   int cm2d_min_cells = 131072;  // 2D Newton levels of at least this many cells store J9 colour-major
-  // 2D V-cycles: levels of at most tail2[precision] cells run in the one-block tail (0 FP64, 1 mixed)
-  int tail2[2] = {nswe::tail2_cells<double>(), nswe::tail2_cells<float>()};
+  // 2D V-cycles: levels of at most tail2[precision] cells (0 FP64, 1 mixed) run on one cluster
+  long tail2[2] = {nswe::tail2_cells<double>(), nswe::tail2_cells<float>()};
   std::vector<nswe_tuned2d> tuned2;  // nswe_autotune_2d's choices per size and precision
 };
 
@@ -357,7 +371,6 @@ struct nswe_prob_s {
   nswe::ProbDev2 *dev2;
   double *dense;         // coarsest dense LU factors [N3][N3]
   int *piv;              // [N3]
-  double *xbuf;          // [N3]
   int *flag;             // device flag (zero pivot / non-positive depth)
   double *res_dev;       // device scalar
   double *res_host;      // pinned host scalar
@@ -366,3 +379,18 @@ struct nswe_prob_s {
   double *partials2;     // 2D: [1024] per-block partial sums of res (per problem, so
                          // that several 2D solves can run concurrently)
 };
+
+namespace nswe {
+// First level that V-cycles from level l0 (stencil st0) of p run on the cluster.
+template <typename T>
+int tail2_first(const nswe_prob_s *p, int l0, int st0, long max_cells, int max_ctas) {
+  Tail2<T> t = {};
+  t.L = p->levels - 1;
+  for (int m = l0, st = st0; m <= t.L; ++m, st = st_coarse_host(st)) {
+    t.Nx[m] = p->Nx >> m;
+    t.Ny[m] = p->Ny >> m;
+    t.st[m] = st;
+  }
+  return plan_tail2<T>(t, l0, 0, max_cells, max_ctas);
+}
+}  // namespace nswe

@@ -57,7 +57,6 @@ __device__ __forceinline__ int st_off(int st, int k, int d) {
   return st == ST_J9 ? c_off_j9[k][d] : st == ST_J21 ? c_off_j21[k][d] : st == ST_P5 ? c_off_p5[k][d] : c_off_p9[k][d];
 }
 __device__ __forceinline__ int st_center(int st) { return st == ST_J9 ? 4 : st == ST_J21 ? 10 : st == ST_P5 ? 2 : 4; }
-__device__ __forceinline__ int st_coarse(int st) { return (st == ST_J9 || st == ST_P5) ? ST_P5 : ST_P9; }
 
 struct Geo2 {
   int Nx, Ny;
@@ -80,17 +79,6 @@ __device__ __forceinline__ Geo2 make_geo2(const ProbDev2 &P, int l) {
   return G;
 }
 
-// Largest colour pass (cells) that runs as k2_sor_split, per precision.
-#ifndef NSWE_SOR_SPLIT_F64
-#define NSWE_SOR_SPLIT_F64 (1L << 40)
-#endif
-#ifndef NSWE_SOR_SPLIT_F32
-#define NSWE_SOR_SPLIT_F32 (1L << 40)
-#endif
-#ifndef NSWE_SOR_UNROLL
-#define NSWE_SOR_UNROLL 1
-#endif
-constexpr long kSorSplitF64 = NSWE_SOR_SPLIT_F64, kSorSplitF32 = NSWE_SOR_SPLIT_F32;
 __device__ double block_sum2(double v, double *red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -144,34 +132,87 @@ __global__ void __launch_bounds__(kTile2Threads, 1) k2_jacobian(const ProbDev2 *
   jacobian_tiles2<TJ, FROZEN>(P, level, st, U, eps, alpha, R, J, cm, TX, TY, blockIdx.x, gridDim.x);
 }
 
+// Rounded products, the last steps of a smoother update and divisions,
+// written out so that all kernels of the smoother round alike.
+__device__ __forceinline__ double mul_r(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_r(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double div_r(double a, double b) { return fast_div(a, b, fast_rcp(b)); }
+__device__ __forceinline__ float div_r(float a, float b) { return __fdiv_rn(a, b); }
+// Row (d0, d1, d2) of the inverse diagonal block times r.
+template <typename T>
+__device__ __forceinline__ T dinv_row(T d0, T d1, T d2, T r0, T r1, T r2) {
+  return fma(d2, r2, fma(d0, r0, mul_r(d1, r1)));
+}
+// `reps` relaxations x := (1 - omega) x - omega t.
+template <typename T>
+__device__ __forceinline__ T relax(T x, T t, T omega, int reps) {
+  const T keep = T(1.0) - omega, wt = mul_r(omega, t);
+  for (int s = 0; s < reps; ++s) x = fma(keep, x, -wt);
+  return x;
+}
+
+// Galerkin coarse operator (Eq. 24), one item per (coarse cell, entry of its
+// 3x3 blocks): sums over the four fine cells of the aggregate and their
+// blocks, in that order. With the stencil known at compile time the coarse
+// block of every term is too, and the loads issue together; one thread per
+// coarse cell searching each term's block took 62 us at 64 x 32 in FP64.
+template <int ST>
+__device__ constexpr int off_c(int k, int d) {
+  constexpr int j9[9][2] = {{0, -2}, {0, -1}, {-2, 0}, {-1, 0}, {0, 0}, {1, 0}, {2, 0}, {0, 1}, {0, 2}};
+  constexpr int p5[5][2] = {{0, -1}, {-1, 0}, {0, 0}, {1, 0}, {0, 1}};
+  constexpr int p9[9][2] = {{-1, -1}, {0, -1}, {1, -1}, {-1, 0}, {0, 0}, {1, 0}, {-1, 1}, {0, 1}, {1, 1}};
+  constexpr int j21[21][2] = {{-1, -2}, {0, -2}, {1, -2}, {-2, -1}, {-1, -1}, {0, -1}, {1, -1},
+                              {2, -1},  {-2, 0}, {-1, 0}, {0, 0},   {1, 0},   {2, 0},  {-2, 1},
+                              {-1, 1},  {0, 1},  {1, 1},  {2, 1},   {-1, 2},  {0, 2},  {1, 2}};
+  return ST == ST_J9 ? j9[ST == ST_J9 ? k : 0][d] : ST == ST_P5 ? p5[ST == ST_P5 ? k : 0][d]
+                     : ST == ST_P9 ? p9[ST == ST_P9 ? k : 0][d] : j21[k][d];
+}
+// The coarse block that a fine cell (a, b) of its aggregate couples to through block k.
+template <int ST>
+__device__ constexpr int coarse_block(int a, int b, int k) {
+  constexpr int CS = (ST == ST_J9 || ST == ST_P5) ? ST_P5 : ST_P9;
+  const int ox = a + off_c<ST>(k, 0), oy = b + off_c<ST>(k, 1);
+  const int fx = ox < 0 ? (ox - 1) / 2 : ox / 2, fy = oy < 0 ? (oy - 1) / 2 : oy / 2;
+  for (int t = 0; t < (CS == ST_P5 ? 5 : 9); ++t)
+    if (off_c<CS>(t, 0) == fx && off_c<CS>(t, 1) == fy) return t;
+  return -1;
+}
+
+template <typename T, int ST>
+__device__ __forceinline__ void coarse_op_items2(int Nx, int Ny, const T *Jf, T *Jc, int cm, int first, int stride) {
+  constexpr int K = ST == ST_J9 ? 9 : ST == ST_J21 ? 21 : ST == ST_P5 ? 5 : 9;
+  constexpr int Kc = (ST == ST_J9 || ST == ST_P5) ? 5 : 9;
+  const int Ncx = Nx / 2, nc = Ncx * (Ny / 2);
+  const size_t Sf = blk_stride(cm, Nx, Ny);
+  for (int w = first; w < 9 * nc; w += stride) {
+    const int e = w / nc, cc = w % nc, I = cc % Ncx, Jy = cc / Ncx;
+    T acc[Kc];
+#pragma unroll
+    for (int t = 0; t < Kc; ++t) acc[t] = T(0.0);
+#pragma unroll
+    for (int ab = 0; ab < 4; ++ab) {
+      const int a = ab & 1, b = ab >> 1, xi = 2 * I + a, yi = 2 * Jy + b;
+      const T *J = Jf + (size_t)e * Sf + blk_pos(cm, Nx, Ny, xi, yi);
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const int ex = xi + off_c<ST>(k, 0), ey = yi + off_c<ST>(k, 1);
+        const bool in = ex >= 0 && ex < Nx && ey >= 0 && ey < Ny;
+        const T v = J[(size_t)(k * 9) * Sf];
+        acc[coarse_block<ST>(a, b, k)] += in ? v : T(0.0);
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < Kc; ++t) Jc[(size_t)(t * 9 + e) * nc + cc] = acc[t];
+  }
+}
+
 template <typename T>
 __device__ __forceinline__ void coarse_op_cells2(int Nx, int Ny, int st, const T *Jf, T *Jc, int cm, int first,
                                                  int stride) {
-  const int Ncx = Nx / 2, Ncy = Ny / 2, nc = Ncx * Ncy, K = st_size(st), cs = st_coarse(st), Kc = st_size(cs);
-  const size_t Sf = blk_stride(cm, Nx, Ny);
-  for (int cc = first; cc < nc; cc += stride) {
-    const int I = cc % Ncx, Jy = cc / Ncx;
-    T acc[9][9];
-    for (int t = 0; t < Kc; ++t)
-      for (int e = 0; e < 9; ++e) acc[t][e] = T(0.0);
-    for (int b = 0; b < 2; ++b)
-      for (int a = 0; a < 2; ++a) {
-        const int xi = 2 * I + a, yi = 2 * Jy + b;
-        const size_t c = blk_pos(cm, Nx, Ny, xi, yi);
-        for (int k = 0; k < K; ++k) {
-          const int ex = xi + st_off(st, k, 0), ey = yi + st_off(st, k, 1);
-          if (ex < 0 || ex >= Nx || ey < 0 || ey >= Ny) continue;
-          const int ox = ex / 2 - I, oy = ey / 2 - Jy;
-          int kk = -1;
-          for (int t = 0; t < Kc; ++t)
-            if (st_off(cs, t, 0) == ox && st_off(cs, t, 1) == oy) kk = t;
-          if (kk < 0) continue;
-          for (int e = 0; e < 9; ++e) acc[kk][e] += Jf[(size_t)(k * 9 + e) * Sf + c];
-        }
-      }
-    for (int t = 0; t < Kc; ++t)
-      for (int e = 0; e < 9; ++e) Jc[(size_t)(t * 9 + e) * nc + cc] = acc[t][e];
-  }
+  if (st == ST_J9) coarse_op_items2<T, ST_J9>(Nx, Ny, Jf, Jc, cm, first, stride);
+  else if (st == ST_P5) coarse_op_items2<T, ST_P5>(Nx, Ny, Jf, Jc, cm, first, stride);
+  else if (st == ST_J21) coarse_op_items2<T, ST_J21>(Nx, Ny, Jf, Jc, cm, first, stride);
+  else coarse_op_items2<T, ST_P9>(Nx, Ny, Jf, Jc, cm, first, stride);
 }
 
 template <typename T>
@@ -189,17 +230,16 @@ __device__ __forceinline__ void dinv_cells2(int Nx, int Ny, int st, const T *J, 
     const size_t c = blk_pos(cm, Nx, Ny, q % Nx, q / Nx);
     T a[9];
     for (int e = 0; e < 9; ++e) a[e] = J[(size_t)(kc * 9 + e) * n + c];
-    const T c00 = a[4] * a[8] - a[5] * a[7], c01 = a[5] * a[6] - a[3] * a[8], c02 = a[3] * a[7] - a[4] * a[6];
-    const T det = a[0] * c00 + a[1] * c01 + a[2] * c02;
-    Dinv[0 * (size_t)n + c] = c00 / det;
-    Dinv[1 * (size_t)n + c] = (a[2] * a[7] - a[1] * a[8]) / det;
-    Dinv[2 * (size_t)n + c] = (a[1] * a[5] - a[2] * a[4]) / det;
-    Dinv[3 * (size_t)n + c] = c01 / det;
-    Dinv[4 * (size_t)n + c] = (a[0] * a[8] - a[2] * a[6]) / det;
-    Dinv[5 * (size_t)n + c] = (a[2] * a[3] - a[0] * a[5]) / det;
-    Dinv[6 * (size_t)n + c] = c02 / det;
-    Dinv[7 * (size_t)n + c] = (a[1] * a[6] - a[0] * a[7]) / det;
-    Dinv[8 * (size_t)n + c] = (a[0] * a[4] - a[1] * a[3]) / det;
+    // cofactors over the determinant
+    const auto minor = [](T p, T q, T r, T t) { return fma(p, q, -mul_r(r, t)); };
+    const T c00 = minor(a[4], a[8], a[5], a[7]), c01 = minor(a[5], a[6], a[3], a[8]),
+            c02 = minor(a[3], a[7], a[4], a[6]);
+    const T det = fma(a[2], c02, fma(a[0], c00, mul_r(a[1], c01)));
+    const T inv[9] = {c00, minor(a[2], a[7], a[1], a[8]), minor(a[1], a[5], a[2], a[4]),
+                      c01, minor(a[0], a[8], a[2], a[6]), minor(a[2], a[3], a[0], a[5]),
+                      c02, minor(a[1], a[6], a[0], a[7]), minor(a[0], a[4], a[1], a[3])};
+#pragma unroll
+    for (int e = 0; e < 9; ++e) Dinv[(size_t)e * n + c] = div_r(inv[e], det);
   }
 }
 
@@ -209,39 +249,16 @@ __global__ void __launch_bounds__(kThreads) k2_dinv(int Nx, int Ny, int st, cons
   dinv_cells2<T>(Nx, Ny, st, J, Dinv, cm, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
-// Block SOR update (Eq. 22) of cell (i, j), relaxation applied reps times
-// (consecutive visits of a colour see the same neighbours).
+// The inverse diagonal blocks of the levels l0 .. L - 1 of a hierarchy in one
+// launch: block x of the grid takes blocks of the level that block0 puts it in.
 template <typename T>
-__device__ __forceinline__ void sor_cell2(int Nx, int Ny, int st, const T *J, const T *Dinv, const T *R, T *dU,
-                                          double omega_d, int reps, int i, int j, int cm) {
-  const T omega = T(omega_d);
-  const int n = Nx * Ny, K = st_size(st), kc = st_center(st), c = j * Nx + i;
-  const size_t S = blk_stride(cm, Nx, Ny), pc = blk_pos(cm, Nx, Ny, i, j);  // J, Dinv
-  T r[3] = {R[c], R[n + c], R[2 * n + c]};
-  for (int k = 0; k < K; ++k) {
-    if (k == kc) continue;
-    const int p = i + st_off(st, k, 0), q = j + st_off(st, k, 1);
-    if (p < 0 || p >= Nx || q < 0 || q >= Ny) continue;
-    const int cp = q * Nx + p;
-    const T x0 = dU[cp], x1 = dU[n + cp], x2 = dU[2 * n + cp];
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {  // a chain of fused multiply-adds (the order of sor_pass_split)
-      r[l] = fma(J[(size_t)(k * 9 + l * 3 + 0) * S + pc], x0, r[l]);
-      r[l] = fma(J[(size_t)(k * 9 + l * 3 + 1) * S + pc], x1, r[l]);
-      r[l] = fma(J[(size_t)(k * 9 + l * 3 + 2) * S + pc], x2, r[l]);
-    }
-  }
-  T t[3];
-#pragma unroll
-  for (int l = 0; l < 3; ++l)
-    t[l] = Dinv[(size_t)(l * 3 + 0) * S + pc] * r[0] + Dinv[(size_t)(l * 3 + 1) * S + pc] * r[1] +
-           Dinv[(size_t)(l * 3 + 2) * S + pc] * r[2];
-#pragma unroll
-  for (int l = 0; l < 3; ++l) {
-    T x = dU[l * n + c];
-    for (int s = 0; s < reps; ++s) x = (T(1.0) - omega) * x - omega * t[l];
-    dU[l * n + c] = x;
-  }
+__global__ void __launch_bounds__(kThreads) k2_dinv_levels(const __grid_constant__ Tail2<T> t, int l0) {
+  pdl_enter();
+  int l = l0;
+  while (l + 1 < t.L && (int)blockIdx.x >= t.off[l + 1]) ++l;
+  const int nb = t.off[l + 1] - t.off[l];
+  dinv_cells2<T>(t.Nx[l], t.Ny[l], t.st[l], t.J[l], t.Dinv[l], l == l0 ? t.cm : 0,
+                 (blockIdx.x - t.off[l]) * blockDim.x + threadIdx.x, nb * blockDim.x);
 }
 
 // The cells of colour col, enumerated directly so that every lane of a warp
@@ -269,36 +286,7 @@ __device__ __forceinline__ void sor_items(int Nx, int Ny, int st, int &mode, int
   }
 }
 
-// One colour pass over the items first, first + stride, ... (a grid-wide or a
-// block-wide stride).
-template <typename T>
-__device__ void sor_pass(int Nx, int Ny, int st, const T *J, const T *Dinv, const T *R, T *dU, double omega,
-                         int mode, int Kc, int col, int reps, int first, int stride, int cm = 0) {
-  int P, W, items;
-  sor_items(Nx, Ny, st, mode, Kc, col, P, W, items);
-  if (mode == 0) {
-    const int a = col % P, b = col / P;
-    for (int t = first; t < items; t += stride)
-      sor_cell2(Nx, Ny, st, J, Dinv, R, dU, omega, reps, a + (t % W) * P, b + (t / W) * P, cm);
-    return;
-  }
-  for (int t = first; t < items; t += stride) {
-    const int j = t / W, m = t % W;
-    const int a = mode == 1 ? col - j : j + Nx - 1 - col;
-    const int i = ((a % Kc) + Kc) % Kc + m * Kc;
-    if (i < Nx) sor_cell2(Nx, Ny, st, J, Dinv, R, dU, omega, reps, i, j, cm);
-  }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k2_sor(int Nx, int Ny, int st, const T *J, const T *Dinv, const T *R,
-                                                   T *dU, double omega, int mode, int Kc, int col, int reps, int cm) {
-  pdl_enter();
-  sor_pass<T>(Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, blockIdx.x * blockDim.x + threadIdx.x,
-              gridDim.x * blockDim.x, cm);
-}
-
-// Cell (i, j) of item t of a colour pass (the enumeration of sor_pass);
+// Cell (i, j) of item t of a colour pass (the enumeration of sor_items);
 // false if the item lies beyond the grid.
 __device__ __forceinline__ bool sor_item_cell(int Nx, int mode, int Kc, int col, int P, int W, int t, int &i, int &j) {
   if (mode == 0) {
@@ -312,10 +300,10 @@ __device__ __forceinline__ bool sor_item_cell(int Nx, int mode, int Kc, int col,
   return i < Nx;
 }
 
-// The same colour pass with three lanes per cell: lane l of a cell's group
-// forms component l of r = R + sum_k J_k dU_k (the expression of sor_cell2,
-// so the results are the same bits), the group exchanges r by shuffles, and
-// lane l updates dU component l. Ten cells per warp (lanes 30, 31 idle). On
+// One colour pass of the block SOR (Eq. 22), relaxation applied reps times
+// (consecutive visits of a colour see the same neighbours), with three lanes
+// per cell: lane l of a cell's group forms component l of r = R + sum_k J_k
+// dU_k, the group exchanges r by shuffles, and lane l updates dU component l. Ten cells per warp (lanes 30, 31 idle). On
 // small grids this spreads a pass over three times as many warps, each with a
 // third of the dependent FP64 instructions: an FP64 warp instruction holds
 // its SMSP's FP64 unit for tens of cycles, so the length of one thread's
@@ -355,11 +343,9 @@ __device__ __forceinline__ void sor_pass_split(int Nx, int Ny, int st_arg, const
     const T r1 = __shfl_sync(0xffffffffu, r, min(src + 1, 31));
     const T r2 = __shfl_sync(0xffffffffu, r, min(src + 2, 31));
     if (on) {
-      const T tl = Dinv[(size_t)(l * 3 + 0) * S + pc] * r0 + Dinv[(size_t)(l * 3 + 1) * S + pc] * r1 +
-                   Dinv[(size_t)(l * 3 + 2) * S + pc] * r2;
-      T x = dU[l * n + c];
-      for (int s = 0; s < reps; ++s) x = (T(1.0) - omega) * x - omega * tl;
-      dU[l * n + c] = x;
+      const T tl = dinv_row(Dinv[(size_t)(l * 3 + 0) * S + pc], Dinv[(size_t)(l * 3 + 1) * S + pc],
+                            Dinv[(size_t)(l * 3 + 2) * S + pc], r0, r1, r2);
+      dU[l * n + c] = relax(dU[l * n + c], tl, omega, reps);
     }
   }
 }
@@ -371,25 +357,6 @@ __global__ void __launch_bounds__(kThreads) k2_sor_split(int Nx, int Ny, int st,
   pdl_enter();
   sor_pass_split<T, STC>(Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps,
                          (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5, cm);
-}
-
-// A colour pass by the threads of one block (the tail kernel): in FP64 split
-// as above; in FP32, where the dependent chains are short, one thread per
-// cell measured faster.
-template <typename T>
-__device__ void sor_pass_block_split(int Nx, int Ny, int st, const T *J, const T *Dinv, const T *R, T *dU,
-                                     double omega, int mode, int Kc, int col, int reps) {
-  if (!std::is_same<T, double>::value) {
-    sor_pass<T>(Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, threadIdx.x, blockDim.x);
-    return;
-  }
-  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (st == ST_J9)
-    sor_pass_split<T, ST_J9>(Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, w, nw, 0);
-  else if (st == ST_P5)
-    sor_pass_split<T, ST_P5>(Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, w, nw, 0);
-  else
-    sor_pass_split<T, -1>(Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, w, nw, 0);
 }
 
 template <typename T>
@@ -534,12 +501,12 @@ __device__ void lu_block2(int N3, T *A, int *piv, int *flag) {
       }
     __syncthreads();
     const T d = A[(size_t)k * N3 + k];
-    for (int i = k + 1 + threadIdx.x; i < N3; i += blockDim.x) A[(size_t)i * N3 + k] = A[(size_t)i * N3 + k] / d;
+    for (int i = k + 1 + threadIdx.x; i < N3; i += blockDim.x) A[(size_t)i * N3 + k] = div_r(A[(size_t)i * N3 + k], d);
     __syncthreads();
     const int rows = N3 - k - 1;
     for (int t = threadIdx.x; t < rows * rows; t += blockDim.x) {
       const int i = k + 1 + t / rows, c = k + 1 + t % rows;
-      A[(size_t)i * N3 + c] -= A[(size_t)i * N3 + k] * A[(size_t)k * N3 + c];
+      A[(size_t)i * N3 + c] = fma(-A[(size_t)i * N3 + k], A[(size_t)k * N3 + c], A[(size_t)i * N3 + c]);
     }
     __syncthreads();
   }
@@ -551,106 +518,137 @@ __global__ void __launch_bounds__(kThreads) k2_lu(int N3, T *A, int *piv, int *f
   lu_block2<T>(N3, A, piv, flag);
 }
 
-// dU = -A^{-1} R with the factors (one warp; unknown 3c+m).
-// Called by the 32 lanes of one warp (lane = threadIdx.x & 31).
-template <typename T>
-__device__ void lu_solve_warp(int n, const T *A, const int *piv, const T *R, T *x, T *dU) {
-  const int N3 = 3 * n, lane = threadIdx.x & 31;
-  for (int t = lane; t < n; t += 32)
-    for (int m = 0; m < 3; ++m) x[3 * t + m] = -R[m * n + t];
-  __syncwarp();
-  for (int k = 0; k < N3; ++k) {
-    const int p = piv[k];
-    if (lane == 0 && p != k) {
-      const T t = x[k];
-      x[k] = x[p];
-      x[p] = t;
-    }
-    __syncwarp();
-    const T xk = x[k];
-    for (int i = k + 1 + lane; i < N3; i += 32) x[i] -= A[(size_t)i * N3 + k] * xk;
-    __syncwarp();
-  }
-  for (int i = N3 - 1; i >= 0; --i) {
-    T s = T(0.0);
-    for (int c = i + 1 + lane; c < N3; c += 32) s += A[(size_t)i * N3 + c] * x[c];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) x[i] = (x[i] - s) / A[(size_t)i * N3 + i];
-    __syncwarp();
-  }
-  for (int t = lane; t < n; t += 32)
-    for (int m = 0; m < 3; ++m) dU[m * n + t] = x[3 * t + m];
+// The row of largest |a| among the lanes' (a, row), ties to the lowest row: the
+// bit patterns of non-negative values order as the values (a NaN counts as 0),
+// so the integer reductions of the warp find it.
+__device__ __forceinline__ int pivot_row2(float a, int row) {
+  const unsigned key = a == a ? __float_as_uint(a) & 0x7fffffffu : 0u;
+  const unsigned m = __reduce_max_sync(0xffffffffu, row >= 0 ? key : 0u);
+  return (int)__reduce_min_sync(0xffffffffu, row >= 0 && key == m ? (unsigned)row : 0xffffffffu);
+}
+__device__ __forceinline__ int pivot_row2(double a, int row) {
+  const unsigned hi = a == a ? (unsigned)__double2hiint(a) & 0x7fffffffu : 0u;
+  const unsigned lo = a == a ? (unsigned)__double2loint(a) : 0u;
+  const unsigned mh = __reduce_max_sync(0xffffffffu, row >= 0 ? hi : 0u);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, row >= 0 && hi == mh ? lo : 0u);
+  return (int)__reduce_min_sync(0xffffffffu, row >= 0 && hi == mh && lo == ml ? (unsigned)row : 0xffffffffu);
+}
+// |a| > |b| as the keys above order them.
+__device__ __forceinline__ bool larger2(float a, float b) { return !(b == b) ? a == a && a != 0.0f : fabsf(a) > fabsf(b); }
+__device__ __forceinline__ bool larger2(double a, double b) {
+  const unsigned long long ka = a == a ? (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull : 0ull;
+  const unsigned long long kb = b == b ? (unsigned long long)__double_as_longlong(b) & 0x7fffffffffffffffull : 0ull;
+  return ka > kb;
 }
 
+// The dense coarsest system of block operator J (cell-contiguous) assembled
+// in shared memory, factored there as lu_block2 does (the same pivots and
+// updates), and written to A; by one block of kLu2Threads. Every warp finds
+// the pivot itself and forms the multipliers of its own rows (one lane each),
+// so a step without an exchange of rows has one barrier; four warps up to 128
+// unknowns, one per FP64 unit.
 template <typename T>
-__global__ void k2_lu_solve(int n, const T *A, const int *piv, const T *R, T *x, T *dU) {
-  pdl_enter();
-  if (threadIdx.x < 32) lu_solve_warp<T>(n, A, piv, R, x, dU);
-}
-
-// Smoothing of level l by the calling block, the same sequence of colour
-// passes as the host's schedule (directional: four diagonal sweeps per step;
-// otherwise two symmetric passes of the stencil colouring with consecutive
-// visits of a colour fused).
-__device__ __forceinline__ int st_ncolours(int st) { return st == ST_J9 ? 3 : st == ST_J21 ? 9 : st == ST_P5 ? 2 : 4; }
-
-template <typename T>
-__device__ void smooth_block(const Tail2<T> &t, int l, int steps, double omega, int Kc) {
-  const int Nx = t.Nx[l], Ny = t.Ny[l], st = t.st[l];
-  if (Kc >= 3 && (st == ST_J9 || st == ST_P5)) {
-    for (int s = 0; s < steps; ++s)
-      for (int d = 0; d < 4; ++d)
-        for (int q = 0; q < Kc; ++q) {
-          const int mode = (d % 2) + 1, col = d < 2 ? q : Kc - 1 - q;
-          sor_pass_block_split<T>(Nx, Ny, st, t.J[l], t.Dinv[l], t.R[l], t.dU[l], omega, mode, Kc, col, 1);
-          __syncthreads();
-        }
-    return;
-  }
-  const int C = st_ncolours(st);
-  int prev = -1, reps = 0;
-  for (int s = 0; s < steps; ++s)
-    for (int pass = 0; pass < 4 * C; ++pass) {
-      const int q = pass % (2 * C), col = q < C ? q : 2 * C - 1 - q;
-      if (col == prev) {
-        ++reps;
-        continue;
-      }
-      if (prev >= 0) {
-        sor_pass_block_split<T>(Nx, Ny, st, t.J[l], t.Dinv[l], t.R[l], t.dU[l], omega, 0, 0, prev, reps);
-        __syncthreads();
-      }
-      prev = col;
-      reps = 1;
-    }
-  if (prev >= 0) {
-    sor_pass_block_split<T>(Nx, Ny, st, t.J[l], t.Dinv[l], t.R[l], t.dU[l], omega, 0, 0, prev, reps);
-    __syncthreads();
-  }
-}
-
-template <typename T>
-__device__ void vcycle_tail_block2(const Tail2<T> &t, int nu1, int nu2, double omega, int Kc) {
-  for (int l = t.ls; l < t.L; ++l) {
-    smooth_block<T>(t, l, nu1, omega, Kc);
-    restrict_cells2<T>(t.Nx[l], t.Ny[l], t.st[l], t.J[l], t.R[l], t.dU[l], t.R[l + 1], t.dU[l + 1], threadIdx.x,
-                       blockDim.x);
-    __syncthreads();
-  }
-  if (threadIdx.x < 32) lu_solve_warp<T>(t.Nx[t.L] * t.Ny[t.L], t.A, t.piv, t.R[t.L], t.x, t.dU[t.L]);
+__device__ void lu_smem_block2(int Nx, int Ny, int st, const T *J, T *A, int *piv, int *flag) {
+  extern __shared__ __align__(16) unsigned char g_lu2_smem[];
+  T *M = reinterpret_cast<T *>(g_lu2_smem);
+  const int n = Nx * Ny, N3 = 3 * n, ld = N3 + 1, K = st_size(st);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int t = threadIdx.x; t < N3 * ld; t += blockDim.x) M[t] = T(0.0);
   __syncthreads();
-  for (int l = t.L - 1; l >= t.ls; --l) {
-    prolong_cells2<T>(t.Nx[l], t.Ny[l], t.dU[l], t.dU[l + 1], threadIdx.x, blockDim.x);
-    __syncthreads();
-    smooth_block<T>(t, l, nu2, omega, Kc);
+  for (int t = threadIdx.x; t < 9 * n * K; t += blockDim.x) {
+    const int c = t % n, ke = t / n, k = ke / 9, e = ke % 9, p = c % Nx + st_off(st, k, 0), q = c / Nx + st_off(st, k, 1);
+    if (p >= 0 && p < Nx && q >= 0 && q < Ny) M[(3 * c + e / 3) * ld + 3 * (q * Nx + p) + e % 3] = J[(size_t)ke * n + c];
   }
+  __syncthreads();
+  for (int k = 0; k < N3; ++k) {
+    T best = T(0.0);
+    int row = -1;
+    for (int i = k + lane; i < N3; i += 32) {
+      const T a = M[i * ld + k];
+      if (row < 0 || larger2(a, best)) {
+        best = a;
+        row = i;
+      }
+    }
+    const int p = pivot_row2(best, row);
+    if (threadIdx.x == 0) {
+      piv[k] = p;
+      if (M[p * ld + k] == T(0.0)) *flag = 1;
+    }
+    if (p != k) {  // block-uniform; only the active columns, as lu_block2
+      __syncthreads();
+      for (int c = k + threadIdx.x; c < N3; c += blockDim.x) {
+        const T t = M[k * ld + c];
+        M[k * ld + c] = M[p * ld + c];
+        M[p * ld + c] = t;
+      }
+      __syncthreads();
+    }
+    // rows k + 1 + warp, + nw, ...: at most 32 of them (lu2_smem). The matrix
+    // is banded: rows whose multiplier is zero and columns whose pivot-row
+    // entries are zero keep their values, unless the other factor is not finite.
+    const int first = k + 1 + warp, rows = first < N3 ? (N3 - first + nw - 1) / nw : 0;
+    T mult = T(0.0);
+    if (lane < rows) {
+      const T a = M[(first + lane * nw) * ld + k], d = M[k * ld + k];
+      mult = a == T(0.0) && d != T(0.0) && isfinite(d) ? T(0.0) : -div_r(a, d);
+    }
+    const unsigned nz = __ballot_sync(0xffffffffu, mult != T(0.0));
+    const bool odd_mult = __any_sync(0xffffffffu, !isfinite(mult));
+    for (int c0 = k + 1; c0 < N3; c0 += 32) {
+      const int c = c0 + lane;
+      const T u = c < N3 ? M[k * ld + c] : T(0.0);
+      if (!odd_mult && !__any_sync(0xffffffffu, u != T(0.0))) continue;
+      const unsigned todo = __any_sync(0xffffffffu, !isfinite(u)) ? 0xffffffffu : nz;
+      for (int q = 0; q < rows; q += 4) {
+        if (!((todo >> q) & 15u)) continue;
+        T *a = M + (first + q * nw) * ld + c, v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = q + i < rows && c < N3 ? a[i * nw * ld] : T(0.0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = fma(__shfl_sync(0xffffffffu, mult, (q + i) & 31), u, v[i]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (q + i < rows && c < N3) a[i * nw * ld] = v[i];
+      }
+    }
+    __syncthreads();  // every warp has searched column k: it may take the multipliers
+    if (lane < rows) M[(first + lane * nw) * ld + k] = -mult;
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < N3 * N3; t += blockDim.x) A[t] = M[(t / N3) * ld + t % N3];
+}
+
+constexpr int kLu2Threads = 256;
+inline int lu2_threads(int N3) { return N3 <= 128 ? 128 : kLu2Threads; }
+
+template <typename T>
+__global__ void __launch_bounds__(kLu2Threads, 1) k2_lu_smem(int Nx, int Ny, int st, const T *J, T *A, int *piv,
+                                                             int *flag) {
+  pdl_enter();
+  lu_smem_block2<T>(Nx, Ny, st, J, A, piv, flag);
+}
+
+}  // namespace
+}  // namespace nswe
+
+#include "nswe_cluster2d.cuh"
+
+namespace nswe {
+namespace {
+
+extern __shared__ __align__(16) unsigned char g_lus2_smem[];
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k2_lu_solve(int n, const T *A, const int *piv, const T *R, T *dU) {
+  pdl_enter();
+  lu_solve_block<T>(n, A, 3 * n, 1, piv, R, reinterpret_cast<T *>(g_lus2_smem), dU);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kTail2Threads, 1) k2_vcycle_tail(Tail2<T> t, int nu1, int nu2, double omega,
-                                                                  int Kc) {
-  pdl_enter();
-  vcycle_tail_block2<T>(t, nu1, nu2, omega, Kc);
+__global__ void __launch_bounds__(kTail2Threads, 1) k2_vcycle_tail(const __grid_constant__ Tail2<T> t, int nu1, int nu2,
+                                                                  double omega, int Kc, int cycles) {
+  vcycle_cluster2<T>(t, nu1, nu2, omega, Kc, cycles);
 }
 
 __global__ void __launch_bounds__(kThreads) k2_to_f32(long count, const double *src, float *dst) {
@@ -743,19 +741,27 @@ void launchk2(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Arg
   launchk2s(kern, grid, block, 0, s, std::forward<Args>(args)...);
 }
 
-// Launches a tile kernel with `smem` bytes of dynamic shared memory; the
-// kernel's limit is raised once per device (up to the 227 KB of an SM).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_tile2(std::atomic<unsigned> &raised, void (*kern)(KArgs...), int grid, size_t smem, cudaStream_t s,
-                         Args &&...args) {
+// Raises a kernel's limit of dynamic shared memory to that of an SM (227 KB
+// less a little static), and with `clusters` allows cluster sizes above 8;
+// once per device.
+template <typename... KArgs>
+cudaError_t raise_smem(std::atomic<unsigned> &raised, void (*kern)(KArgs...), bool clusters = false) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const unsigned bit = 1u << (dev & 31);
-  if (!(raised.load(std::memory_order_acquire) & bit)) {
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTile2MaxSmem))) return e;
-    raised.fetch_or(bit, std::memory_order_release);
-  }
+  if (raised.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTile2MaxSmem))) return e;
+  if (clusters && (e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1))) return e;
+  raised.fetch_or(bit, std::memory_order_release);
+  return cudaSuccess;
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_tile2(std::atomic<unsigned> &raised, void (*kern)(KArgs...), int grid, size_t smem, cudaStream_t s,
+                         Args &&...args) {
+  const cudaError_t e = raise_smem(raised, kern);
+  if (e != cudaSuccess) return e;
   launchk2s(kern, grid, kTile2Threads, smem, s, std::forward<Args>(args)...);
   return cudaGetLastError();
 }
@@ -827,13 +833,26 @@ cudaError_t launch2_jacobian(const ProbDev2 *p, int level, int Nx, int Ny, int s
 
 template <typename T>
 cudaError_t launch2_coarse_op(int Nx, int Ny, int st, const T *Jf, T *Jc, int cm, cudaStream_t s) {
-  launchk2(k2_coarse_op<T>, grid2((long)(Nx / 2) * (Ny / 2)), kThreads, s, Nx, Ny, st, Jf, Jc, cm);
+  launchk2(k2_coarse_op<T>, grid2(9L * (Nx / 2) * (Ny / 2)), kThreads, s, Nx, Ny, st, Jf, Jc, cm);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch2_dinv(int Nx, int Ny, int st, const T *J, T *Dinv, int cm, cudaStream_t s) {
   launchk2(k2_dinv<T>, grid2((long)Nx * Ny), kThreads, s, Nx, Ny, st, J, Dinv, cm);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch2_dinv_levels(Tail2<T> t, int l0, int cm0, cudaStream_t s) {
+  int blocks = 0;
+  for (int l = l0; l < t.L; ++l) {
+    t.off[l] = blocks;
+    blocks += grid2((long)t.Nx[l] * t.Ny[l]);
+  }
+  t.off[t.L] = blocks;
+  t.cm = cm0;
+  if (blocks) launchk2(k2_dinv_levels<T>, blocks, kThreads, s, t, l0);
   return cudaGetLastError();
 }
 
@@ -845,21 +864,17 @@ cudaError_t launch2_sor(int Nx, int Ny, int st, const T *J, const T *Dinv, const
   if (mode == 0 && (st == ST_J9 || st == ST_P5)) items = (long)((Nx + (st == ST_J9 ? 3 : 2) - 1) / (st == ST_J9 ? 3 : 2)) * Ny;
   else if (mode == 0) items = (long)((Nx + 2) / (st == ST_J21 ? 3 : 2) + 1) * ((Ny + 2) / (st == ST_J21 ? 3 : 2) + 1);
   else items = (long)((Nx + Kc - 1) / Kc) * Ny;
-  if (items <= (std::is_same<T, double>::value ? kSorSplitF64 : kSorSplitF32)) {
-    // three lanes per cell; one warp per block on small passes so that the
-    // block scheduler spreads the warps over the SMs
-    const long warps = (items + 9) / 10;
-    const int bs = warps <= 4L * 152 ? 32 : 128;
-    const unsigned grid = (unsigned)((warps * 32 + bs - 1) / bs);
-    if (NSWE_SOR_UNROLL && st == ST_J9)
-      launchk2(k2_sor_split<T, ST_J9>, grid, bs, s, Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, cm);
-    else if (NSWE_SOR_UNROLL && st == ST_P5)
-      launchk2(k2_sor_split<T, ST_P5>, grid, bs, s, Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, cm);
-    else
-      launchk2(k2_sor_split<T, -1>, grid, bs, s, Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, cm);
-  } else {
-    launchk2(k2_sor<T>, grid2(items), kThreads, s, Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, cm);
-  }
+  // three lanes per cell; one warp per block on small passes so that the
+  // block scheduler spreads the warps over the SMs
+  const long warps = (items + 9) / 10;
+  const int bs = warps <= 4L * kSmCount ? 32 : 128;
+  const unsigned grid = (unsigned)((warps * 32 + bs - 1) / bs);
+  if (st == ST_J9)
+    launchk2(k2_sor_split<T, ST_J9>, grid, bs, s, Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, cm);
+  else if (st == ST_P5)
+    launchk2(k2_sor_split<T, ST_P5>, grid, bs, s, Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, cm);
+  else
+    launchk2(k2_sor_split<T, -1>, grid, bs, s, Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, cm);
   return cudaGetLastError();
 }
 
@@ -876,9 +891,23 @@ cudaError_t launch2_prolong(int Nx, int Ny, T *dU, const T *dUc, cudaStream_t s)
   return cudaGetLastError();
 }
 
+// Shared memory of the factorisation of an N3 x N3 system (0: too large for it).
+template <typename T>
+size_t lu2_smem(int N3) {
+  const size_t b = sizeof(T) * (size_t)N3 * (N3 + 1);
+  return b <= (size_t)kTile2MaxSmem && N3 <= kLu2Threads ? b : 0;  // (at most 32 rows per warp)
+}
+
 template <typename T>
 cudaError_t launch2_dense_factor(int Nx, int Ny, int st, const T *J, T *A, int *piv, int *flag, cudaStream_t s) {
+  static std::atomic<unsigned> raised{0};
   const long N3 = 3L * Nx * Ny;
+  if (const size_t smem = lu2_smem<T>((int)N3)) {
+    const cudaError_t e = raise_smem(raised, k2_lu_smem<T>);
+    if (e != cudaSuccess) return e;
+    launchk2s(k2_lu_smem<T>, 1, lu2_threads((int)N3), smem, s, Nx, Ny, st, J, A, piv, flag);
+    return cudaGetLastError();
+  }
   launchk2(k2_zero<T>, grid2(N3 * N3), kThreads, s, N3 * N3, A);
   launchk2(k2_scatter<T>, grid2((long)Nx * Ny * (st == ST_J21 ? 21 : 9)), kThreads, s, Nx, Ny, st, J, A);
   launchk2(k2_lu<T>, 1, kThreads, s, (int)N3, A, piv, flag);
@@ -886,8 +915,8 @@ cudaError_t launch2_dense_factor(int Nx, int Ny, int st, const T *J, T *A, int *
 }
 
 template <typename T>
-cudaError_t launch2_dense_solve(int n, const T *A, const int *piv, const T *R, T *x, T *dU, cudaStream_t s) {
-  launchk2(k2_lu_solve<T>, 1, 32, s, n, A, piv, R, x, dU);
+cudaError_t launch2_dense_solve(int n, const T *A, const int *piv, const T *R, T *dU, cudaStream_t s) {
+  launchk2s(k2_lu_solve<T>, 1, kThreads, sizeof(T) * 9 * (size_t)n, s, n, A, piv, R, dU);
   return cudaGetLastError();
 }
 
@@ -898,9 +927,86 @@ cudaError_t launch2_update(int n, double *U, const T *dU, double tau, int *flag,
 }
 
 template <typename T>
-cudaError_t launch2_vcycle_tail(const Tail2<T> &t, int nu1, int nu2, double omega, int Kc, cudaStream_t s) {
-  launchk2(k2_vcycle_tail<T>, 1, kTail2Threads, s, t, nu1, nu2, omega, Kc);
-  return cudaGetLastError();
+int plan_tail2(Tail2<T> &t, int l0, int cm0, long max_cells, int max_ctas) {
+  const size_t cap = kTile2MaxSmem / sizeof(T);
+  const int N3 = 3 * t.Nx[t.L] * t.Ny[t.L];
+  const size_t xs = 3 * (size_t)N3;
+  t.l0 = l0;
+  t.cm = cm0;
+  t.ls = t.L;
+  for (int m = l0; m < t.L; ++m)
+    if ((long)t.Nx[m] * t.Ny[m] <= max_cells && band2_values(t.Nx[m], t.Ny[m], t.st[m], max_ctas, sizeof(T)) + xs <= cap) {
+      t.ls = m;
+      break;
+    }
+  t.ctas = t.ls < t.L ? (t.Ny[t.ls] / 2 < max_ctas ? t.Ny[t.ls] / 2 : max_ctas) : 1;
+  // The larger levels keep their place for the whole launch as long as the
+  // smaller ones fit beside them; those that do not all fit share one place
+  // and are loaded again for each smoothing.
+  size_t val[NSWE_MAX_LEVELS], rest[NSWE_MAX_LEVELS + 1], most[NSWE_MAX_LEVELS + 1], sum = 0;
+  rest[t.L] = most[t.L] = 0;
+  for (int m = t.L - 1; m >= t.ls; --m) {
+    val[m] = band2_values(t.Nx[m], t.Ny[m], t.st[m], t.ctas, sizeof(T));
+    rest[m] = rest[m + 1] + val[m];
+    most[m] = most[m + 1] > val[m] ? most[m + 1] : val[m];
+  }
+  t.shared_from = t.ls;
+  while (t.shared_from < t.L && sum + rest[t.shared_from] + xs > cap &&
+         sum + val[t.shared_from] + most[t.shared_from + 1] + xs <= cap)
+    sum += val[t.shared_from++];
+  const bool all = sum + rest[t.shared_from] + xs <= cap;
+  size_t at = 0;
+  for (int m = t.ls; m < t.L; ++m) {
+    t.off[m] = (int)at;
+    if (all || m < t.shared_from) at += val[m];
+  }
+  if (!all) at += most[t.shared_from];
+  if (all) t.shared_from = t.L;
+  // a warp per ten cells of the largest colour pass, at least the direct solve's rows
+  int groups = (N3 + 31) / 32;
+  for (int m = t.ls; m < t.L; ++m) {
+    const int pairs = t.Ny[m] / 2, nA = pairs < t.ctas ? pairs : t.ctas, rows = 2 * ((pairs + nA - 1) / nA);
+    const int g = (band2_slots(t.Nx[m], t.st[m], rows) + 9) / 10;
+    groups = g > groups ? g : groups;
+  }
+  t.threads = groups <= 4 ? 128 : groups <= 8 ? 256 : kTail2Threads;
+  t.lu_off = (int)at;
+  t.lu_smem = t.lu_off + (size_t)N3 * (N3 + 1) + xs <= cap;
+  t.smem = sizeof(T) * (t.lu_off + (t.lu_smem ? (size_t)N3 * (N3 + 1) : 0) + xs);
+  return t.ls;
+}
+
+namespace {
+// One cluster of `ctas` CTAs per problem, `count` problems.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_clusters2(std::atomic<unsigned> &raised, void (*kern)(KArgs...), int count, int ctas, int threads,
+                             size_t smem, bool after_factor, cudaStream_t s, Args &&...args) {
+  cudaError_t e = raise_smem(raised, kern, true);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)count * (unsigned)ctas, 1, 1);
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)ctas;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = after_factor ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+}  // namespace
+
+template <typename T>
+cudaError_t launch2_vcycle_tail(const Tail2<T> &t, int nu1, int nu2, double omega, int Kc, int cycles,
+                                bool after_factor, cudaStream_t s) {
+  static std::atomic<unsigned> raised{0};
+  return launch_clusters2(raised, k2_vcycle_tail<T>, 1, t.ctas, t.threads, t.smem, after_factor, s, t, nu1, nu2,
+                          omega, Kc, cycles);
 }
 
 cudaError_t launch2_to_f32(long count, const double *src, float *dst, cudaStream_t s) {
@@ -919,9 +1025,11 @@ cudaError_t launch2_to_f32(long count, const double *src, float *dst, cudaStream
                                            cudaStream_t);                                                        \
   template cudaError_t launch2_prolong<T>(int, int, T *, const T *, cudaStream_t);                               \
   template cudaError_t launch2_dense_factor<T>(int, int, int, const T *, T *, int *, int *, cudaStream_t);       \
-  template cudaError_t launch2_dense_solve<T>(int, const T *, const int *, const T *, T *, T *, cudaStream_t);    \
+  template cudaError_t launch2_dense_solve<T>(int, const T *, const int *, const T *, T *, cudaStream_t);         \
+  template cudaError_t launch2_dinv_levels<T>(Tail2<T>, int, int, cudaStream_t);                                 \
+  template int plan_tail2<T>(Tail2<T> &, int, int, long, int);                                                   \
   template cudaError_t launch2_update<T>(int, double *, const T *, double, int *, cudaStream_t);                 \
-  template cudaError_t launch2_vcycle_tail<T>(const Tail2<T> &, int, int, double, int, cudaStream_t);
+  template cudaError_t launch2_vcycle_tail<T>(const Tail2<T> &, int, int, double, int, int, bool, cudaStream_t);
 NSWE_2D_INSTANTIATE(double)
 NSWE_2D_INSTANTIATE(float)
 #undef NSWE_2D_INSTANTIATE
@@ -1048,10 +1156,18 @@ __global__ void __launch_bounds__(kThreads) kb2_prolong(const BTask2<T> *tasks, 
 template <typename T>
 __global__ void __launch_bounds__(kTail2Threads, 1) kb2_vcycle_tail(const Tail2<T> *tails, const BTask2<T> *tasks,
                                                                    const int *done, int nu1, int nu2, double omega,
-                                                                   int Kc) {
+                                                                   int Kc, int cycles) {
+  const int i = blockIdx.x / cooperative_groups::this_cluster().num_blocks();
+  if (done && done[tasks[i].prob]) return;  // the whole cluster
+  vcycle_cluster2<T>(tails[i], nu1, nu2, omega, Kc, cycles);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kLu2Threads, 1) kb2_lu_smem(const BTask2<T> *tasks, const int *done, int *flags) {
   pdl_enter();
-  if (done && done[tasks[blockIdx.x].prob]) return;
-  vcycle_tail_block2<T>(tails[blockIdx.x], nu1, nu2, omega, Kc);
+  const BTask2<T> &t = tasks[blockIdx.x];
+  if (done && done[t.prob]) return;
+  lu_smem_block2<T>(t.Nx, t.Ny, t.st, t.J, t.A, t.piv, flags + t.prob);
 }
 
 template <typename T>
@@ -1081,11 +1197,12 @@ __global__ void __launch_bounds__(kThreads) kb2_lu(const BTask2<T> *tasks, const
 }
 
 template <typename T>
-__global__ void kb2_lu_solve(const BTask2<T> *tasks, const int *done) {
+__global__ void __launch_bounds__(kThreads) kb2_lu_solve(const BTask2<T> *tasks, const int *done) {
   pdl_enter();
   const BTask2<T> &t = tasks[blockIdx.x];
-  if ((done && done[t.prob]) || threadIdx.x >= 32) return;
-  lu_solve_warp<T>(t.Nx * t.Ny, t.A, t.piv, t.R, t.x, t.dU);
+  if (done && done[t.prob]) return;
+  const int n = t.Nx * t.Ny;
+  lu_solve_block<T>(n, t.A, 3 * n, 1, t.piv, t.R, reinterpret_cast<T *>(g_lus2_smem), t.dU);
 }
 
 template <typename T>
@@ -1151,9 +1268,9 @@ template <typename T>
 cudaError_t launchb2_sor(const Batch2Launch<T> &b, const int *done, int st, double omega, int mode, int Kc, int col,
                          int reps, cudaStream_t s) {
   if (b.ntask == 0) return cudaSuccess;
-  if (NSWE_SOR_UNROLL && st == ST_J9)
+  if (st == ST_J9)
     launchk2(kb2_sor_split<T, ST_J9>, b.blocks, kB2SorThreads, s, b.tasks, b.ntask, done, st, omega, mode, Kc, col, reps);
-  else if (NSWE_SOR_UNROLL && st == ST_P5)
+  else if (st == ST_P5)
     launchk2(kb2_sor_split<T, ST_P5>, b.blocks, kB2SorThreads, s, b.tasks, b.ntask, done, st, omega, mode, Kc, col, reps);
   else
     launchk2(kb2_sor_split<T, -1>, b.blocks, kB2SorThreads, s, b.tasks, b.ntask, done, st, omega, mode, Kc, col, reps);
@@ -1175,17 +1292,26 @@ cudaError_t launchb2_prolong(const Batch2Launch<T> &b, const int *done, cudaStre
 }
 
 template <typename T>
-cudaError_t launchb2_vcycle_tail(const Tail2<T> *tails, const BTask2<T> *tasks, int ntask, const int *done, int nu1,
-                                 int nu2, double omega, int Kc, cudaStream_t s) {
+cudaError_t launchb2_vcycle_tail(const Tail2<T> *tails, const BTask2<T> *tasks, int ntask, int ctas, int threads,
+                                 size_t smem, const int *done, int nu1, int nu2, double omega, int Kc, int cycles,
+                                 bool after_factor, cudaStream_t s) {
   if (ntask == 0) return cudaSuccess;
-  launchk2(kb2_vcycle_tail<T>, ntask, kTail2Threads, s, tails, tasks, done, nu1, nu2, omega, Kc);
-  return cudaGetLastError();
+  static std::atomic<unsigned> raised{0};
+  return launch_clusters2(raised, kb2_vcycle_tail<T>, ntask, ctas, threads, smem, after_factor, s, tails, tasks, done,
+                          nu1, nu2, omega, Kc, cycles);
 }
 
 template <typename T>
 cudaError_t launchb2_dense_factor(const Batch2Launch<T> &zero, const Batch2Launch<T> &scatter, const BTask2<T> *tasks,
-                                  int ntask, const int *done, int *flags, cudaStream_t s) {
+                                  int ntask, int max_cells, const int *done, int *flags, cudaStream_t s) {
   if (ntask == 0) return cudaSuccess;
+  static std::atomic<unsigned> raised{0};
+  if (const size_t smem = lu2_smem<T>(3 * max_cells)) {
+    const cudaError_t e = raise_smem(raised, kb2_lu_smem<T>);
+    if (e != cudaSuccess) return e;
+    launchk2s(kb2_lu_smem<T>, ntask, lu2_threads(3 * max_cells), smem, s, tasks, done, flags);
+    return cudaGetLastError();
+  }
   launchk2(kb2_dense_zero<T>, zero.blocks, kThreads, s, zero.tasks, zero.ntask, done);
   launchk2(kb2_scatter<T>, scatter.blocks, kThreads, s, scatter.tasks, scatter.ntask, done);
   launchk2(kb2_lu<T>, ntask, kThreads, s, tasks, done, flags);
@@ -1193,9 +1319,9 @@ cudaError_t launchb2_dense_factor(const Batch2Launch<T> &zero, const Batch2Launc
 }
 
 template <typename T>
-cudaError_t launchb2_dense_solve(const BTask2<T> *tasks, int ntask, const int *done, cudaStream_t s) {
+cudaError_t launchb2_dense_solve(const BTask2<T> *tasks, int ntask, int max_cells, const int *done, cudaStream_t s) {
   if (ntask == 0) return cudaSuccess;
-  launchk2(kb2_lu_solve<T>, ntask, 32, s, tasks, done);
+  launchk2s(kb2_lu_solve<T>, ntask, kThreads, sizeof(T) * 9 * (size_t)max_cells, s, tasks, done);
   return cudaGetLastError();
 }
 
@@ -1215,11 +1341,11 @@ cudaError_t launchb2_update(const Batch2Launch<T> &b, const int *done, int *flag
                                        cudaStream_t);                                                             \
   template cudaError_t launchb2_restrict<T>(const Batch2Launch<T> &, const int *, cudaStream_t);                  \
   template cudaError_t launchb2_prolong<T>(const Batch2Launch<T> &, const int *, cudaStream_t);                   \
-  template cudaError_t launchb2_vcycle_tail<T>(const Tail2<T> *, const BTask2<T> *, int, const int *, int, int,   \
-                                               double, int, cudaStream_t);                                        \
+  template cudaError_t launchb2_vcycle_tail<T>(const Tail2<T> *, const BTask2<T> *, int, int, int, size_t,         \
+                                               const int *, int, int, double, int, int, bool, cudaStream_t);      \
   template cudaError_t launchb2_dense_factor<T>(const Batch2Launch<T> &, const Batch2Launch<T> &,                 \
-                                                const BTask2<T> *, int, const int *, int *, cudaStream_t);        \
-  template cudaError_t launchb2_dense_solve<T>(const BTask2<T> *, int, const int *, cudaStream_t);                \
+                                                const BTask2<T> *, int, int, const int *, int *, cudaStream_t);   \
+  template cudaError_t launchb2_dense_solve<T>(const BTask2<T> *, int, int, const int *, cudaStream_t);           \
   template cudaError_t launchb2_update<T>(const Batch2Launch<T> &, const int *, int *, cudaStream_t);
 NSWE_B2_INSTANTIATE(double)
 NSWE_B2_INSTANTIATE(float)
