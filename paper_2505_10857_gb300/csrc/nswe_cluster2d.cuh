@@ -17,9 +17,9 @@
 // A pass is bound by the FP64 unit in FP64 (30 instructions of 64 cycles per
 // warp and round of cells at J9) and by the latency of one warp's loads in
 // FP32. V-cycles with nu = 20, GB300, before (a launch per pass, the last
-// levels on one block) and after: FP64 32 x 16 3.11 -> 0.85 ms, 64 x 32 3.75 ->
+// levels on one block) and after: FP64 32 x 16 3.11 -> 0.86 ms, 64 x 32 3.75 ->
 // 1.11; FP32 32 x 16 1.64 -> 0.40, 64 x 32 3.18 -> 0.56, 128 x 64 3.15 -> 1.01;
-// J21 at 64 x 32 15.8 -> 6.0 and 36.0 -> 2.1.
+// J21 at 64 x 32 FP64 15.8 -> 6.0, FP32 36.0 -> 2.1.
 #pragma once
 
 #include <cooperative_groups.h>

@@ -977,7 +977,10 @@ int plan_tail2(Tail2<T> &t, int l0, int cm0, long max_cells, int max_ctas) {
 }
 
 namespace {
-// One cluster of `ctas` CTAs per problem, `count` problems.
+// One cluster of `ctas` CTAs per problem, `count` problems. Behind the coarsest
+// factorisation, and with the overlap switch on, the cluster begins its way
+// down while the factorisation runs and waits for it before the direct solve;
+// into a capture too, where this is one edge per V-cycle.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_clusters2(std::atomic<unsigned> &raised, void (*kern)(KArgs...), int count, int ctas, int threads,
                              size_t smem, bool after_factor, cudaStream_t s, Args &&...args) {
@@ -996,7 +999,7 @@ cudaError_t launch_clusters2(std::atomic<unsigned> &raised, void (*kern)(KArgs..
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = after_factor ? 2 : 1;
+  cfg.numAttrs = after_factor && g_pdl2.load(std::memory_order_relaxed) ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 }  // namespace

@@ -23,7 +23,7 @@ def nswe():
     return N
 
 
-@pytest.mark.parametrize("grid", [(8, 8, 2), (12, 40, 3), (20, 24, 3), (10, 36, 2), (88, 48, 4)])
+@pytest.mark.parametrize("grid", [(8, 8, 2), (16, 40, 3), (20, 24, 3), (10, 36, 2), (88, 48, 4)])
 @pytest.mark.parametrize("nb,colours", [(9, 0), (9, 4), (21, 0)])
 def test_vcycles_match_the_oracle_on_and_off_the_cluster(nswe, grid, nb, colours):
     Nx, Ny, levels = grid
