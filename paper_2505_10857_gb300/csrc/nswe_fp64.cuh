@@ -57,8 +57,20 @@ __device__ __forceinline__ double fast_div(double a, double b, double rb) {
   return fma(fma(-b, q, a), rb, q);
 }
 
+// x^(-1/2): e = 1 - x y^2, y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + ...), cut
+// after e^2: relative error before the last rounding below 2^-54.
+__device__ __forceinline__ double fast_rsqrt(double x) {
+  if ((unsigned)(__double2hiint(x) >> 20) - 2u > 2040u) return rsqrt(x);  // negative, zero, subnormal, huge, NaN
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
 // fast_* for FP64 arguments, the plain operation in FP32.
 __device__ __forceinline__ double rcp_t(double x) { return fast_rcp(x); }
 __device__ __forceinline__ float rcp_t(float x) { return 1.0f / x; }
+__device__ __forceinline__ double rsqrt_t(double x) { return fast_rsqrt(x); }
+__device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
 
 }  // namespace nswe

@@ -14,6 +14,7 @@
 #include <cmath>
 #include <type_traits>
 
+#include "nswe_fp64.cuh"
 #include "nswe_internal.h"
 
 namespace nswe {
@@ -94,52 +95,68 @@ __device__ __forceinline__ void ghost(int kind, double bh, double bq, double sb,
 
 // WENO3 in one cell from averages a, b, c (cells k-1, k, k+1), Eq. 7-8 with
 // the linear weights (1/3, 2/3) for U^+_{k-1/2} and (2/3, 1/3) for
-// U^-_{k+1/2}. With s_r = (zeta + beta_r)^2 the normalised weights are
-// w0 = s1/(s1 + 2 s0), w1 = 2 s0/(s1 + 2 s0) and v0 = 2 s1/(2 s1 + s0),
-// v1 = s0/(2 s1 + s0); both quotients share one reciprocal.
+// U^-_{k+1/2}. With the differences d0 = c - b, d1 = b - a and
+// s_r = (zeta + beta_r)^2, beta_r = d_r^2, the weighted means are
+//   U^+_{k-1/2} = b - (s1 d0 + 2 s0 d1) / (2 (s1 + 2 s0)),
+//   U^-_{k+1/2} = b + (2 s1 d0 + s0 d1) / (2 (2 s1 + s0));
+// both quotients share one reciprocal. The FP64 pipe bounds every kernel
+// that calls this (64 cycles per warp instruction): 21 instruction slots
+// instead of the 33 of the candidate polynomials, and a small correction is
+// rounded instead of the value itself.
 template <typename T>
-__device__ __forceinline__ void weno3(T a, T b, T c, T &up, T &um) {
-  T d0 = c - b, d1 = b - a;
-  T e0 = T(kZeta) + d0 * d0, e1 = T(kZeta) + d1 * d1;
-  T s0 = e0 * e0, s1 = e1 * e1;
-  T p0 = T(1.5) * b - T(0.5) * c, p1 = T(0.5) * a + T(0.5) * b;   // U^(0), U^(1) at k-1/2
-  T q0 = T(0.5) * b + T(0.5) * c, q1 = T(-0.5) * a + T(1.5) * b;  // U^(0), U^(1) at k+1/2
-  T D1 = s1 + T(2.0) * s0, D2 = T(2.0) * s1 + s0;
-  T inv = T(1.0) / (D1 * D2);
-  up = (s1 * p0 + T(2.0) * s0 * p1) * (D2 * inv);
-  um = (T(2.0) * s1 * q0 + s0 * q1) * (D1 * inv);
-}
-
-__device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
-__device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
-
-// Quantities of one interface state entering the HLL flux at a face of width
-// sigma: velocity u = Q/H, celerity c = sqrt(g H/sigma) and physical flux
-// F = (Q, Q^2/H + g H^2/(2 sigma)) (Eq. 4). One reciprocal square root
-// r = H^(-1/2) gives both 1/H = r^2 and c = sqrt(g/sigma) H r; isg = 1/sigma
-// and cg = sqrt(g/sigma) are per-face geometry. r2 = 1/H and the pressure
-// term P = g H^2/(2 sigma) are kept, so that a state differing only in Q
-// (fstate_q) costs one multiply and one fused multiply-add, with the same
-// bits as a full evaluation.
-template <typename T>
-struct FState {
-  T H, Q, u, c, F1, r2, P;
+struct Slope {
+  T d, s;  // difference and (zeta + d^2)^2
 };
 
 template <typename T>
-__device__ __forceinline__ FState<T> fstate(T H, T Q, T isg, T cg, T g) {
-  FState<T> s;
-  s.H = H;
-  s.Q = Q;
-  const T r = rsq(H);
-  s.r2 = r * r;
-  s.u = Q * s.r2;
-  const T h = H * isg;
-  s.c = cg * (H * r);
-  s.P = (T(0.5) * g * H) * h;
-  s.F1 = fma(Q, s.u, s.P);
-  return s;
+__device__ __forceinline__ Slope<T> slope(T d) {
+  const T e = fma(d, d, T(kZeta));
+  return {d, e * e};
 }
+
+template <typename T>
+__device__ __forceinline__ void weno3(T b, const Slope<T> &S0, const Slope<T> &S1, T &up, T &um) {
+  const T x = S1.s * S0.d, y = S0.s * S1.d;
+  const T D1 = fma(T(2.0), S0.s, S1.s), D2 = fma(T(2.0), S1.s, S0.s);
+  const T hinv = T(0.5) * rcp_t(D1 * D2);
+  up = fma(-fma(T(2.0), y, x), D2 * hinv, b);
+  um = fma(fma(T(2.0), x, y), D1 * hinv, b);
+}
+
+template <typename T>
+__device__ __forceinline__ void weno3(T a, T b, T c, T &up, T &um) {
+  weno3<T>(b, slope<T>(c - b), slope<T>(b - a), up, um);
+}
+
+// FP32: the candidate polynomials with the normalised weights w0 = s1/(s1 +
+// 2 s0), v0 = 2 s1/(2 s1 + s0). The FP32 pipe bounds no kernel here, and the
+// difference quotients of the FP32 Jacobian show every rounding (2e-5 of its
+// largest block), so its passes keep their sequence of operations.
+template <>
+__device__ __forceinline__ void weno3<float>(float a, float b, float c, float &up, float &um) {
+  float d0 = c - b, d1 = b - a;
+  float e0 = float(kZeta) + d0 * d0, e1 = float(kZeta) + d1 * d1;
+  float s0 = e0 * e0, s1 = e1 * e1;
+  float p0 = 1.5f * b - 0.5f * c, p1 = 0.5f * a + 0.5f * b;   // U^(0), U^(1) at k-1/2
+  float q0 = 0.5f * b + 0.5f * c, q1 = -0.5f * a + 1.5f * b;  // U^(0), U^(1) at k+1/2
+  float D1 = s1 + 2.0f * s0, D2 = 2.0f * s1 + s0;
+  float inv = 1.0f / (D1 * D2);
+  up = (s1 * p0 + 2.0f * s0 * p1) * (D2 * inv);
+  um = (2.0f * s1 * q0 + s0 * q1) * (D1 * inv);
+}
+
+// Quantities of one interface state entering the flux at a face of width
+// sigma: velocity u = Q/H, the wave speeds lo = u - c and hi = u + c with the
+// celerity c = sqrt(g H/sigma), and the physical flux F = (Q, Q^2/H +
+// g H^2/(2 sigma)) (Eq. 4). One reciprocal square root r = H^(-1/2) gives
+// both 1/H = r^2 and c = sqrt(g/sigma) H r; cg = sqrt(g/sigma), isg = 1/sigma
+// and hg = g/(2 sigma) are per-face values. r2 = 1/H, c and the pressure term P =
+// g H^2/(2 sigma) are kept, so that a state differing only in Q (fstate_q)
+// costs four instructions, with the same bits as a full evaluation.
+template <typename T>
+struct FState {
+  T H, Q, u, c, lo, hi, F1, r2, P;
+};
 
 // The state of `b` with its discharge replaced by Q.
 template <typename T>
@@ -147,8 +164,32 @@ __device__ __forceinline__ FState<T> fstate_q(const FState<T> &b, T Q) {
   FState<T> s = b;
   s.Q = Q;
   s.u = Q * b.r2;
+  s.lo = s.u - b.c;
+  s.hi = s.u + b.c;
   s.F1 = fma(Q, s.u, b.P);
   return s;
+}
+
+template <typename T>
+struct Face {
+  T isg, cg, g, hg;
+};
+
+template <typename T>
+__device__ __forceinline__ Face<T> face(T isg, T cg, T g) {
+  return {isg, cg, g, T(0.5) * g * isg};
+}
+
+template <typename T>
+__device__ __forceinline__ FState<T> fstate(T H, T Q, const Face<T> &f) {
+  FState<T> s;
+  s.H = H;
+  const T r = rsqrt_t(H);
+  s.r2 = r * r;
+  s.c = f.cg * (H * r);
+  if constexpr (std::is_same<T, float>::value) s.P = (0.5f * f.g * H) * (H * f.isg);  // as weno3<float>
+  else s.P = (f.hg * H) * H;
+  return fstate_q(s, Q);
 }
 
 // Ordering keys of FP64 values on the integer pipe (the FP64 pipe is the
@@ -170,11 +211,12 @@ __device__ __forceinline__ bool knonpos(float a) { return a <= 0.0f; }
 
 // HLL flux of two interface states: S_L = min(u_L - c_L, u_R - c_R),
 // S_R = max(u_L + c_L, u_R + c_R), upwind fluxes outside the fan, the HLL
-// average inside.
+// average inside, written as the left flux and a correction: with
+// w = -S_L / (S_R - S_L), F = F_L + w (F_R - F_L - S_R (U_R - U_L)).
 template <typename T>
 __device__ __forceinline__ void hll_states(const FState<T> &L, const FState<T> &R, T &F0, T &F1) {
-  T SL = kmin(L.u - L.c, R.u - R.c);
-  T SR = kmax(L.u + L.c, R.u + R.c);
+  const T SL = kmin(L.lo, R.lo);
+  const T SR = kmax(L.hi, R.hi);
   if (knonneg(SL)) {
     F0 = L.Q;
     F1 = L.F1;
@@ -182,9 +224,16 @@ __device__ __forceinline__ void hll_states(const FState<T> &L, const FState<T> &
     F0 = R.Q;
     F1 = R.F1;
   } else {
-    T iw = T(1.0) / (SR - SL);
-    F0 = (SR * L.Q - SL * R.Q + SL * SR * (R.H - L.H)) * iw;
-    F1 = (SR * L.F1 - SL * R.F1 + SL * SR * (R.Q - L.Q)) * iw;
+    if constexpr (std::is_same<T, float>::value) {  // as weno3<float>
+      const T iw = 1.0f / (SR - SL);
+      F0 = (SR * L.Q - SL * R.Q + SL * SR * (R.H - L.H)) * iw;
+      F1 = (SR * L.F1 - SL * R.F1 + SL * SR * (R.Q - L.Q)) * iw;
+      return;
+    }
+    const T w = -SL * rcp_t(SR - SL);
+    const T dQ = R.Q - L.Q;
+    F0 = fma(w, fma(-SR, R.H - L.H, dQ), L.Q);
+    F1 = fma(w, fma(-SR, dQ, R.F1 - L.F1), L.F1);
   }
 }
 
@@ -278,22 +327,69 @@ template <> struct GeoT<float> {
 
 // Two-point Gauss source of cell j (Eq. 9): S = (dx/2) sum_q [g h^2 sigma_x/2
 // - g sigma h b_x] at the Gauss points, h = H_h/sigma, H_h the cubic through
-// the interface values p0..p3 of H at t = -3/2, -1/2, 1/2, 3/2.
-// With H_h = sigma h the second term is g H_h b_x; 1/sigma is per-cell
-// geometry.
+// the interface values p0..p3 of H at t = -3/2, -1/2, 1/2, 3/2. With
+// H_h = sigma h this is sum_q H_h (A_q H_h - B_q), A_q = dx g sigma_x /
+// (4 sigma^2) and B_q = dx g b_x / 2 of the cell (1/sigma is per-cell
+// geometry), which a Jacobian pass forms once for its perturbed sources.
 template <typename T>
-__device__ __forceinline__ T source_at(const Geo &G, int j, T p0, T p1, T p2, T p3) {
-  T S = T(0.0);
-  const T g = GeoT<T>::g(G);
+struct SrcCell {
+  T A[2], B[2];
+};
+
+template <typename T>
+__device__ __forceinline__ SrcCell<T> src_cell(const Geo &G, int j) {
+  SrcCell<T> c;
+  const T gd = GeoT<T>::g(G) * GeoT<T>::hdx(G);
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
-    T Hh = T(kLag[q][0]) * p0 + T(kLag[q][1]) * p1 + T(kLag[q][2]) * p2 + T(kLag[q][3]) * p3;
-    T sigx = GeoT<T>::sigx(G, q * G.N + j);
-    T bx = GeoT<T>::bx(G, q * G.N + j);
-    T h = Hh * GeoT<T>::igq(G, q * G.N + j);
-    S += T(0.5) * g * h * h * sigx - g * Hh * bx;
+    const T is = GeoT<T>::igq(G, q * G.N + j);
+    c.A[q] = (T(0.5) * gd) * GeoT<T>::sigx(G, q * G.N + j) * (is * is);
+    c.B[q] = gd * GeoT<T>::bx(G, q * G.N + j);
   }
-  return S * GeoT<T>::hdx(G);
+  return c;
+}
+
+// FP32: the terms as they stand in Eq. 9 (as weno3<float>).
+template <>
+struct SrcCell<float> {
+  float is[2], sigx[2], bx[2], g, hdx;
+};
+
+template <>
+__device__ __forceinline__ SrcCell<float> src_cell<float>(const Geo &G, int j) {
+  SrcCell<float> c;
+  c.g = GeoT<float>::g(G);
+  c.hdx = GeoT<float>::hdx(G);
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    c.is[q] = GeoT<float>::igq(G, q * G.N + j);
+    c.sigx[q] = GeoT<float>::sigx(G, q * G.N + j);
+    c.bx[q] = GeoT<float>::bx(G, q * G.N + j);
+  }
+  return c;
+}
+
+__device__ __forceinline__ float source_at(const SrcCell<float> &c, float p0, float p1, float p2, float p3) {
+  float S = 0.0f;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    float Hh = float(kLag[q][0]) * p0 + float(kLag[q][1]) * p1 + float(kLag[q][2]) * p2 + float(kLag[q][3]) * p3;
+    float h = Hh * c.is[q];
+    S += 0.5f * c.g * h * h * c.sigx[q] - c.g * Hh * c.bx[q];
+  }
+  return S * c.hdx;
+}
+
+template <typename T>
+__device__ __forceinline__ T source_at(const SrcCell<T> &c, T p0, T p1, T p2, T p3) {
+  T S[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const T Hh = fma(T(kLag[q][3]), p3, fma(T(kLag[q][0]), p0, fma(T(kLag[q][2]), p2, T(kLag[q][1]) * p1)));
+    const T t = fma(c.A[q], Hh, -c.B[q]);
+    S[q] = q == 0 ? Hh * t : fma(Hh, t, S[0]);
+  }
+  return S[1];
 }
 
 // Local residual R_j (Eq. 10) from a filled window.
@@ -305,11 +401,10 @@ __device__ __forceinline__ void local_residual(const Geo &G, int j, const Win &w
     weno3(w.Q[p], w.Q[p + 1], w.Q[p + 2], upQ[p], umQ[p]);
   }
   double Fr0, Fr1, Fl0, Fl1;
-  num_flux<-1>(fstate(umH[1], umQ[1], G.isf[j + 1], G.cgf[j + 1], G.g),
-               fstate(upH[2], upQ[2], G.isf[j + 1], G.cgf[j + 1], G.g), G.flux, Fr0, Fr1);
-  num_flux<-1>(fstate(umH[0], umQ[0], G.isf[j], G.cgf[j], G.g), fstate(upH[1], upQ[1], G.isf[j], G.cgf[j], G.g),
-               G.flux, Fl0, Fl1);
-  double S = source_at(G, j, upH[0], upH[1], umH[1], umH[2]);
+  const Face<double> fr = face(G.isf[j + 1], G.cgf[j + 1], G.g), fl = face(G.isf[j], G.cgf[j], G.g);
+  num_flux<-1>(fstate(umH[1], umQ[1], fr), fstate(upH[2], upQ[2], fr), G.flux, Fr0, Fr1);
+  num_flux<-1>(fstate(umH[0], umQ[0], fl), fstate(upH[1], upQ[1], fl), G.flux, Fl0, Fl1);
+  const double S = source_at(src_cell<double>(G, j), upH[0], upH[1], umH[1], umH[2]);
   R0 = Fr0 - Fl0;
   R1 = Fr1 - Fl1 - S;
 }
@@ -466,6 +561,9 @@ __device__ double residual_cells_staged(const Geo &G, const double *U, double *R
 //      on the diagonal.
 // Each perturbed R_j is the same arithmetic on the same values as a full
 // re-evaluation of the local residual, at a fraction of the cost.
+// FP64 issue bounds the passes: about 510 instruction slots per cell for J3
+// (744 with the candidate polynomials, full HLL averages and CUDA's divisions):
+// 2^20 cells 1491 -> 1105 us, the 608-problem solve launch 443 -> 354 ms.
 
 template <typename T>
 struct JW {
@@ -508,23 +606,69 @@ __device__ __forceinline__ T pval(const Geo &G, const double *U, int m, int kk, 
   return T(m == 0 ? Hg : Qg);
 }
 
-// Pass A. Variant v = 0: base; v = 1, 2, 3: cell k + v - 2 perturbed.
+// Pass A. Variant v = 0: base; v = 1, 2, 3: cell k + v - 2 perturbed. One
+// item forms the four variants of a cell and component: perturbing cell k-1
+// (k+1) leaves the difference d0 (d1) and its smoothness term. Next to the
+// boundary the ghost cells follow the perturbed edge cell; the differences
+// kept are zero there (two ghost cells are equal), as in the base state.
 template <typename T>
 __device__ void jac_pass_a(const Geo &G, const double *U, double eps, const JW<T> &W, int first, int stride) {
-  const int N = G.N, items = (N + 2) * 8;
+  const int N = G.N, items = (N + 2) * 2;
   const T eps_t = T(eps);
   for (int it = first; it < items; it += stride) {
-    const int k = it % (N + 2) - 1, mv = it / (N + 2), m = mv >> 2, v = mv & 3;
-    int ip = -1;
-    if (v > 0) {
-      ip = k + v - 2;
-      if (ip < 0 || ip >= N) continue;
+    const int m = it >= N + 2, k = it - m * (N + 2) - 1;
+    T a, b, c, a1, b1, c1, a2, b2, c2, a3, b3, c3;  // window of the base state and what each variant has in its place
+    if (k > 0 && k < N - 1) {
+      a = GeoT<T>::u(G, U, m * N + k - 1);
+      b = b1 = b3 = GeoT<T>::u(G, U, m * N + k);
+      c = GeoT<T>::u(G, U, m * N + k + 1);
+      a2 = a3 = a;
+      c1 = c2 = c;
+      a1 = a + eps_t;
+      b2 = b + eps_t;
+      c3 = c + eps_t;
+    } else {
+      auto at = [&](int kk, int ip) { return pval<T>(G, U, m, kk, ip, eps, eps_t); };
+      a = at(k - 1, -1);
+      b = at(k, -1);
+      c = at(k + 1, -1);
+      a1 = at(k - 1, k - 1);
+      b1 = at(k, k - 1);
+      c1 = at(k + 1, k - 1);
+      a2 = at(k - 1, k);
+      b2 = at(k, k);
+      c2 = at(k + 1, k);
+      a3 = at(k - 1, k + 1);
+      b3 = at(k, k + 1);
+      c3 = at(k + 1, k + 1);
     }
+    // variant v has the difference (and smoothness) at the `kept` side of the base state
+    const Slope<T> S0 = slope<T>(c - b), S1 = slope<T>(b - a);
+    auto rec = [&](T va, T vb, T vc, bool keep0, bool keep1, T &vup, T &vum) {
+      if constexpr (std::is_same<T, float>::value)
+        weno3<float>(va, vb, vc, vup, vum);
+      else
+        weno3<T>(vb, keep0 ? S0 : slope<T>(vc - vb), keep1 ? S1 : slope<T>(vb - va), vup, vum);
+    };
     T up, um;
-    weno3<T>(pval<T>(G, U, m, k - 1, ip, eps, eps_t), pval<T>(G, U, m, k, ip, eps, eps_t),
-             pval<T>(G, U, m, k + 1, ip, eps, eps_t), up, um);
-    W.r(m, v, 0, k) = up;
-    W.r(m, v, 1, k) = um;
+    rec(a, b, c, true, true, up, um);
+    W.r(m, 0, 0, k) = up;
+    W.r(m, 0, 1, k) = um;
+    if (k >= 1) {
+      rec(a1, b1, c1, true, false, up, um);
+      W.r(m, 1, 0, k) = up;
+      W.r(m, 1, 1, k) = um;
+    }
+    if (k >= 0 && k < N) {
+      rec(a2, b2, c2, false, false, up, um);
+      W.r(m, 2, 0, k) = up;
+      W.r(m, 2, 1, k) = um;
+    }
+    if (k < N - 1) {
+      rec(a3, b3, c3, false, true, up, um);
+      W.r(m, 3, 0, k) = up;
+      W.r(m, 3, 1, k) = um;
+    }
   }
 }
 
@@ -544,9 +688,9 @@ __device__ void jac_pass_b(const Geo &G, const JW<T> &W, int first, int stride) 
   const int N = G.N;
   const T g = GeoT<T>::g(G);
   for (int f = first; f <= N; f += stride) {
-    const T isg = GeoT<T>::isf(G, f), cg = GeoT<T>::cgf(G, f);
-    const FState<T> Lb = fstate<T>(W.r(0, 0, 1, f - 1), W.r(1, 0, 1, f - 1), isg, cg, g);
-    const FState<T> Rb = fstate<T>(W.r(0, 0, 0, f), W.r(1, 0, 0, f), isg, cg, g);
+    const Face<T> fc = face<T>(GeoT<T>::isf(G, f), GeoT<T>::cgf(G, f), g);
+    const FState<T> Lb = fstate<T>(W.r(0, 0, 1, f - 1), W.r(1, 0, 1, f - 1), fc);
+    const FState<T> Rb = fstate<T>(W.r(0, 0, 0, f), W.r(1, 0, 0, f), fc);
     T F0, F1;
     num_flux<FLUX>(Lb, Rb, G.flux, F0, F1);
     W.f(0, 0, f) = F0;
@@ -561,10 +705,10 @@ __device__ void jac_pass_b(const Geo &G, const JW<T> &W, int first, int stride) 
         // the base state
         FState<T> Ls = Lb, Rs = Rb;
         if (p <= 2)
-          Ls = m == 0 ? fstate<T>(W.r(0, p + 1, 1, f - 1), W.r(1, 0, 1, f - 1), isg, cg, g)
+          Ls = m == 0 ? fstate<T>(W.r(0, p + 1, 1, f - 1), Lb.Q, fc)
                       : fstate_q<T>(Lb, W.r(1, p + 1, 1, f - 1));
         if (p >= 1)
-          Rs = m == 0 ? fstate<T>(W.r(0, p, 0, f), W.r(1, 0, 0, f), isg, cg, g) : fstate_q<T>(Rb, W.r(1, p, 0, f));
+          Rs = m == 0 ? fstate<T>(W.r(0, p, 0, f), Rb.Q, fc) : fstate_q<T>(Rb, W.r(1, p, 0, f));
         num_flux<FLUX>(Ls, Rs, G.flux, F0, F1);
         const int w = 1 + 2 * p + m;
         W.f(w, 0, f) = F0;
@@ -594,7 +738,8 @@ __device__ double jac_pass_c(const Geo &G, int nb, double eps, double alpha, con
   const T ieps = T(1.0) / T(eps);
   double acc = 0.0;
   for (int j = first; j < N; j += stride) {
-    const T Sb = source_at<T>(G, j, W.r(0, 0, 0, j - 1), W.r(0, 0, 0, j), W.r(0, 0, 1, j), W.r(0, 0, 1, j + 1));
+    const SrcCell<T> sc = src_cell<T>(G, j);
+    const T Sb = source_at(sc, W.r(0, 0, 0, j - 1), W.r(0, 0, 0, j), W.r(0, 0, 1, j), W.r(0, 0, 1, j + 1));
     const T R0 = W.f(0, 0, j + 1) - W.f(0, 0, j);
     const T R1 = W.f(0, 1, j + 1) - W.f(0, 1, j) - Sb;
     if (Rout) {
@@ -615,7 +760,7 @@ __device__ double jac_pass_c(const Geo &G, int nb, double eps, double alpha, con
         T S = Sb;
         if (m == 0) {
           const int v0 = rec_variant(i, j - 1), v1 = rec_variant(i, j), v2 = rec_variant(i, j + 1);
-          S = source_at<T>(G, j, W.r(0, v0, 0, j - 1), W.r(0, v1, 0, j), W.r(0, v1, 1, j), W.r(0, v2, 1, j + 1));
+          S = source_at(sc, W.r(0, v0, 0, j - 1), W.r(0, v1, 0, j), W.r(0, v1, 1, j), W.r(0, v2, 1, j + 1));
         }
         const int wr = flux_variant(i, m, j + 1), wl = flux_variant(i, m, j);
         const T P0 = W.f(wr, 0, j + 1) - W.f(wl, 0, j);
@@ -710,8 +855,9 @@ template <int FLUX>
 __device__ void res_pass_b(const Geo &G, const RW &W, int first, int stride) {
   for (int f = first; f <= G.N; f += stride) {
     double F0, F1;
-    num_flux<FLUX>(fstate(W.r(0, 1, f - 1), W.r(1, 1, f - 1), G.isf[f], G.cgf[f], G.g),
-                   fstate(W.r(0, 0, f), W.r(1, 0, f), G.isf[f], G.cgf[f], G.g), G.flux, F0, F1);
+    const Face<double> fc = face(G.isf[f], G.cgf[f], G.g);
+    num_flux<FLUX>(fstate(W.r(0, 1, f - 1), W.r(1, 1, f - 1), fc), fstate(W.r(0, 0, f), W.r(1, 0, f), fc), G.flux, F0,
+                   F1);
     W.f(0, f) = F0;
     W.f(1, f) = F1;
   }
@@ -721,7 +867,7 @@ __device__ double res_pass_c(const Geo &G, const RW &W, double *R, int first, in
   const int N = G.N;
   double acc = 0.0;
   for (int j = first; j < N; j += stride) {
-    const double S = source_at<double>(G, j, W.r(0, 0, j - 1), W.r(0, 0, j), W.r(0, 1, j), W.r(0, 1, j + 1));
+    const double S = source_at<double>(src_cell<double>(G, j), W.r(0, 0, j - 1), W.r(0, 0, j), W.r(0, 1, j), W.r(0, 1, j + 1));
     const double R0 = W.f(0, j + 1) - W.f(0, j);
     const double R1 = W.f(1, j + 1) - W.f(1, j) - S;
     R[j] = R0;
@@ -749,18 +895,19 @@ __device__ void geom_derive_items(const ProbDev &P, int first, int stride) {
   }
 }
 
-// Inverse of the diagonal 2x2 blocks.
+// Inverse of the diagonal 2x2 blocks, times -omega: the factor with which the
+// smoother applies them.
 template <typename T>
-__device__ void dinv_cells(int N, int nb, const T *J, T *Dinv, int first, int stride) {
+__device__ void dinv_cells(int N, int nb, const T *J, T *Dinv, double omega, int first, int stride) {
   const int hw = (nb - 1) / 2;
   for (int j = first; j < N; j += stride) {
     T a = J[(hw * 4 + 0) * N + j], b = J[(hw * 4 + 1) * N + j];
     T c = J[(hw * 4 + 2) * N + j], d = J[(hw * 4 + 3) * N + j];
-    T idet = T(1.0) / (a * d - b * c);
-    Dinv[0 * N + j] = d * idet;
-    Dinv[1 * N + j] = -b * idet;
-    Dinv[2 * N + j] = -c * idet;
-    Dinv[3 * N + j] = a * idet;
+    const T s = T(-omega) * rcp_t(fma(a, d, -(b * c)));
+    Dinv[0 * N + j] = d * s;
+    Dinv[1 * N + j] = -b * s;
+    Dinv[2 * N + j] = -c * s;
+    Dinv[3 * N + j] = a * s;
   }
 }
 
@@ -811,34 +958,39 @@ __device__ void coarse_op_cells(int Nf, int nbf, const T *Jf, int Nc, T *Jc, int
 }
 
 // Block SOR update (Eq. 19) of the cells of one colour (j mod C == col),
-// applied `reps` times in a row. Cells of one colour do not couple, so a
-// repeated visit of the same colour sees the same neighbour values: the
-// correction t is computed once and the relaxation applied reps times, which
-// is exactly the sequence of reps separate passes. The neighbour sum is a
-// chain of fused multiply-adds (two per product pair instead of a multiply,
-// a fused multiply-add and an add).
+// x := (1 - omega) x - omega D^-1 r, applied `reps` times in a row. Cells of
+// one colour do not couple, so a repeated visit of the same colour sees the
+// same neighbour values: the correction t = -omega D^-1 r is computed once
+// and the relaxation applied reps times, which is the sequence of reps
+// separate passes. -omega is in the stored inverse (dinv_cells), so a visit
+// costs 14 FP64 instructions with two neighbours. zero: dU is all zero (the
+// first pass after a restriction), and the neighbour sums are left out.
 template <typename T>
 __device__ void sor_colour(int N, int nb, const T *J, const T *Dinv, const T *R, T *dU, double omega_d, int C,
-                           int col, int reps, int first, int stride) {
-  const T omega = T(omega_d);
+                           int col, int reps, bool zero, int first, int stride) {
+  const T keep = T(1.0) - T(omega_d);
   const int hw = (nb - 1) / 2;
   for (int j = col + C * first; j < N; j += C * stride) {
     T r0 = R[j], r1 = R[N + j];
-    for (int k = 0; k < nb; ++k) {
-      int i = j + k - hw;
-      if (k == hw || i < 0 || i >= N) continue;
-      T x0 = dU[i], x1 = dU[N + i];
-      r0 = fma(J[(k * 4 + 0) * N + j], x0, r0);
-      r0 = fma(J[(k * 4 + 1) * N + j], x1, r0);
-      r1 = fma(J[(k * 4 + 2) * N + j], x0, r1);
-      r1 = fma(J[(k * 4 + 3) * N + j], x1, r1);
+    T x0 = T(0.0), x1 = T(0.0);
+    if (!zero) {
+      for (int k = 0; k < nb; ++k) {
+        int i = j + k - hw;
+        if (k == hw || i < 0 || i >= N) continue;
+        const T y0 = dU[i], y1 = dU[N + i];
+        r0 = fma(J[(k * 4 + 0) * N + j], y0, r0);
+        r0 = fma(J[(k * 4 + 1) * N + j], y1, r0);
+        r1 = fma(J[(k * 4 + 2) * N + j], y0, r1);
+        r1 = fma(J[(k * 4 + 3) * N + j], y1, r1);
+      }
+      x0 = dU[j];
+      x1 = dU[N + j];
     }
-    T t0 = Dinv[0 * N + j] * r0 + Dinv[1 * N + j] * r1;
-    T t1 = Dinv[2 * N + j] * r0 + Dinv[3 * N + j] * r1;
-    T x0 = dU[j], x1 = dU[N + j];
+    const T t0 = fma(Dinv[0 * N + j], r0, Dinv[1 * N + j] * r1);
+    const T t1 = fma(Dinv[2 * N + j], r0, Dinv[3 * N + j] * r1);
     for (int r = 0; r < reps; ++r) {
-      x0 = (T(1.0) - omega) * x0 - omega * t0;
-      x1 = (T(1.0) - omega) * x1 - omega * t1;
+      x0 = fma(keep, x0, t0);
+      x1 = fma(keep, x1, t1);
     }
     dU[j] = x0;
     dU[N + j] = x1;
@@ -983,7 +1135,8 @@ __device__ bool band_lu_warp(const Band<T> &B) {
     // One division for 1/d (lane 0) and the multipliers A(k+i, k)/d (lane i).
     const T d = B.A(k, k);
     const bool mrow = lane >= 1 && lane <= kl && k + lane <= imax;
-    const T q = (lane == 0 ? T(1.0) : (mrow ? B.A(k + lane, k) : T(0.0))) / d;
+    const T rd = rcp_t(d);
+    const T q = lane == 0 ? rd : (mrow ? fast_div(B.A(k + lane, k), d, rd) : T(0.0));
     if (lane == 0) {
       B.rinv[k] = q;
       if (d == T(0.0)) sing = true;
@@ -1265,7 +1418,7 @@ __device__ __forceinline__ int team_split(const MG<T> &mg, int team_cells) {
 // once per Newton step since J is fixed during its V-cycles. Returns whether
 // a pivot was exactly zero, in every thread of the team.
 template <typename T, class TM = BlockTeam>
-__device__ bool mg_setup(const MG<T> &mg, Band<T> &B, const TM &team = TM(), int team_cells = 0) {
+__device__ bool mg_setup(const MG<T> &mg, Band<T> &B, double omega, const TM &team = TM(), int team_cells = 0) {
   const int lt = team_split<T, TM>(mg, team_cells);
   for (int l = mg.l0 + 1; l < lt; ++l) {
     coarse_op_cells(mg.N[l - 1], mg.nb[l - 1], mg.J[l - 1], mg.N[l], mg.J[l], team.tid(), team.size());
@@ -1276,10 +1429,10 @@ __device__ bool mg_setup(const MG<T> &mg, Band<T> &B, const TM &team = TM(), int
       coarse_op_cells(mg.N[l - 1], mg.nb[l - 1], mg.J[l - 1], mg.N[l], mg.J[l], threadIdx.x, blockDim.x);
       __syncthreads();
     }
-  for (int l = mg.l0; l < lt; ++l) dinv_cells(mg.N[l], mg.nb[l], mg.J[l], mg.Dinv[l], team.tid(), team.size());
+  for (int l = mg.l0; l < lt; ++l) dinv_cells(mg.N[l], mg.nb[l], mg.J[l], mg.Dinv[l], omega, team.tid(), team.size());
   bool sing = false;
   if (team.lead()) {
-    for (int l = lt; l < mg.L; ++l) dinv_cells(mg.N[l], mg.nb[l], mg.J[l], mg.Dinv[l], threadIdx.x, blockDim.x);
+    for (int l = lt; l < mg.L; ++l) dinv_cells(mg.N[l], mg.nb[l], mg.J[l], mg.Dinv[l], omega, threadIdx.x, blockDim.x);
     sing = band_factor(B, mg.N[mg.L], mg.nb[mg.L], mg.J[mg.L]);
   }
   if constexpr (TM::kMulti) {
@@ -1290,9 +1443,9 @@ __device__ bool mg_setup(const MG<T> &mg, Band<T> &B, const TM &team = TM(), int
 }
 
 // `steps` symmetric multicolour SOR steps (colours 0..C-1 then C-1..0 each);
-// consecutive visits of one colour run as one pass.
+// consecutive visits of one colour run as one pass. zero: dU is all zero.
 template <typename T, class TM = BlockTeam>
-__device__ void sor_smooth(const MG<T> &mg, int l, int steps, double omega, const TM &team = TM()) {
+__device__ void sor_smooth(const MG<T> &mg, int l, int steps, double omega, bool zero, const TM &team = TM()) {
   const int nb = mg.nb[l], C = (nb - 1) / 2 + 1;
   int prev = -1, reps = 0;
   for (int s = 0; s < steps; ++s)
@@ -1303,35 +1456,38 @@ __device__ void sor_smooth(const MG<T> &mg, int l, int steps, double omega, cons
         continue;
       }
       if (prev >= 0) {
-        sor_colour(mg.N[l], nb, mg.J[l], mg.Dinv[l], mg.R[l], mg.dU[l], omega, C, prev, reps, team.tid(),
+        sor_colour(mg.N[l], nb, mg.J[l], mg.Dinv[l], mg.R[l], mg.dU[l], omega, C, prev, reps, zero, team.tid(),
                    team.size());
         team.sync();
+        zero = false;
       }
       prev = col;
       reps = 1;
     }
   if (prev >= 0) {
-    sor_colour(mg.N[l], nb, mg.J[l], mg.Dinv[l], mg.R[l], mg.dU[l], omega, C, prev, reps, team.tid(), team.size());
+    sor_colour(mg.N[l], nb, mg.J[l], mg.Dinv[l], mg.R[l], mg.dU[l], omega, C, prev, reps, zero, team.tid(),
+               team.size());
     team.sync();
   }
 }
 
-// Algorithm 2 from level l0, unrolled over levels. A cluster team smooths,
+// Algorithm 2 from level l0, unrolled over levels. zero: dU of level l0 is
+// all zero (that of a coarser level always is, by the restriction). A cluster team smooths,
 // restricts and prolongs the levels l0..lt-1; the leader CTA runs the
 // V-cycle below them (levels lt..L) between two cluster barriers.
 template <typename T, class TM = BlockTeam>
-__device__ void mg_vcycle(const MG<T> &mg, const Band<T> &B, const nswe_params &prm, const TM &team = TM(),
-                          int team_cells = 0) {
+__device__ void mg_vcycle(const MG<T> &mg, const Band<T> &B, const nswe_params &prm, bool zero,
+                          const TM &team = TM(), int team_cells = 0) {
   const int lt = team_split<T, TM>(mg, team_cells);
   for (int l = mg.l0; l < lt; ++l) {
-    sor_smooth(mg, l, prm.nu1, prm.omega, team);
+    sor_smooth(mg, l, prm.nu1, prm.omega, zero || l > mg.l0, team);
     restrict_cells(mg.N[l], mg.nb[l], mg.J[l], mg.R[l], mg.dU[l], mg.N[l + 1], mg.R[l + 1], mg.dU[l + 1],
                    team.tid(), team.size());
     team.sync();
   }
   if (team.lead()) {
     for (int l = lt; l < mg.L; ++l) {
-      sor_smooth(mg, l, prm.nu1, prm.omega);
+      sor_smooth(mg, l, prm.nu1, prm.omega, zero || l > mg.l0);
       restrict_cells(mg.N[l], mg.nb[l], mg.J[l], mg.R[l], mg.dU[l], mg.N[l + 1], mg.R[l + 1], mg.dU[l + 1],
                      threadIdx.x, blockDim.x);
       __syncthreads();
@@ -1340,14 +1496,14 @@ __device__ void mg_vcycle(const MG<T> &mg, const Band<T> &B, const nswe_params &
     for (int l = mg.L - 1; l >= lt; --l) {
       prolong_cells(mg.N[l], mg.dU[l], mg.N[l + 1], mg.dU[l + 1], threadIdx.x, blockDim.x);
       __syncthreads();
-      sor_smooth(mg, l, prm.nu2, prm.omega);
+      sor_smooth(mg, l, prm.nu2, prm.omega, false);
     }
   }
   if constexpr (TM::kMulti) team.sync();
   for (int l = lt - 1; l >= mg.l0; --l) {
     prolong_cells(mg.N[l], mg.dU[l], mg.N[l + 1], mg.dU[l + 1], team.tid(), team.size());
     team.sync();
-    sor_smooth(mg, l, prm.nu2, prm.omega, team);
+    sor_smooth(mg, l, prm.nu2, prm.omega, false, team);
   }
 }
 
@@ -1442,9 +1598,9 @@ __global__ void __launch_bounds__(kThreads) k_vcycle(const ProbDev *P, int level
   MG<T> mg;
   mg_bind<T>(mg, *P, level, nb, J, R, dU);
   Band<T> B = band_view<T>(n_cap, ldab_cap);
-  bool sing = mg_setup<T>(mg, B);
+  bool sing = mg_setup<T>(mg, B, prm.omega);
   __syncthreads();
-  mg_vcycle<T>(mg, B, prm);
+  mg_vcycle<T>(mg, B, prm, false);
   if (threadIdx.x == 0) *status = sing ? NSWE_ESINGULAR : NSWE_OK;
 }
 
@@ -1567,7 +1723,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
       }
       MG<T> mg;
       mg_bind<T>(mg, P, l, nb, J, Rs, dU);
-      bool sing = mg_setup<T, TM>(mg, B, team, team_cells);
+      bool sing = mg_setup<T, TM>(mg, B, prm.omega, team, team_cells);
       team.sync();
       if (sing) {
         st = NSWE_ESINGULAR;
@@ -1580,7 +1736,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
         for (int t = team.tid(); t < 2 * N; t += team.size()) dU[t] = T(0.0);
         team.sync();
         for (int m = 0; m < prm.nu3; ++m) {
-          mg_vcycle<T, TM>(mg, B, prm, team, team_cells);
+          mg_vcycle<T, TM>(mg, B, prm, m == 0, team, team_cells);
           ++vcycles;
         }
       }
@@ -1676,7 +1832,7 @@ cudaError_t launch_residual(const ProbDev *p, int level, int N, const double *U,
 
 cudaError_t launch_jacobian(const ProbDev *p, int level, int N, int nb, const double *U, double eps,
                             double alpha, double *R, double *J, double *res, double *partials, cudaStream_t s) {
-  k_jac_a<double><<<grid_for((N + 2) * 8), kThreads, 0, s>>>(p, level, U, eps);
+  k_jac_a<double><<<grid_for((N + 2) * 2), kThreads, 0, s>>>(p, level, U, eps);
   k_jac_b<double><<<grid_for(N + 1), kThreads, 0, s>>>(p, level);
   const int grid = grid_for(N * nb);
   k_jac_c<double><<<grid, kThreads, 0, s>>>(p, level, nb, eps, alpha, nullptr, R, J, partials);
@@ -1690,7 +1846,7 @@ cudaError_t launch_jacobian_f32(const ProbDev *p, int level, int N, int nb, cons
   // the FP32 pass C reuses it (it writes zeros there).
   cudaError_t e = launch_residual(p, level, N, U, R, res, partials, s);
   if (e != cudaSuccess) return e;
-  k_jac_a<float><<<grid_for((N + 2) * 8), kThreads, 0, s>>>(p, level, U, eps);
+  k_jac_a<float><<<grid_for((N + 2) * 2), kThreads, 0, s>>>(p, level, U, eps);
   k_jac_b<float><<<grid_for(N + 1), kThreads, 0, s>>>(p, level);
   k_jac_c<float><<<grid_for(N * nb), kThreads, 0, s>>>(p, level, nb, eps, alpha, R, nullptr, J, partials);
   return cudaGetLastError();
