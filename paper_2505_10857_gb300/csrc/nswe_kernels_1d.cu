@@ -252,49 +252,6 @@ __device__ __forceinline__ void num_flux(const FState<T> &L, const FState<T> &R,
   }
 }
 
-// Five-cell window j-2..j+2 of one residual evaluation.
-struct Win {
-  double H[5], Q[5];
-};
-
-__device__ __forceinline__ void load_win(const Geo &G, const double *H, const double *Q, int j, Win &w) {
-#pragma unroll
-  for (int p = 0; p < 5; ++p) {
-    int k = min(max(j - 2 + p, 0), G.N - 1);  // clamped: ghosts are filled later
-    w.H[p] = H[k];
-    w.Q[p] = Q[k];
-  }
-}
-
-// Ghost positions of the window take the boundary state built from the
-// window's (possibly perturbed) edge cell.
-__device__ __forceinline__ void fill_ghosts(const Geo &G, int j, Win &w) {
-  if (j < 2) {
-    double He = (j == 0) ? w.H[2] : w.H[1];
-    double Qe = (j == 0) ? w.Q[2] : w.Q[1];
-    double Hg, Qg;
-    ghost(G.bl, G.blh, G.blq, G.sf[0], He, Qe, Hg, Qg);
-#pragma unroll
-    for (int p = 0; p < 2; ++p)
-      if (j - 2 + p < 0) {
-        w.H[p] = Hg;
-        w.Q[p] = Qg;
-      }
-  }
-  if (j > G.N - 3) {
-    double He = (j == G.N - 1) ? w.H[2] : w.H[3];
-    double Qe = (j == G.N - 1) ? w.Q[2] : w.Q[3];
-    double Hg, Qg;
-    ghost(G.br, G.brh, G.brq, G.sf[G.N], He, Qe, Hg, Qg);
-#pragma unroll
-    for (int p = 3; p < 5; ++p)
-      if (j - 2 + p >= G.N) {
-        w.H[p] = Hg;
-        w.Q[p] = Qg;
-      }
-  }
-}
-
 // Level data in the precision T of a pass: FP64 values as stored; FP32
 // values from the copies when the level has them, else converted at use.
 template <typename T> struct GeoT;
@@ -392,23 +349,6 @@ __device__ __forceinline__ T source_at(const SrcCell<T> &c, T p0, T p1, T p2, T 
   return S[1];
 }
 
-// Local residual R_j (Eq. 10) from a filled window.
-__device__ __forceinline__ void local_residual(const Geo &G, int j, const Win &w, double &R0, double &R1) {
-  double upH[3], umH[3], upQ[3], umQ[3];
-#pragma unroll
-  for (int p = 0; p < 3; ++p) {
-    weno3(w.H[p], w.H[p + 1], w.H[p + 2], upH[p], umH[p]);
-    weno3(w.Q[p], w.Q[p + 1], w.Q[p + 2], upQ[p], umQ[p]);
-  }
-  double Fr0, Fr1, Fl0, Fl1;
-  const Face<double> fr = face(G.isf[j + 1], G.cgf[j + 1], G.g), fl = face(G.isf[j], G.cgf[j], G.g);
-  num_flux<-1>(fstate(umH[1], umQ[1], fr), fstate(upH[2], upQ[2], fr), G.flux, Fr0, Fr1);
-  num_flux<-1>(fstate(umH[0], umQ[0], fl), fstate(upH[1], upQ[1], fl), G.flux, Fl0, Fl1);
-  const double S = source_at(src_cell<double>(G, j), upH[0], upH[1], umH[1], umH[2]);
-  R0 = Fr0 - Fl0;
-  R1 = Fr1 - Fl1 - S;
-}
-
 // ----------------------------------------------------------------------------
 // Block-level helpers.
 
@@ -490,61 +430,6 @@ struct ClusterTeam {
     return v;
   }
 };
-
-// Residual of cells [first, N) with stride; returns sum_j ||R_j||_1.
-__device__ double residual_cells(const Geo &G, const double *U, double *R, int first, int stride) {
-  const double *H = U, *Q = U + G.N;
-  double acc = 0.0;
-  for (int j = first; j < G.N; j += stride) {
-    Win w;
-    load_win(G, H, Q, j, w);
-    fill_ghosts(G, j, w);
-    double R0, R1;
-    local_residual(G, j, w, R0, R1);
-    R[j] = R0;
-    R[G.N + j] = R1;
-    acc += fabs(R0) + fabs(R1);
-  }
-  return acc;
-}
-
-// The same residual with each block's five-cell windows staged in shared
-// memory: the block reads cells t0-2 .. t0+B+1 of a tile of B = blockDim.x
-// cells once, coalesced, and every thread builds its window from the tile.
-// Thread tid of block bid takes cells bid*B + tid + k*nblk*B, the cells and
-// the order of residual_cells with first = bid*B + tid, stride = nblk*B, so
-// the partial sums are the same bits. sH, sQ: B + 4 doubles each.
-__device__ double residual_cells_staged(const Geo &G, const double *U, double *R, int bid, int nblk, double *sH,
-                                        double *sQ) {
-  const int B = blockDim.x, N = G.N;
-  const double *H = U, *Q = U + N;
-  double acc = 0.0;
-  for (int t0 = bid * B; t0 < N; t0 += nblk * B) {  // block-uniform
-    __syncthreads();                                // the previous tile's windows are read
-    for (int i = threadIdx.x; i < B + 4; i += B) {
-      const int k = min(max(t0 - 2 + i, 0), N - 1);  // clamped as load_win: ghosts are filled later
-      sH[i] = H[k];
-      sQ[i] = Q[k];
-    }
-    __syncthreads();
-    const int j = t0 + threadIdx.x;
-    if (j < N) {
-      Win w;
-#pragma unroll
-      for (int p = 0; p < 5; ++p) {
-        w.H[p] = sH[threadIdx.x + p];
-        w.Q[p] = sQ[threadIdx.x + p];
-      }
-      fill_ghosts(G, j, w);
-      double R0, R1;
-      local_residual(G, j, w, R0, R1);
-      R[j] = R0;
-      R[N + j] = R1;
-      acc += fabs(R0) + fabs(R1);
-    }
-  }
-  return acc;
-}
 
 // ----------------------------------------------------------------------------
 // Regularized FD Jacobian (Eq. 12-13) in three passes that share work between
@@ -1531,32 +1416,80 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// NSWE_RESIDUAL_SMEM (default 1): the standalone residual stages its WENO
-// windows in shared memory (residual_cells_staged); 0 reads them through L1.
-#ifndef NSWE_RESIDUAL_SMEM
-#define NSWE_RESIDUAL_SMEM 1
-#endif
+// The standalone residual by tiles of cells in shared memory: every WENO
+// reconstruction formed once (one per cell and component), then every face
+// flux and, on other warps, every source, then the differences. The FP64 pipe
+// bounds it: about 110 instruction slots per cell against 220 where each cell
+// rebuilds its neighbours' reconstructions and both its fluxes. Small levels
+// take tiles of 31 cells (32 faces: one warp), so that one channel spreads over
+// many SMs and the chain of a warp is one reconstruction and one flux; levels
+// that fill the chip that way take 254 (512 reconstructions for 256 threads).
+// The blocks of a level of at most 16 tiles are one cluster and form res too
+// (res given); else their sums go to `partials` for k_finish_res.
+constexpr int kResTileSmall = 31, kResThreadsSmall = 128, kResTile = 254, kResThreads = 256;
+constexpr int kResMaxBlocks = 1024;  // partial sums of a context
 
-__global__ void __launch_bounds__(kThreads) k_residual(const ProbDev *P, int level, const double *U, double *R,
-                                                       double *partials) {
-  __shared__ double red[33];
-  Geo G = make_geo(*P, level);
-#if NSWE_RESIDUAL_SMEM
-  __shared__ double sH[kThreads + 4], sQ[kThreads + 4];
-  double acc = residual_cells_staged(G, U, R, blockIdx.x, gridDim.x, sH, sQ);
-#else
-  double acc = residual_cells(G, U, R, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
-#endif
-  double s = block_sum(acc, red);
-  if (threadIdx.x == 0) partials[blockIdx.x] = s;
+template <int TILE, int THREADS>
+__global__ void __launch_bounds__(THREADS) k_residual(const ProbDev *P, int level, const double *U, double *R,
+                                                      double *partials, double *res) {
+  __shared__ double rec[2][2][TILE + 2], flx[2][TILE + 1], src[TILE], red[34];
+  const Geo G = make_geo(*P, level);
+  const int N = G.N;
+  double acc = 0.0;
+  for (int t0 = blockIdx.x * TILE; t0 < N; t0 += gridDim.x * TILE) {
+    const int cells = min(TILE, N - t0), w = cells + 2;
+    for (int it = threadIdx.x; it < 2 * w; it += THREADS) {
+      const int m = it >= w, i = it - m * w, k = t0 + i - 1;
+      auto at = [&](int kk) { return pval<double>(G, U, m, kk, -1, 0.0, 0.0); };
+      weno3<double>(at(k - 1), at(k), at(k + 1), rec[m][0][i], rec[m][1][i]);  // cell t0 + i - 1
+    }
+    __syncthreads();
+    const int first_src = (cells + 1 + 31) & ~31;
+    for (int it = threadIdx.x; it < first_src + cells; it += THREADS) {
+      if (it <= cells) {
+        const int f = t0 + it;
+        const Face<double> fc = face(G.isf[f], G.cgf[f], G.g);
+        num_flux<-1>(fstate(rec[0][1][it], rec[1][1][it], fc), fstate(rec[0][0][it + 1], rec[1][0][it + 1], fc), G.flux,
+                     flx[0][it], flx[1][it]);
+      } else if (it >= first_src) {
+        const int i = it - first_src;
+        src[i] = source_at(src_cell<double>(G, t0 + i), rec[0][0][i], rec[0][0][i + 1], rec[0][1][i + 1],
+                           rec[0][1][i + 2]);
+      }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < cells; i += THREADS) {
+      const double R0 = flx[0][i + 1] - flx[0][i];
+      const double R1 = flx[1][i + 1] - flx[1][i] - src[i];
+      R[t0 + i] = R0;
+      R[N + t0 + i] = R1;
+      acc += fabs(R0) + fabs(R1);
+    }
+    __syncthreads();  // the tile is read before the next one is built
+  }
+  const double s = block_sum(acc, red);
+  if (!res) {
+    if (threadIdx.x == 0) partials[blockIdx.x] = s;
+    return;
+  }
+  auto cl = cooperative_groups::this_cluster();
+  if (threadIdx.x == 0) red[33] = s;
+  cl.sync();
+  if (cl.block_rank() == 0 && threadIdx.x < 32) {
+    double v = threadIdx.x < cl.num_blocks() ? *cl.map_shared_rank(red + 33, threadIdx.x) : 0.0;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (threadIdx.x == 0) *res = v / N;
+  }
+  cl.sync();  // no block leaves while its sum may be read
 }
 
+// res from the block sums, by one block (one thread took 36 us for 1024).
 __global__ void __launch_bounds__(kThreads) k_finish_res(const double *partials, int n, int N, double *res) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < n; ++i) s += partials[i];
-    *res = s / N;
-  }
+  __shared__ double red[33];
+  double v = 0.0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) v += partials[i];
+  const double s = block_sum(v, red);
+  if (threadIdx.x == 0) *res = s / N;
 }
 
 __global__ void __launch_bounds__(kThreads) k_geom_derive(const ProbDev *P) {
@@ -1804,6 +1737,23 @@ __global__ void __launch_bounds__(THREADS, MINB)
   if constexpr (TM::kMulti) team.sync();  // no CTA leaves while another may read its shared memory
 }
 
+// A launch of `blocks` blocks in clusters of `ctas`; at: storage of its attribute.
+cudaLaunchConfig_t cluster_config(int blocks, int ctas, int threads, size_t smem, cudaStream_t s,
+                                  cudaLaunchAttribute *at) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks, 1, 1);
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)ctas;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
 int grid_for(int items) {
   int b = (items + kThreads - 1) / kThreads;
   return b < 1 ? 1 : (b > 1024 ? 1024 : b);
@@ -1824,10 +1774,26 @@ cudaError_t launch_geom_derive_batch(const SolveTask *tasks, int count, cudaStre
 
 cudaError_t launch_residual(const ProbDev *p, int level, int N, const double *U, double *R, double *res,
                             double *partials, cudaStream_t s) {
-  int grid = grid_for(N);
-  k_residual<<<grid, kThreads, 0, s>>>(p, level, U, R, partials);
-  if (res) k_finish_res<<<1, 32, 0, s>>>(partials, grid, N, res);
-  return cudaGetLastError();
+  const int small = (N + kResTileSmall - 1) / kResTileSmall;
+  if (small > 4 * kSmCount) {
+    const int tiles = (N + kResTile - 1) / kResTile, grid = tiles < kResMaxBlocks ? tiles : kResMaxBlocks;
+    k_residual<kResTile, kResThreads><<<grid, kResThreads, 0, s>>>(p, level, U, R, partials, nullptr);
+    if (res) k_finish_res<<<1, kThreads, 0, s>>>(partials, grid, N, res);
+    return cudaGetLastError();
+  }
+  auto kern = k_residual<kResTileSmall, kResThreadsSmall>;
+  if (!res || small > kMaxClusterCtas) {
+    kern<<<small, kResThreadsSmall, 0, s>>>(p, level, U, R, partials, nullptr);
+    if (res) k_finish_res<<<1, kThreads, 0, s>>>(partials, small, N, res);
+    return cudaGetLastError();
+  }
+  if (small > 8) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchAttribute at[1];
+  const cudaLaunchConfig_t cfg = cluster_config(small, small, kResThreadsSmall, 0, s, at);
+  return cudaLaunchKernelEx(&cfg, kern, p, level, U, R, partials, res);
 }
 
 cudaError_t launch_jacobian(const ProbDev *p, int level, int N, int nb, const double *U, double eps,
@@ -1836,7 +1802,7 @@ cudaError_t launch_jacobian(const ProbDev *p, int level, int N, int nb, const do
   k_jac_b<double><<<grid_for(N + 1), kThreads, 0, s>>>(p, level);
   const int grid = grid_for(N * nb);
   k_jac_c<double><<<grid, kThreads, 0, s>>>(p, level, nb, eps, alpha, nullptr, R, J, partials);
-  if (res) k_finish_res<<<1, 32, 0, s>>>(partials, grid, N, res);
+  if (res) k_finish_res<<<1, kThreads, 0, s>>>(partials, grid, N, res);
   return cudaGetLastError();
 }
 
@@ -1898,18 +1864,8 @@ cudaError_t launch_cluster_t(const SolveTask *tasks, int count, const nswe_param
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)count * (unsigned)ctas, 1, 1);
-  cfg.blockDim = dim3(kClusterThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)ctas;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
+  const cudaLaunchConfig_t cfg = cluster_config(count * ctas, ctas, kClusterThreads, smem, s, at);
   return cudaLaunchKernelEx(&cfg, kern, tasks, prm, n_cap, ldab_cap, team_cells);
 }
 }  // namespace
