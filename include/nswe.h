@@ -467,10 +467,11 @@ nswe_status nswe_ctx_get_solve_shape(nswe_ctx ctx, int precision, int *shape);
  * itself is unchanged): with ctas >= 2, nswe_newton_solve and
  * nswe_newton_solve_batch give each 1D problem a thread-block cluster of
  * `ctas` CTAs (128 threads each) on as many SMs instead of one thread block.
- * The residual, Jacobian, update and the multigrid levels of at least
- * team_cells cells run on all CTAs of the cluster, with cluster barriers
- * between phases; the coarser levels and the coarsest LU run on its first
- * CTA. Every cell sees the same arithmetic as in the block form; the sum
+ * The residual, Jacobian, update and the multigrid run on all CTAs of the
+ * cluster, with cluster barriers between phases; the smallest levels (and, of
+ * those whose smoother goes pass by pass, as with the full Jacobian or more
+ * than two smoothing steps, the levels of less than team_cells cells) and the
+ * coarsest LU run on its first CTA. Every cell sees the same arithmetic as in the block form; the sum
  * that forms res is taken in another order, so res (and in rare cases the
  * Newton step at which it crosses tol) may differ in the last bits.
  * Worthwhile for few problems at a time (one solve's latency); a full batch

@@ -1030,10 +1030,8 @@ nswe_status nswe_mg_vcycle_f32(nswe_ctx ctx, nswe_prob prob, int level, int nb, 
   DeviceGuard dg(ctx->device);
   if (prob->dim == 2) return vcycle2d_entry<float>(ctx, prob, level, nb, J, R, dU, *params);
   if (nb != 3 && nb != 5) return NSWE_EINVAL;
-  const int coarse = prob->N >> (prob->levels - 1);
-  const int coarse_nb = (level == prob->levels - 1) ? nb : 3;
-  return launch_vcycle_f32(prob->dev, level, nb, J, R, dU, *params, ctx->status, coarse, coarse_nb, ctx->stream) ==
-                 cudaSuccess
+  return launch_vcycle_f32(prob->dev, level, prob->levels, prob->N >> level, nb, J, R, dU, *params, ctx->status,
+                           ctx->stream) == cudaSuccess
              ? NSWE_OK
              : NSWE_ECUDA;
 }
@@ -1046,10 +1044,8 @@ nswe_status nswe_mg_vcycle(nswe_ctx ctx, nswe_prob prob, int level, int nb, cons
   DeviceGuard dg(ctx->device);
   if (prob->dim == 2) return vcycle2d_entry<double>(ctx, prob, level, nb, J, R, dU, *params);
   if (nb != 3 && nb != 5) return NSWE_EINVAL;
-  const int coarse = prob->N >> (prob->levels - 1);
-  const int coarse_nb = (level == prob->levels - 1) ? nb : 3;
-  return launch_vcycle(prob->dev, level, nb, J, R, dU, *params, ctx->status, coarse, coarse_nb, ctx->stream) ==
-                 cudaSuccess
+  return launch_vcycle(prob->dev, level, prob->levels, prob->N >> level, nb, J, R, dU, *params, ctx->status,
+                       ctx->stream) == cudaSuccess
              ? NSWE_OK
              : NSWE_ECUDA;
 }

@@ -780,12 +780,12 @@ __device__ void geom_derive_items(const ProbDev &P, int first, int stride) {
   }
 }
 
-// Inverse of the diagonal 2x2 blocks, times -omega: the factor with which the
+// Inverse of the diagonal 2x2 blocks of cells first, first + stride, .. < end, times -omega: the factor with which the
 // smoother applies them.
 template <typename T>
-__device__ void dinv_cells(int N, int nb, const T *J, T *Dinv, double omega, int first, int stride) {
+__device__ void dinv_cells(int N, int nb, const T *J, T *Dinv, double omega, int first, int end, int stride) {
   const int hw = (nb - 1) / 2;
-  for (int j = first; j < N; j += stride) {
+  for (int j = first; j < end; j += stride) {
     T a = J[(hw * 4 + 0) * N + j], b = J[(hw * 4 + 1) * N + j];
     T c = J[(hw * 4 + 2) * N + j], d = J[(hw * 4 + 3) * N + j];
     const T s = T(-omega) * rcp_t(fma(a, d, -(b * c)));
@@ -801,9 +801,9 @@ __device__ void dinv_cells(int N, int nb, const T *J, T *Dinv, double omega, int
 // coarse blocks J_-1(2j), J_0(2j) + J_+1(2j) + J_-1(2j+1) + J_0(2j+1) and
 // J_+1(2j+1), summed in the order of the general loop below.
 template <typename T>
-__device__ void coarse_op_cells(int Nf, int nbf, const T *Jf, int Nc, T *Jc, int first, int stride) {
+__device__ void coarse_op_cells(int Nf, int nbf, const T *Jf, int Nc, T *Jc, int first, int end, int stride) {
   const int hf = (nbf - 1) / 2;
-  for (int j = first; j < Nc; j += stride) {
+  for (int j = first; j < end; j += stride) {
     if (nbf == 3 && j > 0 && 2 * j + 2 < Nf) {
       const int x0 = 2 * j, x1 = 2 * j + 1;
 #pragma unroll
@@ -1287,44 +1287,168 @@ __device__ void mg_bind(MG<T> &mg, const ProbDev &P, int l0, int nb0, const T *J
   }
 }
 
-// First multigrid level run by the leader CTA alone: a cluster team runs
-// the levels with at least team_cells cells (from l0 down) on all its CTAs
-// and the coarser ones, with the coarsest solve, on the leader; a block team
-// runs every level (the coarsest solve is level L).
-template <typename T, class TM>
-__device__ __forceinline__ int team_split(const MG<T> &mg, int team_cells) {
-  if constexpr (!TM::kMulti) return mg.L;
-  int lt = mg.l0;
-  while (lt < mg.L && mg.N[lt] >= team_cells) ++lt;
-  return lt;
+// ----------------------------------------------------------------------------
+// Legs: the smoothing of one level with the restriction behind it (down) or
+// the prolongation before it (up) as one pass without barriers. A warp takes
+// a tile of 16 cell pairs, two lanes per pair (one per component), holds the
+// pairs' operator rows, right-hand side and correction in registers and runs
+// all colour passes on them, neighbours' values by shuffles. Values spoil from
+// the tile's edges by one cell per pass: with at most five passes (two
+// symmetric steps of the two-colour smoother) and the restriction, 3 pairs on
+// either side, so tiles overlap by 6 pairs and each writes its inner ones; at
+// the domain's ends nothing spoils. What a tile reads is never what another
+// writes: a leg's result goes to another buffer than its source.
+// Why: on few SMs a pass is a barrier (0.2 us in a cluster), a trip to L2 for
+// operator and correction (0.4 us) and 14 FP64 instructions of 64 cycles; a
+// leg pays the first two once instead of six times and, with two lanes per
+// cell, 7 instructions per pass, for 1.6 times the arithmetic. A full batch,
+// one block per problem, is bound by the FP64 pipe and smooths pass by pass.
+// Cells see the operations of sor_colour, restrict_cells and prolong_cells in
+// their order.
+// GB300: a 4096-cell solve on 16 CTAs 77.3 -> 69.4 ms.
+constexpr int kLegPairs = 16, kLegOwn = 10, kLegHalo = 3, kLegSteps = 2;
+
+__host__ __device__ inline int leg_tiles(int N) {
+  return N / 2 <= kLegPairs ? 1 : (N / 2 - kLegPairs + kLegOwn - 1) / kLegOwn + 1;
+}
+// Whether a level is smoothed by legs.
+__host__ __device__ inline bool leg_level(int nb, const nswe_params &prm) {
+  return nb == 3 && prm.nu1 >= 1 && prm.nu1 <= kLegSteps && prm.nu2 >= 1 && prm.nu2 <= kLegSteps;
+}
+
+// One tile. src: the correction on entry (null: zero). Down: Rc receives the
+// restricted defect. UP: dUc, the coarse correction, is added first.
+template <typename T, bool UP>
+__device__ __forceinline__ void leg_tile(int N, const T *J, const T *Dinv, const T *R, const T *src, T *dst,
+                                         const T *dUc, T *Rc, int steps, T keep, int tile, int tiles) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, p = lane >> 1, c = lane & 1, pairs = N / 2;
+  const int P = kLegOwn * tile + p, je = 2 * P, jo = je + 1;
+  const bool in = P < pairs;
+  auto blk = [&](int k, int q, int j, bool on) { return on ? J[(k * 4 + 2 * c + q) * N + j] : T(0.0); };
+  const bool left = in && je > 0, right = in && jo < N - 1;
+  const T em0 = blk(0, 0, je, left), em1 = blk(0, 1, je, left), ep0 = blk(2, 0, je, in), ep1 = blk(2, 1, je, in);
+  const T om0 = blk(0, 0, jo, in), om1 = blk(0, 1, jo, in), op0 = blk(2, 0, jo, right), op1 = blk(2, 1, jo, right);
+  auto at = [&](const T *A, int i) { return in ? A[i] : T(0.0); };
+  const T ed0 = at(Dinv, 2 * c * N + je), ed1 = at(Dinv, (2 * c + 1) * N + je);
+  const T od0 = at(Dinv, 2 * c * N + jo), od1 = at(Dinv, (2 * c + 1) * N + jo);
+  const T re = at(R, c * N + je), ro = at(R, c * N + jo);
+  T xe = T(0.0), xo = T(0.0);
+  if (src) {
+    xe = at(src, c * N + je);
+    xo = at(src, c * N + jo);
+  }
+  if (UP) {
+    const T xc = at(dUc, c * pairs + P);
+    xe += xc;
+    xo += xc;
+  }
+  // both components of a lane's value and of the value of the pair before / after it
+  auto both = [&](T v, int pp, T &v0, T &v1) {
+    const int at0 = 2 * min(max(pp, 0), kLegPairs - 1);
+    v0 = __shfl_sync(FULL, v, at0);
+    v1 = __shfl_sync(FULL, v, at0 + 1);
+  };
+  T a0, a1, b0, b1;  // neighbours before and after
+  auto relax = [&](T r, T d0, T d1, T x, int reps) {
+    const T other = __shfl_xor_sync(FULL, r, 1);
+    const T r0 = c ? other : r, r1 = c ? r : other;
+    const T t = fma(d0, r0, d1 * r1);
+    x = fma(keep, x, t);
+    return reps == 2 ? fma(keep, x, t) : x;
+  };
+  for (int v = 0; v <= 2 * steps; ++v) {
+    const int reps = v == 0 || v == 2 * steps ? 1 : 2;
+    if ((v & 1) == 0) {
+      T r = re;
+      if (UP || src || v > 0) {
+        both(xo, p - 1, a0, a1);
+        both(xo, p, b0, b1);
+        r = fma(ep1, b1, fma(ep0, b0, fma(em1, a1, fma(em0, a0, r))));
+      }
+      xe = relax(r, ed0, ed1, xe, reps);
+    } else {
+      both(xe, p, a0, a1);
+      both(xe, p + 1, b0, b1);
+      const T r = fma(op1, b1, fma(op0, b0, fma(om1, a1, fma(om0, a0, ro))));
+      xo = relax(r, od0, od1, xo, reps);
+    }
+  }
+  const bool own = in && (p >= kLegHalo || tile == 0) && (p < kLegHalo + kLegOwn || tile == tiles - 1);
+  if (own) {
+    dst[c * N + je] = xe;
+    dst[c * N + jo] = xo;
+  }
+  if (!UP) {
+    T l0, l1, e0, e1, o0, o1, n0, n1;
+    both(xo, p - 1, l0, l1);
+    both(xe, p, e0, e1);
+    both(xo, p, o0, o1);
+    both(xe, p + 1, n0, n1);
+    const T ec0 = blk(1, 0, je, in), ec1 = blk(1, 1, je, in), oc0 = blk(1, 0, jo, in), oc1 = blk(1, 1, jo, in);
+    const T se = fma(ep1, o1, fma(ep0, o0, fma(ec1, e1, fma(ec0, e0, fma(em1, l1, fma(em0, l0, re))))));
+    const T so = fma(op1, n1, fma(op0, n0, fma(oc1, o1, fma(oc0, o0, fma(om1, e1, fma(om0, e0, ro))))));
+    if (own) Rc[c * pairs + P] = se + so;
+  }
+}
+
+// The leg's tiles `warp`, `warp` + warps, ...
+template <typename T, bool UP>
+__device__ void leg(int N, const T *J, const T *Dinv, const T *R, const T *src, T *dst, const T *dUc, T *Rc,
+                    int steps, double omega, int warp, int warps) {
+  const int tiles = leg_tiles(N);
+  for (int t = warp; t < tiles; t += warps)
+    leg_tile<T, UP>(N, J, Dinv, R, src, dst, dUc, Rc, steps, T(1.0) - T(omega), t, tiles);
+}
+
+// Where the up leg of a level leaves its correction: beside the level's
+// operator in its storage (20 N values of FP64, of which J3 takes 12 N and a
+// mixed step's right-hand side 2 N). The other levels' stays in dU.
+template <typename T>
+__device__ __forceinline__ T *leg_out(T *J, int N) {
+  return J + 14 * (size_t)N;
+}
+
+// Coarse operators of the levels below l0 and diagonal inverses, block `part`
+// of `parts`: its share of the coarsest cells and the cells below them on
+// every level, which need nothing from outside.
+template <typename T>
+__device__ void mg_setup_part(const MG<T> &mg, double omega, int part, int parts) {
+  const int NL = mg.N[mg.L], c0 = NL * part / parts, c1 = NL * (part + 1) / parts;
+  for (int l = mg.l0 + 1; l <= mg.L; ++l) {
+    const int sh = mg.L - l;
+    coarse_op_cells(mg.N[l - 1], mg.nb[l - 1], mg.J[l - 1], mg.N[l], mg.J[l], (c0 << sh) + (int)threadIdx.x, c1 << sh,
+                    (int)blockDim.x);
+    __syncthreads();
+  }
+  for (int l = mg.l0; l < mg.L; ++l) {
+    const int sh = mg.L - l;
+    dinv_cells(mg.N[l], mg.nb[l], mg.J[l], mg.Dinv[l], omega, (c0 << sh) + (int)threadIdx.x, c1 << sh,
+               (int)blockDim.x);
+  }
 }
 
 // Coarse operators, diagonal inverses and the coarsest factorisation; done
 // once per Newton step since J is fixed during its V-cycles. Returns whether
 // a pivot was exactly zero, in every thread of the team.
 template <typename T, class TM = BlockTeam>
-__device__ bool mg_setup(const MG<T> &mg, Band<T> &B, double omega, const TM &team = TM(), int team_cells = 0) {
-  const int lt = team_split<T, TM>(mg, team_cells);
-  for (int l = mg.l0 + 1; l < lt; ++l) {
-    coarse_op_cells(mg.N[l - 1], mg.nb[l - 1], mg.J[l - 1], mg.N[l], mg.J[l], team.tid(), team.size());
+__device__ bool mg_setup(const MG<T> &mg, Band<T> &B, double omega, const TM &team = TM()) {
+  if constexpr (TM::kMulti) {
+    mg_setup_part(mg, omega, team.rank, team.n);
     team.sync();
-  }
-  if (team.lead())
-    for (int l = max(mg.l0 + 1, lt); l <= mg.L; ++l) {
-      coarse_op_cells(mg.N[l - 1], mg.nb[l - 1], mg.J[l - 1], mg.N[l], mg.J[l], threadIdx.x, blockDim.x);
+    if (team.lead()) band_factor(B, mg.N[mg.L], mg.nb[mg.L], mg.J[mg.L]);
+    team.sync();  // the leader's factors and flag are done
+    return team.lead_value(&s_sing) != 0;
+  } else {
+    for (int l = mg.l0 + 1; l <= mg.L; ++l) {
+      coarse_op_cells(mg.N[l - 1], mg.nb[l - 1], mg.J[l - 1], mg.N[l], mg.J[l], (int)threadIdx.x, mg.N[l],
+                      (int)blockDim.x);
       __syncthreads();
     }
-  for (int l = mg.l0; l < lt; ++l) dinv_cells(mg.N[l], mg.nb[l], mg.J[l], mg.Dinv[l], omega, team.tid(), team.size());
-  bool sing = false;
-  if (team.lead()) {
-    for (int l = lt; l < mg.L; ++l) dinv_cells(mg.N[l], mg.nb[l], mg.J[l], mg.Dinv[l], omega, threadIdx.x, blockDim.x);
-    sing = band_factor(B, mg.N[mg.L], mg.nb[mg.L], mg.J[mg.L]);
+    for (int l = mg.l0; l < mg.L; ++l)
+      dinv_cells(mg.N[l], mg.nb[l], mg.J[l], mg.Dinv[l], omega, (int)threadIdx.x, mg.N[l], (int)blockDim.x);
+    return band_factor(B, mg.N[mg.L], mg.nb[mg.L], mg.J[mg.L]);
   }
-  if constexpr (TM::kMulti) {
-    team.sync();  // the team's inverses and the leader's factors and flag are done
-    sing = team.lead_value(&s_sing) != 0;
-  }
-  return sing;
 }
 
 // `steps` symmetric multicolour SOR steps (colours 0..C-1 then C-1..0 each);
@@ -1356,40 +1480,76 @@ __device__ void sor_smooth(const MG<T> &mg, int l, int steps, double omega, bool
   }
 }
 
-// Algorithm 2 from level l0, unrolled over levels. zero: dU of level l0 is
-// all zero (that of a coarser level always is, by the restriction). A cluster team smooths,
-// restricts and prolongs the levels l0..lt-1; the leader CTA runs the
-// V-cycle below them (levels lt..L) between two cluster barriers.
-template <typename T, class TM = BlockTeam>
-__device__ void mg_vcycle(const MG<T> &mg, const Band<T> &B, const nswe_params &prm, bool zero,
-                          const TM &team = TM(), int team_cells = 0) {
-  const int lt = team_split<T, TM>(mg, team_cells);
-  for (int l = mg.l0; l < lt; ++l) {
-    sor_smooth(mg, l, prm.nu1, prm.omega, zero || l > mg.l0, team);
+// Algorithm 2 from level l0 by one block, pass by pass. zero: dU of level l0
+// is all zero (that of a coarser level always is, by the restriction).
+template <typename T>
+__device__ void mg_vcycle(const MG<T> &mg, const Band<T> &B, const nswe_params &prm, bool zero) {
+  for (int l = mg.l0; l < mg.L; ++l) {
+    sor_smooth(mg, l, prm.nu1, prm.omega, zero || l > mg.l0);
     restrict_cells(mg.N[l], mg.nb[l], mg.J[l], mg.R[l], mg.dU[l], mg.N[l + 1], mg.R[l + 1], mg.dU[l + 1],
-                   team.tid(), team.size());
-    team.sync();
+                   threadIdx.x, blockDim.x);
+    __syncthreads();
   }
+  band_solve(B, mg.N[mg.L], mg.R[mg.L], mg.dU[mg.L]);
+  for (int l = mg.L - 1; l >= mg.l0; --l) {
+    prolong_cells(mg.N[l], mg.dU[l], mg.N[l + 1], mg.dU[l + 1], threadIdx.x, blockDim.x);
+    __syncthreads();
+    sor_smooth(mg, l, prm.nu2, prm.omega, false);
+  }
+}
+
+// Algorithm 2 from level ls >= l0 by a cluster. Levels that can be take legs
+// (leg_level), the others (the full Jacobian's own level, more than two
+// smoothing steps) go pass by pass. The levels of at most a tile per warp of a
+// block, and of less than team_cells cells where they go pass by pass, run on
+// the leader CTA with block barriers, and the coarsest solve. out0: the
+// correction of level l0, on return and (unless zero) on entry; for a level
+// smoothed by passes it is mg.dU[l0]. ready: called by the leader before the
+// coarsest solve.
+template <typename T, typename F>
+__device__ void mg_vcycle_cluster(const MG<T> &mg, const Band<T> &B, const nswe_params &prm, bool zero, T *out0,
+                                  const ClusterTeam &team, int team_cells, int ls, F &&ready) {
+  const int nw = (int)blockDim.x >> 5;
+  auto lead_level = [&](int l) {
+    return leg_level(mg.nb[l], prm) ? leg_tiles(mg.N[l]) <= nw : mg.N[l] < team_cells;
+  };
+  int lt = ls;
+  while (lt < mg.L && !lead_level(lt)) ++lt;
+  auto out = [&](int l) {
+    return l == mg.l0 ? out0 : l < mg.L && leg_level(mg.nb[l], prm) ? leg_out(mg.J[l], mg.N[l]) : mg.dU[l];
+  };
+  auto down = [&](int l, const auto &tm) {
+    if (leg_level(mg.nb[l], prm)) {
+      leg<T, false>(mg.N[l], mg.J[l], mg.Dinv[l], mg.R[l], l > mg.l0 || zero ? nullptr : out0, mg.dU[l], nullptr,
+                    mg.R[l + 1], prm.nu1, prm.omega, tm.tid() >> 5, tm.size() >> 5);
+      tm.sync();
+      return;
+    }
+    sor_smooth(mg, l, prm.nu1, prm.omega, zero || l > mg.l0, tm);
+    restrict_cells(mg.N[l], mg.nb[l], mg.J[l], mg.R[l], mg.dU[l], mg.N[l + 1], mg.R[l + 1], mg.dU[l + 1], tm.tid(),
+                   tm.size());
+    tm.sync();
+  };
+  auto up = [&](int l, const auto &tm) {
+    if (leg_level(mg.nb[l], prm)) {
+      leg<T, true>(mg.N[l], mg.J[l], mg.Dinv[l], mg.R[l], mg.dU[l], out(l), out(l + 1), nullptr, prm.nu2, prm.omega,
+                   tm.tid() >> 5, tm.size() >> 5);
+      tm.sync();
+      return;
+    }
+    prolong_cells(mg.N[l], mg.dU[l], mg.N[l + 1], out(l + 1), tm.tid(), tm.size());
+    tm.sync();
+    sor_smooth(mg, l, prm.nu2, prm.omega, false, tm);
+  };
+  for (int l = ls; l < lt; ++l) down(l, team);
   if (team.lead()) {
-    for (int l = lt; l < mg.L; ++l) {
-      sor_smooth(mg, l, prm.nu1, prm.omega, zero || l > mg.l0);
-      restrict_cells(mg.N[l], mg.nb[l], mg.J[l], mg.R[l], mg.dU[l], mg.N[l + 1], mg.R[l + 1], mg.dU[l + 1],
-                     threadIdx.x, blockDim.x);
-      __syncthreads();
-    }
+    for (int l = lt; l < mg.L; ++l) down(l, BlockTeam());
+    ready();
     band_solve(B, mg.N[mg.L], mg.R[mg.L], mg.dU[mg.L]);
-    for (int l = mg.L - 1; l >= lt; --l) {
-      prolong_cells(mg.N[l], mg.dU[l], mg.N[l + 1], mg.dU[l + 1], threadIdx.x, blockDim.x);
-      __syncthreads();
-      sor_smooth(mg, l, prm.nu2, prm.omega, false);
-    }
+    for (int l = mg.L - 1; l >= lt; --l) up(l, BlockTeam());
   }
-  if constexpr (TM::kMulti) team.sync();
-  for (int l = lt - 1; l >= mg.l0; --l) {
-    prolong_cells(mg.N[l], mg.dU[l], mg.N[l + 1], mg.dU[l + 1], team.tid(), team.size());
-    team.sync();
-    sor_smooth(mg, l, prm.nu2, prm.omega, false, team);
-  }
+  team.sync();
+  for (int l = lt - 1; l >= ls; --l) up(l, team);
 }
 
 // Band storage in dynamic shared memory, sized by the host for the coarsest
@@ -1409,6 +1569,12 @@ __device__ __forceinline__ Band<T> band_view(int n_cap, int ldab_cap) {
 
 // ----------------------------------------------------------------------------
 // Kernels.
+
+constexpr int kVcThreads = 128;       // a warp per SM sub-partition: the FP64 pipe sets a leg's time
+// Larger levels are launches over the chip: four rounds of a cluster's 16 x 4
+// warps cost less than a launch and its gap per leg (4096 cells, 205 tiles:
+// 146 us with 256 here, 157 with 64).
+constexpr int kVcClusterTiles = 256;
 
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
@@ -1525,16 +1691,93 @@ __global__ void __launch_bounds__(kThreads) k_jac_c(const ProbDev *P, int level,
   if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 
+// A standalone V-cycle: coarse operators and inverses (k_vc_setup, a block per
+// coarsest cell), the coarsest factorisation (k_vc_factor, one block, left in
+// the Jacobian workspace), then k_vc_cluster with the levels that one cluster
+// of 16 blocks takes, started beside the factorisation; larger levels are
+// launches of their own before and after it (k_vc_leg). One block for all of
+// it took 513 us for 4096 cells, this 146.
+// The factors lie at the front of the workspace: ab, rinv, piv of Band.
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_vcycle(const ProbDev *P, int level, int nb, const T *J, const T *R,
-                                                     T *dU, nswe_params prm, int *status, int n_cap, int ldab_cap) {
+__global__ void __launch_bounds__(kThreads) k_vc_setup(const ProbDev *P, int level, int nb, const T *J,
+                                                       double omega) {
   MG<T> mg;
-  mg_bind<T>(mg, *P, level, nb, J, R, dU);
+  mg_bind<T>(mg, *P, level, nb, J, nullptr, nullptr);
+  mg_setup_part(mg, omega, blockIdx.x, gridDim.x);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_vc_factor(const ProbDev *P, int *status, int n_cap, int ldab_cap) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   Band<T> B = band_view<T>(n_cap, ldab_cap);
-  bool sing = mg_setup<T>(mg, B, prm.omega);
-  __syncthreads();
-  mg_vcycle<T>(mg, B, prm, false);
+  const LevelDev &Lv = P->lev[P->levels - 1];
+  const bool sing = band_factor(B, Lv.N, 3, reinterpret_cast<const T *>(Lv.J));
+  Band<T> G = B;
+  G.ab = reinterpret_cast<T *>(P->jw);
+  G.rinv = G.ab + (size_t)B.ldab * B.n;
+  G.piv = reinterpret_cast<int *>(G.rinv + B.n);
+  for (int t = threadIdx.x; t < B.ldab * B.n; t += blockDim.x) G.ab[t] = B.ab[t];
+  for (int t = threadIdx.x; t < B.n; t += blockDim.x) {
+    G.rinv[t] = B.rinv[t];
+    G.piv[t] = B.piv[t];
+  }
   if (threadIdx.x == 0) *status = sing ? NSWE_ESINGULAR : NSWE_OK;
+}
+
+// ls: the first level of the cluster (l0 = level: all of them).
+template <typename T>
+__global__ void __launch_bounds__(kVcThreads, 1)
+    k_vc_cluster(const ProbDev *P, int level, int ls, int nb, const T *J, const T *R, T *dU,
+                 const __grid_constant__ nswe_params prm, int n_cap, int ldab_cap) {
+  const auto cl = cooperative_groups::this_cluster();
+  const ClusterTeam team{(int)cl.block_rank(), (int)cl.num_blocks()};
+  MG<T> mg;
+  mg_bind<T>(mg, *P, level, nb, J, R, leg_level(nb, prm) ? reinterpret_cast<T *>(P->lev[level].dU) : dU);
+  Band<T> B = band_view<T>(n_cap, ldab_cap);
+  B.n = 2 * mg.N[mg.L];
+  B.kl = 3;
+  B.ldab = 10;
+  mg_vcycle_cluster<T>(mg, B, prm, false, dU, team, 0, ls, [&] {
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the factors are there
+    const T *ab = reinterpret_cast<const T *>(P->jw), *rinv = ab + (size_t)B.ldab * B.n;
+    const int *piv = reinterpret_cast<const int *>(rinv + B.n);
+    for (int t = threadIdx.x; t < B.ldab * B.n; t += blockDim.x) B.ab[t] = ab[t];
+    for (int t = threadIdx.x; t < B.n; t += blockDim.x) {
+      B.rinv[t] = rinv[t];
+      B.piv[t] = piv[t];
+    }
+    __syncthreads();
+  });
+}
+
+// The coarsest level's own system: the direct solve.
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_vc_direct(int N, int nb, const T *J, const T *R, T *dU, int *status,
+                                                        int n_cap, int ldab_cap) {
+  Band<T> B = band_view<T>(n_cap, ldab_cap);
+  const bool sing = band_factor(B, N, nb, J);
+  band_solve(B, N, R, dU);
+  if (threadIdx.x == 0) *status = sing ? NSWE_ESINGULAR : NSWE_OK;
+}
+
+// One leg of one level on the whole chip; level l0 takes the caller's arrays.
+template <typename T, bool UP>
+__global__ void __launch_bounds__(kVcThreads, 4) k_vc_leg(const ProbDev *P, int l, int l0, const T *J, const T *R, T *dU,
+                                                       int steps, double omega) {
+  const LevelDev &Lv = P->lev[l], &Lc = P->lev[l + 1];
+  const int N = Lv.N, warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, warps = (gridDim.x * blockDim.x) >> 5;
+  T *const Jl = l == l0 ? const_cast<T *>(J) : reinterpret_cast<T *>(Lv.J);
+  const T *const Rl = l == l0 ? R : reinterpret_cast<const T *>(Lv.R);
+  T *const mid = reinterpret_cast<T *>(Lv.dU), *const out = l == l0 ? dU : leg_out(Jl, N);
+  const T *const Dinv = reinterpret_cast<const T *>(Lv.Dinv);
+  T *const Jc = reinterpret_cast<T *>(Lc.J);
+  if (UP)
+    leg<T, true>(N, Jl, Dinv, Rl, mid, out,
+                 l + 1 == P->levels - 1 ? reinterpret_cast<const T *>(Lc.dU) : leg_out(Jc, Lc.N), nullptr, steps,
+                 omega, warp, warps);
+  else
+    leg<T, false>(N, Jl, Dinv, Rl, l == l0 ? out : nullptr, mid, nullptr, reinterpret_cast<T *>(Lc.R), steps, omega,
+                  warp, warps);
 }
 
 // The team of the calling thread and the index of its problem: a block per
@@ -1656,28 +1899,39 @@ __global__ void __launch_bounds__(THREADS, MINB)
       }
       MG<T> mg;
       mg_bind<T>(mg, P, l, nb, J, Rs, dU);
-      bool sing = mg_setup<T, TM>(mg, B, prm.omega, team, team_cells);
+      bool sing = mg_setup<T, TM>(mg, B, prm.omega, team);
       team.sync();
       if (sing) {
         st = NSWE_ESINGULAR;
         break;
       }
+      T *x = dU;  // where the correction ends
       if (l == L) {
         if (team.lead()) band_solve<T>(B, N, Rs, dU);
         if constexpr (TM::kMulti) team.sync();
+      } else if constexpr (TM::kMulti) {
+        if (leg_level(nb, prm)) x = leg_out(J, N);
+        if (!leg_level(nb, prm) || prm.nu3 < 1) {
+          for (int t = team.tid(); t < 2 * N; t += team.size()) x[t] = T(0.0);
+          team.sync();
+        }
+        for (int m = 0; m < prm.nu3; ++m) {
+          mg_vcycle_cluster<T>(mg, B, prm, m == 0, x, team, team_cells, l, [] {});
+          ++vcycles;
+        }
       } else {
         for (int t = team.tid(); t < 2 * N; t += team.size()) dU[t] = T(0.0);
         team.sync();
         for (int m = 0; m < prm.nu3; ++m) {
-          mg_vcycle<T, TM>(mg, B, prm, m == 0, team, team_cells);
+          mg_vcycle<T>(mg, B, prm, m == 0);
           ++vcycles;
         }
       }
       bool bad = false;
       for (int j = team.tid(); j < N; j += team.size()) {
-        double h = Lv.U[j] + prm.tau * double(dU[j]);
+        double h = Lv.U[j] + prm.tau * double(x[j]);
         Lv.U[j] = h;
-        Lv.U[N + j] += prm.tau * double(dU[N + j]);
+        Lv.U[N + j] += prm.tau * double(x[N + j]);
         if constexpr (kMixed) {
           U32[j] = float(h);
           U32[N + j] = float(Lv.U[N + j]);
@@ -1822,20 +2076,50 @@ size_t band_smem_bytes(int n_cap, int ldab_cap) {
   return sizeof(double) * ((size_t)ldab_cap * n_cap + 2 * (size_t)n_cap) + sizeof(int) * (size_t)n_cap;
 }
 
-cudaError_t launch_vcycle(const ProbDev *p, int level, int nb, const double *J, const double *R, double *dU,
-                          const nswe_params &prm, int *status, int coarse_cells, int coarse_nb, cudaStream_t s) {
-  const int n_cap = 2 * coarse_cells, ldab_cap = 3 * (coarse_nb == 5 ? 5 : 3) + 1;
-  k_vcycle<double><<<1, kThreads, band_smem_bytes(n_cap, ldab_cap), s>>>(p, level, nb, J, R, dU, prm, status,
-                                                                        n_cap, ldab_cap);
+namespace {
+template <typename T>
+cudaError_t vcycle_t(const ProbDev *p, int level, int levels, int N, int nb, const T *J, const T *R, T *dU,
+                     const nswe_params &prm, int *status, cudaStream_t s) {
+  const int L = levels - 1, NL = N >> (L - level), n_cap = 2 * NL;
+  const int ldab_cap = 3 * (level == L && nb == 5 ? 5 : 3) + 1;
+  const size_t smem = band_smem_bytes(n_cap, ldab_cap);
+  if (level == L) {
+    k_vc_direct<T><<<1, kThreads, smem, s>>>(N, nb, J, R, dU, status, n_cap, ldab_cap);
+    return cudaGetLastError();
+  }
+  k_vc_setup<T><<<NL, kThreads, 0, s>>>(p, level, nb, J, prm.omega);
+  // Levels of more than kVcClusterTiles tiles are launches over the chip.
+  int ls = level;
+  while (ls < L && leg_level(ls == level ? nb : 3, prm) && leg_tiles(N >> (ls - level)) > kVcClusterTiles) ++ls;
+  auto grid = [&](int l) { return (leg_tiles(N >> (l - level)) + kVcThreads / 32 - 1) / (kVcThreads / 32); };
+  for (int l = level; l < ls; ++l)
+    k_vc_leg<T, false><<<grid(l), kVcThreads, 0, s>>>(p, l, level, J, R, dU, prm.nu1, prm.omega);
+  k_vc_factor<T><<<1, kThreads, smem, s>>>(p, status, n_cap, ldab_cap);
+  auto kern = k_vc_cluster<T>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute at[2];
+  cudaLaunchConfig_t cfg = cluster_config(kMaxClusterCtas, kMaxClusterCtas, kVcThreads, smem, s, at);
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if ((e = cudaStreamIsCapturing(s, &cs)) != cudaSuccess) return e;
+  if (cs == cudaStreamCaptureStatusNone) cfg.numAttrs = 2;  // (a capture keeps stream order)
+  if ((e = cudaLaunchKernelEx(&cfg, kern, p, level, ls, nb, J, R, dU, prm, n_cap, ldab_cap)) != cudaSuccess) return e;
+  for (int l = ls - 1; l >= level; --l)
+    k_vc_leg<T, true><<<grid(l), kVcThreads, 0, s>>>(p, l, level, J, R, dU, prm.nu2, prm.omega);
   return cudaGetLastError();
 }
+}  // namespace
 
-cudaError_t launch_vcycle_f32(const ProbDev *p, int level, int nb, const float *J, const float *R, float *dU,
-                              const nswe_params &prm, int *status, int coarse_cells, int coarse_nb, cudaStream_t s) {
-  const int n_cap = 2 * coarse_cells, ldab_cap = 3 * (coarse_nb == 5 ? 5 : 3) + 1;
-  k_vcycle<float><<<1, kThreads, band_smem_bytes(n_cap, ldab_cap), s>>>(p, level, nb, J, R, dU, prm, status,
-                                                                       n_cap, ldab_cap);
-  return cudaGetLastError();
+cudaError_t launch_vcycle(const ProbDev *p, int level, int levels, int N, int nb, const double *J, const double *R,
+                          double *dU, const nswe_params &prm, int *status, cudaStream_t s) {
+  return vcycle_t<double>(p, level, levels, N, nb, J, R, dU, prm, status, s);
+}
+
+cudaError_t launch_vcycle_f32(const ProbDev *p, int level, int levels, int N, int nb, const float *J, const float *R,
+                              float *dU, const nswe_params &prm, int *status, cudaStream_t s) {
+  return vcycle_t<float>(p, level, levels, N, nb, J, R, dU, prm, status, s);
 }
 
 cudaError_t launch_solve(const SolveTask *tasks, int count, const nswe_params &prm, int max_coarse_cells,
