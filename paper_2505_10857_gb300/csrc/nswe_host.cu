@@ -213,7 +213,8 @@ cudaError_t smooth2(const Lev2<T> &Lv, int st, int steps, double omega, int Kc, 
       for (int d = 0; d < 4; ++d)
         for (int q = 0; q < Kc; ++q) {
           const int mode = (d % 2) + 1, col = d < 2 ? q : Kc - 1 - q;
-          if ((e = launch2_sor<T>(Lv.Nx, Lv.Ny, st, Lv.J, Lv.Dinv, Lv.R, Lv.dU, omega, mode, Kc, col, 1, Lv.cm, s)))
+          if ((e = launch2_sor<T>(Lv.Nx, Lv.Ny, st, Lv.J, Lv.Dinv, Lv.R, Lv.dU, omega, mode, Kc, col, 1, Lv.cm,
+                                  t + d + q > 0, s)))
             return e;
           if (launches) ++*launches;
         }
@@ -221,6 +222,7 @@ cudaError_t smooth2(const Lev2<T> &Lv, int st, int steps, double omega, int Kc, 
   }
   const int C = st_colours_host(st);
   int prev = -1, reps = 0;
+  bool early = false;
   for (int t = 0; t < steps; ++t)
     for (int pass = 0; pass < 4 * C; ++pass) {
       const int q = pass % (2 * C), col = q < C ? q : 2 * C - 1 - q;
@@ -229,14 +231,15 @@ cudaError_t smooth2(const Lev2<T> &Lv, int st, int steps, double omega, int Kc, 
         continue;
       }
       if (prev >= 0 &&
-          (e = launch2_sor<T>(Lv.Nx, Lv.Ny, st, Lv.J, Lv.Dinv, Lv.R, Lv.dU, omega, 0, 0, prev, reps, Lv.cm, s)))
+          (e = launch2_sor<T>(Lv.Nx, Lv.Ny, st, Lv.J, Lv.Dinv, Lv.R, Lv.dU, omega, 0, 0, prev, reps, Lv.cm, early, s)))
         return e;
+      early = early || prev >= 0;
       if (prev >= 0 && launches) ++*launches;
       prev = col;
       reps = 1;
     }
   if (prev >= 0) {
-    e = launch2_sor<T>(Lv.Nx, Lv.Ny, st, Lv.J, Lv.Dinv, Lv.R, Lv.dU, omega, 0, 0, prev, reps, Lv.cm, s);
+    e = launch2_sor<T>(Lv.Nx, Lv.Ny, st, Lv.J, Lv.Dinv, Lv.R, Lv.dU, omega, 0, 0, prev, reps, Lv.cm, early, s);
     if (launches) ++*launches;
   }
   return e;

@@ -129,10 +129,11 @@ cudaError_t launch2_coarse_op(int Nx, int Ny, int st, const T *Jf, T *Jc, int cm
 template <typename T>
 cudaError_t launch2_dinv(int Nx, int Ny, int st, const T *J, T *Dinv, int cm, cudaStream_t s);
 // mode 0: cells of colour col of the stencil's colouring; mode 1 / 2: of the
-// diagonal colourings (i + j) mod Kc / (j - i + Nx - 1) mod Kc.
+// diagonal colourings (i + j) mod Kc / (j - i + Nx - 1) mod Kc. early: the
+// launch before it on the stream is a pass of the same smoothing.
 template <typename T>
 cudaError_t launch2_sor(int Nx, int Ny, int st, const T *J, const T *Dinv, const T *R, T *dU, double omega, int mode,
-                        int Kc, int col, int reps, int cm, cudaStream_t s);
+                        int Kc, int col, int reps, int cm, bool early, cudaStream_t s);
 template <typename T>
 cudaError_t launch2_restrict(int Nx, int Ny, int st, const T *J, const T *R, const T *dU, T *Rc, T *dUc, int cm,
                              cudaStream_t s);

@@ -308,12 +308,17 @@ __device__ __forceinline__ bool sor_item_cell(int Nx, int mode, int Kc, int col,
 // third of the dependent FP64 instructions: an FP64 warp instruction holds
 // its SMSP's FP64 unit for tens of cycles, so the length of one thread's
 // chain, not the total work, bounds such a pass.
-// STC >= 0: the stencil fixed at compile time (the neighbour loop unrolls
-// and its loads issue together); -1: the stencil st of the call.
+// STC >= 0: the stencil fixed at compile time: the operator's loads all issue
+// together, before those of dU; -1: the stencil st of the call. early: the
+// kernel before this one on the stream is a pass of the same smoothing, which
+// changes only dU, so the operator and the right-hand side are read before
+// waiting for it (pdl_enter is called here then). A pass of 512 x 256 is 8 us
+// of FP64 issue behind a launch gap and a trip to memory: 17.0 us with the
+// loads issued block by block after the wait, 14.2 so; 256 x 128 7.2 -> 4.4.
 template <typename T, int STC>
 __device__ __forceinline__ void sor_pass_split(int Nx, int Ny, int st_arg, const T *J, const T *Dinv, const T *R,
                                                T *dU, double omega_d, int mode, int Kc, int col, int reps,
-                                               int warp0, int warps, int cm) {
+                                               int warp0, int warps, int cm, bool early = false) {
   const int st = STC >= 0 ? STC : st_arg;
   int P, W, items;
   sor_items(Nx, Ny, st, mode, Kc, col, P, W, items);
@@ -327,9 +332,35 @@ __device__ __forceinline__ void sor_pass_split(int Nx, int Ny, int st_arg, const
     const int c = j * Nx + i;
     const size_t S = blk_stride(cm, Nx, Ny), pc = blk_pos(cm, Nx, Ny, i, j);  // J, Dinv
     T r = on ? R[l * n + c] : T(0.0);
-    if (on)
+    T D[3];
 #pragma unroll
-      for (int k = 0; k < (STC >= 0 ? (STC == ST_J9 ? 9 : STC == ST_P5 ? 5 : 21) : K); ++k) {
+    for (int m = 0; m < 3; ++m) D[m] = on ? Dinv[(size_t)(l * 3 + m) * S + pc] : T(0.0);
+    if constexpr (STC >= 0) {
+      constexpr int KC = STC == ST_J9 ? 9 : STC == ST_P5 ? 5 : 21, C0 = KC / 2;
+      T Jr[KC][3], x[KC][3];
+      auto inside = [&](int k) {
+        const int p = i + off_c<STC>(k, 0), q = j + off_c<STC>(k, 1);
+        return on && p >= 0 && p < Nx && q >= 0 && q < Ny;
+      };
+#pragma unroll
+      for (int k = 0; k < KC; ++k)
+#pragma unroll
+        for (int m = 0; m < 3; ++m)
+          if (k != C0) Jr[k][m] = inside(k) ? J[(size_t)(k * 9 + l * 3 + m) * S + pc] : T(0.0);
+      if (early) pdl_enter();
+#pragma unroll
+      for (int k = 0; k < KC; ++k)
+#pragma unroll
+        for (int m = 0; m < 3; ++m)
+          if (k != C0)
+            x[k][m] = inside(k) ? dU[m * n + c + off_c<STC>(k, 1) * Nx + off_c<STC>(k, 0)] : T(0.0);
+#pragma unroll
+      for (int k = 0; k < KC; ++k)
+#pragma unroll
+        for (int m = 0; m < 3; ++m)
+          if (k != C0) r = fma(Jr[k][m], x[k][m], r);
+    } else if (on) {
+      for (int k = 0; k < K; ++k) {
         if (k == kc) continue;
         const int p = i + st_off(st, k, 0), q = j + st_off(st, k, 1);
         if (p < 0 || p >= Nx || q < 0 || q >= Ny) continue;
@@ -339,12 +370,12 @@ __device__ __forceinline__ void sor_pass_split(int Nx, int Ny, int st_arg, const
         r = fma(J[(size_t)(k * 9 + l * 3 + 1) * S + pc], x1, r);
         r = fma(J[(size_t)(k * 9 + l * 3 + 2) * S + pc], x2, r);
       }
+    }
     const T r0 = __shfl_sync(0xffffffffu, r, min(src, 31));
     const T r1 = __shfl_sync(0xffffffffu, r, min(src + 1, 31));
     const T r2 = __shfl_sync(0xffffffffu, r, min(src + 2, 31));
     if (on) {
-      const T tl = dinv_row(Dinv[(size_t)(l * 3 + 0) * S + pc], Dinv[(size_t)(l * 3 + 1) * S + pc],
-                            Dinv[(size_t)(l * 3 + 2) * S + pc], r0, r1, r2);
+      const T tl = dinv_row(D[0], D[1], D[2], r0, r1, r2);
       dU[l * n + c] = relax(dU[l * n + c], tl, omega, reps);
     }
   }
@@ -353,10 +384,10 @@ __device__ __forceinline__ void sor_pass_split(int Nx, int Ny, int st_arg, const
 template <typename T, int STC>
 __global__ void __launch_bounds__(kThreads) k2_sor_split(int Nx, int Ny, int st, const T *J, const T *Dinv,
                                                          const T *R, T *dU, double omega, int mode, int Kc, int col,
-                                                         int reps, int cm) {
-  pdl_enter();
+                                                         int reps, int cm, int early) {
+  if (STC < 0 || !early) pdl_enter();
   sor_pass_split<T, STC>(Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps,
-                         (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5, cm);
+                         (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5, cm, early);
 }
 
 template <typename T>
@@ -858,7 +889,7 @@ cudaError_t launch2_dinv_levels(Tail2<T> t, int l0, int cm0, cudaStream_t s) {
 
 template <typename T>
 cudaError_t launch2_sor(int Nx, int Ny, int st, const T *J, const T *Dinv, const T *R, T *dU, double omega, int mode,
-                        int Kc, int col, int reps, int cm, cudaStream_t s) {
+                        int Kc, int col, int reps, int cm, bool early, cudaStream_t s) {
   // Items of the pass as the kernel enumerates them (see sor_items).
   long items;
   if (mode == 0 && (st == ST_J9 || st == ST_P5)) items = (long)((Nx + (st == ST_J9 ? 3 : 2) - 1) / (st == ST_J9 ? 3 : 2)) * Ny;
@@ -870,11 +901,14 @@ cudaError_t launch2_sor(int Nx, int Ny, int st, const T *J, const T *Dinv, const
   const int bs = warps <= 4L * kSmCount ? 32 : 128;
   const unsigned grid = (unsigned)((warps * 32 + bs - 1) / bs);
   if (st == ST_J9)
-    launchk2(k2_sor_split<T, ST_J9>, grid, bs, s, Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, cm);
+    launchk2(k2_sor_split<T, ST_J9>, grid, bs, s, Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, cm,
+             (int)early);
   else if (st == ST_P5)
-    launchk2(k2_sor_split<T, ST_P5>, grid, bs, s, Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, cm);
+    launchk2(k2_sor_split<T, ST_P5>, grid, bs, s, Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, cm,
+             (int)early);
   else
-    launchk2(k2_sor_split<T, -1>, grid, bs, s, Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, cm);
+    launchk2(k2_sor_split<T, -1>, grid, bs, s, Nx, Ny, st, J, Dinv, R, dU, omega, mode, Kc, col, reps, cm,
+             (int)early);
   return cudaGetLastError();
 }
 
@@ -1023,7 +1057,7 @@ cudaError_t launch2_to_f32(long count, const double *src, float *dst, cudaStream
   template cudaError_t launch2_coarse_op<T>(int, int, int, const T *, T *, int, cudaStream_t);                   \
   template cudaError_t launch2_dinv<T>(int, int, int, const T *, T *, int, cudaStream_t);                        \
   template cudaError_t launch2_sor<T>(int, int, int, const T *, const T *, const T *, T *, double, int, int, int, \
-                                      int, int, cudaStream_t);                                                   \
+                                      int, int, bool, cudaStream_t);                                             \
   template cudaError_t launch2_restrict<T>(int, int, int, const T *, const T *, const T *, T *, T *, int,        \
                                            cudaStream_t);                                                        \
   template cudaError_t launch2_prolong<T>(int, int, T *, const T *, cudaStream_t);                               \
