@@ -1498,7 +1498,8 @@ __device__ void mg_vcycle(const MG<T> &mg, const Band<T> &B, const nswe_params &
   }
 }
 
-// Algorithm 2 from level ls >= l0 by a cluster. Levels that can be take legs
+// Algorithm 2 from level ls >= l0 with legs: by a cluster, or by one block in
+// FP32, whose pipe does not bound the smoothing. Levels that can be take legs
 // (leg_level), the others (the full Jacobian's own level, more than two
 // smoothing steps) go pass by pass. The levels of at most a tile per warp of a
 // block, and of less than team_cells cells where they go pass by pass, run on
@@ -1506,15 +1507,16 @@ __device__ void mg_vcycle(const MG<T> &mg, const Band<T> &B, const nswe_params &
 // correction of level l0, on return and (unless zero) on entry; for a level
 // smoothed by passes it is mg.dU[l0]. ready: called by the leader before the
 // coarsest solve.
-template <typename T, typename F>
-__device__ void mg_vcycle_cluster(const MG<T> &mg, const Band<T> &B, const nswe_params &prm, bool zero, T *out0,
-                                  const ClusterTeam &team, int team_cells, int ls, F &&ready) {
+template <typename T, class TM, typename F>
+__device__ void mg_vcycle_legs(const MG<T> &mg, const Band<T> &B, const nswe_params &prm, bool zero, T *out0,
+                               const TM &team, int team_cells, int ls, F &&ready) {
   const int nw = (int)blockDim.x >> 5;
   auto lead_level = [&](int l) {
     return leg_level(mg.nb[l], prm) ? leg_tiles(mg.N[l]) <= nw : mg.N[l] < team_cells;
   };
   int lt = ls;
-  while (lt < mg.L && !lead_level(lt)) ++lt;
+  if constexpr (TM::kMulti)
+    while (lt < mg.L && !lead_level(lt)) ++lt;
   auto out = [&](int l) {
     return l == mg.l0 ? out0 : l < mg.L && leg_level(mg.nb[l], prm) ? leg_out(mg.J[l], mg.N[l]) : mg.dU[l];
   };
@@ -1541,15 +1543,18 @@ __device__ void mg_vcycle_cluster(const MG<T> &mg, const Band<T> &B, const nswe_
     tm.sync();
     sor_smooth(mg, l, prm.nu2, prm.omega, false, tm);
   };
-  for (int l = ls; l < lt; ++l) down(l, team);
+  if constexpr (TM::kMulti)
+    for (int l = ls; l < lt; ++l) down(l, team);
   if (team.lead()) {
     for (int l = lt; l < mg.L; ++l) down(l, BlockTeam());
     ready();
     band_solve(B, mg.N[mg.L], mg.R[mg.L], mg.dU[mg.L]);
     for (int l = mg.L - 1; l >= lt; --l) up(l, BlockTeam());
   }
-  team.sync();
-  for (int l = lt - 1; l >= ls; --l) up(l, team);
+  if constexpr (TM::kMulti) {
+    team.sync();
+    for (int l = lt - 1; l >= ls; --l) up(l, team);
+  }
 }
 
 // Band storage in dynamic shared memory, sized by the host for the coarsest
@@ -1737,7 +1742,7 @@ __global__ void __launch_bounds__(kVcThreads, 1)
   B.n = 2 * mg.N[mg.L];
   B.kl = 3;
   B.ldab = 10;
-  mg_vcycle_cluster<T>(mg, B, prm, false, dU, team, 0, ls, [&] {
+  mg_vcycle_legs<T>(mg, B, prm, false, dU, team, 0, ls, [&] {
     asm volatile("griddepcontrol.wait;" ::: "memory");  // the factors are there
     const T *ab = reinterpret_cast<const T *>(P->jw), *rinv = ab + (size_t)B.ldab * B.n;
     const int *piv = reinterpret_cast<const int *>(rinv + B.n);
@@ -1909,14 +1914,14 @@ __global__ void __launch_bounds__(THREADS, MINB)
       if (l == L) {
         if (team.lead()) band_solve<T>(B, N, Rs, dU);
         if constexpr (TM::kMulti) team.sync();
-      } else if constexpr (TM::kMulti) {
+      } else if constexpr (TM::kMulti || kMixed) {
         if (leg_level(nb, prm)) x = leg_out(J, N);
         if (!leg_level(nb, prm) || prm.nu3 < 1) {
           for (int t = team.tid(); t < 2 * N; t += team.size()) x[t] = T(0.0);
           team.sync();
         }
         for (int m = 0; m < prm.nu3; ++m) {
-          mg_vcycle_cluster<T>(mg, B, prm, m == 0, x, team, team_cells, l, [] {});
+          mg_vcycle_legs<T, TM>(mg, B, prm, m == 0, x, team, team_cells, l, [] {});
           ++vcycles;
         }
       } else {
@@ -2172,6 +2177,12 @@ cudaError_t launch_solve_sized(const SolveTask *tasks, int count, const nswe_par
     launch_shape<0, NSWE_FLUX_LLF>(tasks, count, prm, n_cap, ldab_cap, smem, s);
     return cudaGetLastError();
   }
+  // Up to two problems per SM take the default 256 threads with 128 registers
+  // each (shape 2) instead of the 64, with spills, that four blocks per SM
+  // allow. With the legs of the mixed block form: 304 uneven mixed problems
+  // 185 -> 114 ms, 100 of 2048 cells 91 -> 56, one of 4096 108 -> 68 (FP64 219
+  // -> 191); beyond two per SM the legs alone, 608 of 4096 cells 195 -> 159.
+  if (shape == 0 && count <= 2 * kSmCount) shape = 2;
   switch (shape) {
   case 1: launch_shape<1>(tasks, count, prm, n_cap, ldab_cap, smem, s); break;
   case 2: launch_shape<2>(tasks, count, prm, n_cap, ldab_cap, smem, s); break;

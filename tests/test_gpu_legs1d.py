@@ -77,3 +77,25 @@ def test_residual_at_tile_edges(nswe, ctx, N, levels):
     assert np.abs(dR.cpu().numpy() - Rref).max() <= 1e-12 * sc
     assert abs(float(res) - resref) <= 1e-12 * max(resref, sc * 1e-3)
     prob.close()
+
+
+@pytest.mark.parametrize("precision,bound", [(0, 1e-13), (1, 1e-8)])
+@pytest.mark.parametrize("count", [304, 305])
+def test_batches_around_two_problems_per_sm(nswe, ctx, precision, bound, count):
+    """The default launch shape's two register budgets: the same solve, to the
+    compiler's choice of fused multiply-adds (bounds of the cluster form's test)."""
+    inps = [I.channel_small(k % 3, N=128, levels=3) for k in range(count)]
+    prm = nswe.params_from(I.Params1D.for_problem(inps[0], tol=1e-10, n_max=500))
+    prm.precision = precision
+    probs = [nswe.Problem1D.from_inputs(ctx, p) for p in inps]
+    U0s = [dev(p.U0_start) for p in inps]
+    Us = [torch.zeros((2, 128), dtype=torch.float64, device="cuda") for _ in inps]
+    infos = nswe.nswe_newton_solve_batch(ctx, probs, U0s, Us, prm)
+    one = torch.zeros_like(Us[0])
+    for k in range(3):
+        info = nswe.nswe_newton_solve(ctx, probs[k], U0s[k], one, prm)
+        assert info["status"] == 0 and all(infos[i]["status"] == 0 for i in range(k, count, 3))
+        for i in range(k, count, 3):
+            assert float((Us[i] - one).abs().max()) <= bound * float(one.abs().max())
+    for p in probs:
+        p.close()
