@@ -982,15 +982,15 @@ __device__ __forceinline__ unsigned long long abs_key(float a) {
   return a == a ? (unsigned long long)(__float_as_uint(a) & 0x7fffffffu) : 0ull;
 }
 
-// Factorisation by warp 0 (lanes 0..31, all of them calling). Returns true if
-// a pivot was exactly zero.
+// Pivot steps k0 .. k1 - 1 of the factorisation by warp 0 (lanes 0..31, all of
+// them calling). Returns true if a pivot was exactly zero.
 template <typename T>
-__device__ bool band_lu_warp(const Band<T> &B) {
+__device__ bool band_lu_warp(const Band<T> &B, int k0, int k1) {
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int n = B.n, kl = B.kl, w2 = 2 * kl, upd = kl * w2;
   bool sing = false;
-  for (int k = 0; k < n; ++k) {
+  for (int k = k0; k < k1; ++k) {
     const int imax = min(n - 1, k + kl), cmax = min(n - 1, k + w2);
     // Pivot: the first row of largest |A(i, k)|, i = k..imax (kl <= 7).
     unsigned long long key = 0;
@@ -1205,18 +1205,17 @@ __device__ void band_lu_solve_serial(const Band<T> &B) {
   }
 }
 
-// Assemble the band matrix from J (all threads), then factor (warp 0 in
-// FP64, thread 0 in FP32). Returns true if a pivot was exactly zero (all
-// threads).
 __shared__ int s_sing;
 
+// Assemble the band matrix from J (all threads).
 template <typename T>
-__device__ bool band_factor(Band<T> &B, int N, int nb, const T *J) {
+__device__ void band_assemble(Band<T> &B, int N, int nb, const T *J) {
   const int hw = (nb - 1) / 2;
   B.n = 2 * N;
   B.kl = 2 * hw + 1;
   B.ldab = 3 * B.kl + 1;
   const int n = B.n;
+  if (threadIdx.x == 0) s_sing = 0;
   for (int t = threadIdx.x; t < B.ldab * n; t += blockDim.x) B.ab[t] = T(0.0);
   __syncthreads();
   for (int t = threadIdx.x; t < N * nb * 4; t += blockDim.x) {
@@ -1226,14 +1225,30 @@ __device__ bool band_factor(Band<T> &B, int N, int nb, const T *J) {
     B.A(2 * j + l, 2 * i + m) = J[(k * 4 + e) * N + j];
   }
   __syncthreads();
+}
+
+// Pivot steps k0 .. k1 - 1 of the assembled matrix by the calling warp (in
+// FP32 its first thread runs all of them with the first). Sets s_sing if a
+// pivot was exactly zero.
+template <typename T>
+__device__ void band_lu_steps(const Band<T> &B, int k0, int k1) {
+  bool sing = false;
   if constexpr (std::is_same<T, double>::value) {
-    if (threadIdx.x < 32) {
-      const bool sing = band_lu_warp<T>(B);
-      if (threadIdx.x == 0) s_sing = sing ? 1 : 0;
-    }
+    sing = band_lu_warp<T>(B, k0, k1);
   } else {
-    if (threadIdx.x == 0) s_sing = (B.kl == 3 ? band_lu_serial<3, T>(B) : band_lu_serial_smem<T>(B)) ? 1 : 0;
+    if (k0 == 0 && k1 > 0 && (threadIdx.x & 31) == 0)
+      sing = B.kl == 3 ? band_lu_serial<3, T>(B) : band_lu_serial_smem<T>(B);
+    __syncwarp();
   }
+  if (sing && (threadIdx.x & 31) == 0) s_sing = 1;
+}
+
+// Assemble (all threads), then factor (warp 0). Returns true if a pivot was
+// exactly zero (all threads).
+template <typename T>
+__device__ bool band_factor(Band<T> &B, int N, int nb, const T *J) {
+  band_assemble(B, N, nb, J);
+  if (threadIdx.x < 32) band_lu_steps(B, 0, B.n);
   __syncthreads();
   return s_sing != 0;
 }
@@ -1430,12 +1445,17 @@ __device__ void mg_setup_part(const MG<T> &mg, double omega, int part, int parts
 
 // Coarse operators, diagonal inverses and the coarsest factorisation; done
 // once per Newton step since J is fixed during its V-cycles. Returns whether
-// a pivot was exactly zero, in every thread of the team.
+// a pivot was exactly zero, in every thread of the team. A cluster may leave
+// the pivot steps to the first V-cycle (later): false is returned then.
 template <typename T, class TM = BlockTeam>
-__device__ bool mg_setup(const MG<T> &mg, Band<T> &B, double omega, const TM &team = TM()) {
+__device__ bool mg_setup(const MG<T> &mg, Band<T> &B, double omega, const TM &team = TM(), bool later = false) {
   if constexpr (TM::kMulti) {
     mg_setup_part(mg, omega, team.rank, team.n);
     team.sync();
+    if (later) {
+      if (team.lead()) band_assemble(B, mg.N[mg.L], mg.nb[mg.L], mg.J[mg.L]);
+      return false;
+    }
     if (team.lead()) band_factor(B, mg.N[mg.L], mg.nb[mg.L], mg.J[mg.L]);
     team.sync();  // the leader's factors and flag are done
     return team.lead_value(&s_sing) != 0;
@@ -1506,10 +1526,14 @@ __device__ void mg_vcycle(const MG<T> &mg, const Band<T> &B, const nswe_params &
 // the leader CTA with block barriers, and the coarsest solve. out0: the
 // correction of level l0, on return and (unless zero) on entry; for a level
 // smoothed by passes it is mg.dU[l0]. ready: called by the leader before the
-// coarsest solve.
+// coarsest solve. factor: the coarsest matrix is assembled but not factored:
+// while the cluster runs the legs on the way down, the leader's first warp
+// takes the pivot steps in their place, as many beside each leg as it is long
+// (a chain of 2 N_L steps of 900 cycles each, otherwise waited for: a
+// 4096-cell solve on 16 CTAs 69.4 -> 52.6 ms).
 template <typename T, class TM, typename F>
 __device__ void mg_vcycle_legs(const MG<T> &mg, const Band<T> &B, const nswe_params &prm, bool zero, T *out0,
-                               const TM &team, int team_cells, int ls, F &&ready) {
+                               const TM &team, int team_cells, int ls, bool factor, F &&ready) {
   const int nw = (int)blockDim.x >> 5;
   auto lead_level = [&](int l) {
     return leg_level(mg.nb[l], prm) ? leg_tiles(mg.N[l]) <= nw : mg.N[l] < team_cells;
@@ -1517,13 +1541,29 @@ __device__ void mg_vcycle_legs(const MG<T> &mg, const Band<T> &B, const nswe_par
   int lt = ls;
   if constexpr (TM::kMulti)
     while (lt < mg.L && !lead_level(lt)) ++lt;
+  int rounds = 0, done = 0, pivots = 0;  // legs' rounds of tiles: of all levels, so far; pivot steps taken
+  const int lu_warps = factor ? 1 : 0;
+  auto leg_rounds = [&](int l) {
+    const int w = (team.size() >> 5) - lu_warps;
+    return leg_level(mg.nb[l], prm) ? (leg_tiles(mg.N[l]) + w - 1) / w : 0;
+  };
+  if (factor)
+    for (int l = ls; l < lt; ++l) rounds += leg_rounds(l);
   auto out = [&](int l) {
     return l == mg.l0 ? out0 : l < mg.L && leg_level(mg.nb[l], prm) ? leg_out(mg.J[l], mg.N[l]) : mg.dU[l];
   };
   auto down = [&](int l, const auto &tm) {
     if (leg_level(mg.nb[l], prm)) {
-      leg<T, false>(mg.N[l], mg.J[l], mg.Dinv[l], mg.R[l], l > mg.l0 || zero ? nullptr : out0, mg.dU[l], nullptr,
-                    mg.R[l + 1], prm.nu1, prm.omega, tm.tid() >> 5, tm.size() >> 5);
+      const int skip = l < lt ? lu_warps : 0, warp = (tm.tid() >> 5) - skip;
+      if (skip) {
+        done += leg_rounds(l);
+        const int k = 2 * mg.N[mg.L] * done / rounds;
+        if (warp < 0) band_lu_steps(B, pivots, k);
+        pivots = k;
+      }
+      if (warp >= 0)
+        leg<T, false>(mg.N[l], mg.J[l], mg.Dinv[l], mg.R[l], l > mg.l0 || zero ? nullptr : out0, mg.dU[l], nullptr,
+                      mg.R[l + 1], prm.nu1, prm.omega, warp, (tm.size() >> 5) - skip);
       tm.sync();
       return;
     }
@@ -1548,6 +1588,10 @@ __device__ void mg_vcycle_legs(const MG<T> &mg, const Band<T> &B, const nswe_par
   if (team.lead()) {
     for (int l = lt; l < mg.L; ++l) down(l, BlockTeam());
     ready();
+    if (factor && pivots < B.n) {
+      if (threadIdx.x < 32) band_lu_steps(B, pivots, B.n);
+      __syncthreads();
+    }
     band_solve(B, mg.N[mg.L], mg.R[mg.L], mg.dU[mg.L]);
     for (int l = mg.L - 1; l >= lt; --l) up(l, BlockTeam());
   }
@@ -1742,7 +1786,7 @@ __global__ void __launch_bounds__(kVcThreads, 1)
   B.n = 2 * mg.N[mg.L];
   B.kl = 3;
   B.ldab = 10;
-  mg_vcycle_legs<T>(mg, B, prm, false, dU, team, 0, ls, [&] {
+  mg_vcycle_legs<T>(mg, B, prm, false, dU, team, 0, ls, false, [&] {
     asm volatile("griddepcontrol.wait;" ::: "memory");  // the factors are there
     const T *ab = reinterpret_cast<const T *>(P->jw), *rinv = ab + (size_t)B.ldab * B.n;
     const int *piv = reinterpret_cast<const int *>(rinv + B.n);
@@ -1904,8 +1948,10 @@ __global__ void __launch_bounds__(THREADS, MINB)
       }
       MG<T> mg;
       mg_bind<T>(mg, P, l, nb, J, Rs, dU);
-      bool sing = mg_setup<T, TM>(mg, B, prm.omega, team);
-      team.sync();
+      // (a cluster factors the coarsest system beside its first V-cycle)
+      const bool later = TM::kMulti && l < L && prm.nu3 >= 1;
+      bool sing = mg_setup<T, TM>(mg, B, prm.omega, team, later);
+      if (!later) team.sync();
       if (sing) {
         st = NSWE_ESINGULAR;
         break;
@@ -1921,8 +1967,14 @@ __global__ void __launch_bounds__(THREADS, MINB)
           team.sync();
         }
         for (int m = 0; m < prm.nu3; ++m) {
-          mg_vcycle_legs<T, TM>(mg, B, prm, m == 0, x, team, team_cells, l, [] {});
+          mg_vcycle_legs<T, TM>(mg, B, prm, m == 0, x, team, team_cells, l, later && m == 0, [] {});
+          if constexpr (TM::kMulti)
+            if (m == 0 && (sing = team.lead_value(&s_sing) != 0)) break;
           ++vcycles;
+        }
+        if (sing) {
+          st = NSWE_ESINGULAR;
+          break;
         }
       } else {
         for (int t = team.tid(); t < 2 * N; t += team.size()) dU[t] = T(0.0);
