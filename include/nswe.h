@@ -178,8 +178,9 @@ nswe_status nswe_ctx_set_stream(nswe_ctx ctx, void *stream);
  * inverses colour-major, each colour (i + j) mod 3 of the smoother one
  * contiguous plane, so that a colour pass reads only its third of J.
  * min_cells < 0: never. Default 131072 (512 x 256). The standalone calls
- * (nswe_jacobian_*, nswe_mg_vcycle*) always use the cell-contiguous layout
- * they document. */
+ * (nswe_jacobian_*, nswe_mg_vcycle*) always take and return the
+ * cell-contiguous layout they document; a V-cycle on a level of that size
+ * copies its J9 to the other first. */
 nswe_status nswe_ctx_set_colour_major_2d(nswe_ctx ctx, int min_cells);
 /* Formerly the level size from which the 2D FD Jacobian (Eq. 12) took one
  * cell per thread. One kernel now serves every level size; any value is

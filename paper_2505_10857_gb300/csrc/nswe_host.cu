@@ -546,7 +546,19 @@ nswe_status vcycle2d_entry(nswe_ctx ctx, nswe_prob prob, int level, int nb, cons
   long tail;
   resolve2d(prob, prm_in, prm, tail);
   tail = ctx->tail2[std::is_same<T, float>::value ? 1 : 0];  // the standalone call's own precision
-  MG2<T> m = mg2_bind<T>(prob, level, nb == 21 ? ST_J21 : ST_J9, J, R, dU, 0);
+  const int st = nb == 21 ? ST_J21 : ST_J9, Nx = prob->Nx >> level, Ny = prob->Ny >> level;
+  const int minc = ctx->cm2d_min_cells;
+  // A large level's J9 goes colour-major into the level's own (unused) storage
+  // first: a colour pass then reads a third of it instead of every sector
+  // (512 x 256: 12.6 us instead of 14.2, the V-cycle 6.51 -> 6.16 ms).
+  const bool cm = level < prob->levels - 1 && st == ST_J9 && minc >= 0 && (long)Nx * Ny >= minc &&
+                  tail2_first<T>(prob, level, st, tail, kTail2MaxCtas) > level;
+  if (cm) {
+    T *const Jcm = reinterpret_cast<T *>(prob->host2.lev[level].J);
+    if (launch2_colour_major<T>(Nx, Ny, J, Jcm, ctx->stream) != cudaSuccess) return NSWE_ECUDA;
+    J = Jcm;
+  }
+  MG2<T> m = mg2_bind<T>(prob, level, st, J, R, dU, cm ? 1 : 0);
   cudaMemsetAsync(prob->flag, 0, sizeof(int), ctx->stream);
   if (level == prob->levels - 1) {
     const int n = nswe_prob_cells(prob, level);

@@ -139,6 +139,9 @@ cudaError_t launch2_restrict(int Nx, int Ny, int st, const T *J, const T *R, con
                              cudaStream_t s);
 template <typename T>
 cudaError_t launch2_prolong(int Nx, int Ny, T *dU, const T *dUc, cudaStream_t s);
+// J9 of a level from cell-contiguous to colour-major storage (blk_pos).
+template <typename T>
+cudaError_t launch2_colour_major(int Nx, int Ny, const T *J, T *Jcm, cudaStream_t s);
 template <typename T>
 cudaError_t launch2_dense_factor(int Nx, int Ny, int st, const T *J, T *A, int *piv, int *flag, cudaStream_t s);
 template <typename T>

@@ -452,6 +452,22 @@ __global__ void __launch_bounds__(kThreads) k2_prolong(int Nx, int Ny, T *dU, co
 
 // Dense system A (row-major, unknown 3c+m) assembled from a block operator:
 // zero it, then scatter the blocks.
+// A cell-contiguous J9 (81 planes) in colour-major storage. Items run along
+// the destination's rows (plane, colour, row j, slot), so writes coalesce; the
+// reads of a row's three colours share their sectors through L2.
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k2_colour_major(int Nx, int Ny, const T *J, T *Jcm) {
+  pdl_enter();
+  const int W = (Nx + 2) / 3;
+  const long S = 3L * Ny * W, count = 81 * S;
+  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < count; t += (long)gridDim.x * blockDim.x) {
+    const long pl = t / S;
+    const int r = (int)(t - pl * S), slot = r % W, cj = r / W, j = cj % Ny, c = cj / Ny;
+    const int i = 3 * slot + (c - j % 3 + 3) % 3;
+    if (i < Nx) Jcm[t] = J[pl * Nx * Ny + (long)j * Nx + i];
+  }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k2_zero(long count, T *A) {
   pdl_enter();
@@ -925,6 +941,12 @@ cudaError_t launch2_prolong(int Nx, int Ny, T *dU, const T *dUc, cudaStream_t s)
   return cudaGetLastError();
 }
 
+template <typename T>
+cudaError_t launch2_colour_major(int Nx, int Ny, const T *J, T *Jcm, cudaStream_t s) {
+  launchk2(k2_colour_major<T>, grid2(81 * (long)blk_stride(1, Nx, Ny)), kThreads, s, Nx, Ny, J, Jcm);
+  return cudaGetLastError();
+}
+
 // Shared memory of the factorisation of an N3 x N3 system (0: too large for it).
 template <typename T>
 size_t lu2_smem(int N3) {
@@ -1061,6 +1083,7 @@ cudaError_t launch2_to_f32(long count, const double *src, float *dst, cudaStream
   template cudaError_t launch2_restrict<T>(int, int, int, const T *, const T *, const T *, T *, T *, int,        \
                                            cudaStream_t);                                                        \
   template cudaError_t launch2_prolong<T>(int, int, T *, const T *, cudaStream_t);                               \
+  template cudaError_t launch2_colour_major<T>(int, int, const T *, T *, cudaStream_t);                          \
   template cudaError_t launch2_dense_factor<T>(int, int, int, const T *, T *, int *, int *, cudaStream_t);       \
   template cudaError_t launch2_dense_solve<T>(int, const T *, const int *, const T *, T *, cudaStream_t);         \
   template cudaError_t launch2_dinv_levels<T>(Tail2<T>, int, int, cudaStream_t);                                 \
