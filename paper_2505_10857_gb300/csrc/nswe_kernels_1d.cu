@@ -376,7 +376,7 @@ __device__ double block_sum(double v, double *red) {
 // one problem per cluster): the per-cell loops of a phase are strided over
 // all its threads, phases are separated by cluster barriers (release /
 // acquire at cluster scope, so the global writes of one phase are visible to
-// every CTA in the next), and the coarse levels and the coarsest LU run on
+// every CTA in the next), and the smallest levels and the coarsest LU run on
 // the leader CTA alone with block barriers. Every cluster barrier is reached
 // by all threads of the cluster: the branches around them depend only on
 // values that are the same in every CTA (sizes, and res, flags and counters
@@ -1853,8 +1853,8 @@ __device__ __forceinline__ ClusterTeam make_team<ClusterTeam>(int &task_index) {
 // while the FD Jacobian (Eq. 12-13), the coarse operators, the smoother and
 // the coarsest LU run in FP32. FLUX: the numerical flux of every task of the
 // launch (compile-time, so that the HLL kernels carry no LLF code).
-// team_cells: a cluster team runs the multigrid levels with at least that
-// many cells on all its CTAs, the others on the leader CTA.
+// team_cells: of the levels smoothed pass by pass, a cluster team runs those
+// with at least that many cells on all its CTAs, the others on the leader CTA.
 template <typename T, int THREADS, int MINB, int FLUX, class TM = BlockTeam>
 __global__ void __launch_bounds__(THREADS, MINB)
     k_solve(const SolveTask *tasks, nswe_params launch_prm, int n_cap, int ldab_cap, int team_cells) {
