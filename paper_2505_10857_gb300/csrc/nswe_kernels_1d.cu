@@ -22,6 +22,16 @@ namespace {
 
 constexpr double kZeta = 1e-6;  // WENO epsilon (Section 3.1)
 
+// Rounded products and sums. Where a sum takes a product that the compiler
+// could fuse into it, or one of two products, the rounding is written out:
+// left to the compiler it differed between the solve kernel's launch shapes
+// (by their register budgets), so that a problem's bits depended on the number
+// of problems launched with it.
+__device__ __forceinline__ double mul_r(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_r(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double add_r(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float add_r(float a, float b) { return __fadd_rn(a, b); }
+
 // Lagrange weights of the cubic through t = -3/2, -1/2, 1/2, 3/2 evaluated at
 // the Gauss points t = -/+ 1/(2 sqrt 3) (Eq. 9). With t^2 = 1/12 the basis
 // reduces to (t - 3/2)/36, -(13/12)(t - 1/2), (13/12)(t + 1/2), -(t + 3/2)/36.
@@ -82,10 +92,10 @@ __device__ __forceinline__ void ghost(int kind, double bh, double bq, double sb,
     H = He;
     Q = bq;
   } else if (kind == NSWE_BC_DEPTH) {
-    H = sb * bh;
+    H = mul_r(sb, bh);
     Q = Qe;
   } else if (kind == NSWE_BC_STATE) {
-    H = sb * bh;
+    H = mul_r(sb, bh);
     Q = bq;
   } else {
     H = He;
@@ -135,14 +145,14 @@ __device__ __forceinline__ void weno3(T a, T b, T c, T &up, T &um) {
 template <>
 __device__ __forceinline__ void weno3<float>(float a, float b, float c, float &up, float &um) {
   float d0 = c - b, d1 = b - a;
-  float e0 = float(kZeta) + d0 * d0, e1 = float(kZeta) + d1 * d1;
-  float s0 = e0 * e0, s1 = e1 * e1;
-  float p0 = 1.5f * b - 0.5f * c, p1 = 0.5f * a + 0.5f * b;   // U^(0), U^(1) at k-1/2
-  float q0 = 0.5f * b + 0.5f * c, q1 = -0.5f * a + 1.5f * b;  // U^(0), U^(1) at k+1/2
-  float D1 = s1 + 2.0f * s0, D2 = 2.0f * s1 + s0;
-  float inv = 1.0f / (D1 * D2);
-  up = (s1 * p0 + 2.0f * s0 * p1) * (D2 * inv);
-  um = (2.0f * s1 * q0 + s0 * q1) * (D1 * inv);
+  float e0 = fmaf(d0, d0, float(kZeta)), e1 = fmaf(d1, d1, float(kZeta));
+  float s0 = mul_r(e0, e0), s1 = mul_r(e1, e1);
+  float p0 = fmaf(1.5f, b, -0.5f * c), p1 = fmaf(0.5f, a, 0.5f * b);  // U^(0), U^(1) at k-1/2
+  float q0 = fmaf(0.5f, b, 0.5f * c), q1 = fmaf(1.5f, b, -0.5f * a);  // U^(0), U^(1) at k+1/2
+  float D1 = fmaf(2.0f, s0, s1), D2 = fmaf(2.0f, s1, s0);
+  float inv = 1.0f / mul_r(D1, D2);
+  up = mul_r(fmaf(s1, p0, mul_r(2.0f * s0, p1)), mul_r(D2, inv));
+  um = mul_r(fmaf(2.0f * s1, q0, mul_r(s0, q1)), mul_r(D1, inv));
 }
 
 // Quantities of one interface state entering the flux at a face of width
@@ -150,25 +160,16 @@ __device__ __forceinline__ void weno3<float>(float a, float b, float c, float &u
 // celerity c = sqrt(g H/sigma), and the physical flux F = (Q, Q^2/H +
 // g H^2/(2 sigma)) (Eq. 4). One reciprocal square root r = H^(-1/2) gives
 // both 1/H = r^2 and c = sqrt(g/sigma) H r; cg = sqrt(g/sigma), isg = 1/sigma
-// and hg = g/(2 sigma) are per-face values. r2 = 1/H, c and the pressure term P =
-// g H^2/(2 sigma) are kept, so that a state differing only in Q (fstate_q)
-// costs four instructions, with the same bits as a full evaluation.
+// and hg = g/(2 sigma) are per-face values. r2 = 1/H, hr = H r, c and the
+// pressure term P = g H^2/(2 sigma) are kept, so that a state differing only
+// in Q (fstate_q) costs four instructions. Sum says which product of u -+ c the
+// wave speeds take unrounded, for each kernel as it is fastest.
+enum class Sum { kRounded, kFusedC, kFusedU };
+
 template <typename T>
 struct FState {
-  T H, Q, u, c, lo, hi, F1, r2, P;
+  T H, Q, u, c, lo, hi, F1, r2, hr, P;
 };
-
-// The state of `b` with its discharge replaced by Q.
-template <typename T>
-__device__ __forceinline__ FState<T> fstate_q(const FState<T> &b, T Q) {
-  FState<T> s = b;
-  s.Q = Q;
-  s.u = Q * b.r2;
-  s.lo = s.u - b.c;
-  s.hi = s.u + b.c;
-  s.F1 = fma(Q, s.u, b.P);
-  return s;
-}
 
 template <typename T>
 struct Face {
@@ -180,16 +181,29 @@ __device__ __forceinline__ Face<T> face(T isg, T cg, T g) {
   return {isg, cg, g, T(0.5) * g * isg};
 }
 
-template <typename T>
+// The state of `b` with its discharge replaced by Q.
+template <Sum S, typename T>
+__device__ __forceinline__ FState<T> fstate_q(const FState<T> &b, T Q, const Face<T> &f) {
+  FState<T> s = b;
+  s.Q = Q;
+  s.u = mul_r(Q, b.r2);
+  s.lo = S == Sum::kFusedC ? fma(-f.cg, b.hr, s.u) : S == Sum::kFusedU ? fma(Q, b.r2, -b.c) : add_r(s.u, -b.c);
+  s.hi = S == Sum::kFusedC ? fma(f.cg, b.hr, s.u) : S == Sum::kFusedU ? fma(Q, b.r2, b.c) : add_r(s.u, b.c);
+  s.F1 = fma(Q, s.u, b.P);
+  return s;
+}
+
+template <Sum S, typename T>
 __device__ __forceinline__ FState<T> fstate(T H, T Q, const Face<T> &f) {
   FState<T> s;
   s.H = H;
   const T r = rsqrt_t(H);
-  s.r2 = r * r;
-  s.c = f.cg * (H * r);
+  s.r2 = mul_r(r, r);
+  s.hr = mul_r(H, r);
+  s.c = mul_r(f.cg, s.hr);
   if constexpr (std::is_same<T, float>::value) s.P = (0.5f * f.g * H) * (H * f.isg);  // as weno3<float>
   else s.P = (f.hg * H) * H;
-  return fstate_q(s, Q);
+  return fstate_q<S>(s, Q, f);
 }
 
 // Ordering keys of FP64 values on the integer pipe (the FP64 pipe is the
@@ -226,8 +240,9 @@ __device__ __forceinline__ void hll_states(const FState<T> &L, const FState<T> &
   } else {
     if constexpr (std::is_same<T, float>::value) {  // as weno3<float>
       const T iw = 1.0f / (SR - SL);
-      F0 = (SR * L.Q - SL * R.Q + SL * SR * (R.H - L.H)) * iw;
-      F1 = (SR * L.F1 - SL * R.F1 + SL * SR * (R.Q - L.Q)) * iw;
+      const T SLR = mul_r(SL, SR);
+      F0 = mul_r(fma(SLR, R.H - L.H, fma(SR, L.Q, -mul_r(SL, R.Q))), iw);
+      F1 = mul_r(fma(SLR, R.Q - L.Q, fma(SR, L.F1, -mul_r(SL, R.F1))), iw);
       return;
     }
     const T w = -SL * rcp_t(SR - SL);
@@ -330,11 +345,25 @@ __device__ __forceinline__ float source_at(const SrcCell<float> &c, float p0, fl
   float S = 0.0f;
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
-    float Hh = float(kLag[q][0]) * p0 + float(kLag[q][1]) * p1 + float(kLag[q][2]) * p2 + float(kLag[q][3]) * p3;
-    float h = Hh * c.is[q];
-    S += 0.5f * c.g * h * h * c.sigx[q] - c.g * Hh * c.bx[q];
+    float Hh = fmaf(float(kLag[q][0]), p0, mul_r(float(kLag[q][1]), p1));
+    Hh = fmaf(float(kLag[q][3]), p3, fmaf(float(kLag[q][2]), p2, Hh));
+    float h = mul_r(Hh, c.is[q]);
+    S = add_r(S, fmaf(mul_r(mul_r(0.5f * c.g, h), h), c.sigx[q], -mul_r(mul_r(c.g, Hh), c.bx[q])));
   }
-  return S * c.hdx;
+  return S;
+}
+
+// The FP32 source_at leaves out the factor dx/2: the source, and d less the
+// source in one rounding.
+__device__ __forceinline__ float source_value(const SrcCell<float> &c, float S) { return mul_r(S, c.hdx); }
+__device__ __forceinline__ float less_source(const SrcCell<float> &c, float d, float S) { return fmaf(-S, c.hdx, d); }
+template <typename T>
+__device__ __forceinline__ T source_value(const SrcCell<T> &, T S) {
+  return S;
+}
+template <typename T>
+__device__ __forceinline__ T less_source(const SrcCell<T> &, T d, T S) {
+  return d - S;
 }
 
 template <typename T>
@@ -570,12 +599,16 @@ __device__ __forceinline__ int rec_variant(int i, int kk) {
 // not perturb that side.
 template <typename T, int FLUX>
 __device__ void jac_pass_b(const Geo &G, const JW<T> &W, int first, int stride) {
+  // The fused forms shorten the FP64 solve's chains: 608 problems of 4096 cells
+  // 365 -> 361 ms.
+  constexpr bool kFused = FLUX == NSWE_FLUX_HLL && std::is_same<T, double>::value;
+  constexpr Sum kBase = kFused ? Sum::kFusedC : Sum::kRounded, kQ = kFused ? Sum::kFusedU : Sum::kRounded;
   const int N = G.N;
   const T g = GeoT<T>::g(G);
   for (int f = first; f <= N; f += stride) {
     const Face<T> fc = face<T>(GeoT<T>::isf(G, f), GeoT<T>::cgf(G, f), g);
-    const FState<T> Lb = fstate<T>(W.r(0, 0, 1, f - 1), W.r(1, 0, 1, f - 1), fc);
-    const FState<T> Rb = fstate<T>(W.r(0, 0, 0, f), W.r(1, 0, 0, f), fc);
+    const FState<T> Lb = fstate<kBase>(W.r(0, 0, 1, f - 1), W.r(1, 0, 1, f - 1), fc);
+    const FState<T> Rb = fstate<kBase>(W.r(0, 0, 0, f), W.r(1, 0, 0, f), fc);
     T F0, F1;
     num_flux<FLUX>(Lb, Rb, G.flux, F0, F1);
     W.f(0, 0, f) = F0;
@@ -590,10 +623,10 @@ __device__ void jac_pass_b(const Geo &G, const JW<T> &W, int first, int stride) 
         // the base state
         FState<T> Ls = Lb, Rs = Rb;
         if (p <= 2)
-          Ls = m == 0 ? fstate<T>(W.r(0, p + 1, 1, f - 1), Lb.Q, fc)
-                      : fstate_q<T>(Lb, W.r(1, p + 1, 1, f - 1));
+          Ls = m == 0 ? fstate<Sum::kFusedC>(W.r(0, p + 1, 1, f - 1), Lb.Q, fc)
+                      : fstate_q<kQ>(Lb, W.r(1, p + 1, 1, f - 1), fc);
         if (p >= 1)
-          Rs = m == 0 ? fstate<T>(W.r(0, p, 0, f), Rb.Q, fc) : fstate_q<T>(Rb, W.r(1, p, 0, f));
+          Rs = m == 0 ? fstate<Sum::kFusedC>(W.r(0, p, 0, f), Rb.Q, fc) : fstate_q<kQ>(Rb, W.r(1, p, 0, f), fc);
         num_flux<FLUX>(Ls, Rs, G.flux, F0, F1);
         const int w = 1 + 2 * p + m;
         W.f(w, 0, f) = F0;
@@ -624,7 +657,8 @@ __device__ double jac_pass_c(const Geo &G, int nb, double eps, double alpha, con
   double acc = 0.0;
   for (int j = first; j < N; j += stride) {
     const SrcCell<T> sc = src_cell<T>(G, j);
-    const T Sb = source_at(sc, W.r(0, 0, 0, j - 1), W.r(0, 0, 0, j), W.r(0, 0, 1, j), W.r(0, 0, 1, j + 1));
+    const T Sb =
+        source_value(sc, source_at(sc, W.r(0, 0, 0, j - 1), W.r(0, 0, 0, j), W.r(0, 0, 1, j), W.r(0, 0, 1, j + 1)));
     const T R0 = W.f(0, 0, j + 1) - W.f(0, 0, j);
     const T R1 = W.f(0, 1, j + 1) - W.f(0, 1, j) - Sb;
     if (Rout) {
@@ -632,7 +666,9 @@ __device__ double jac_pass_c(const Geo &G, int nb, double eps, double alpha, con
       Rout[N + j] = double(R1);
       acc += fabs(double(R0)) + fabs(double(R1));
     }
-    const T reg = Rreg ? T(alpha * (fabs(Rreg[j]) + fabs(Rreg[N + j]))) : T(alpha) * (fabs(R0) + fabs(R1));
+    // on the diagonal: v + alpha ||R_j||_1
+    const T norm = Rreg ? T(alpha * (fabs(Rreg[j]) + fabs(Rreg[N + j]))) : fabs(R0) + fabs(R1);
+    auto regularised = [&](T v) { return Rreg ? add_r(v, norm) : fma(T(alpha), norm, v); };
     for (int k = 0; k < nb; ++k) {
       const int i = j + k - hw;
       if (i < 0 || i >= N) {
@@ -642,18 +678,20 @@ __device__ double jac_pass_c(const Geo &G, int nb, double eps, double alpha, con
       }
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
-        T S = Sb;
-        if (m == 0) {
-          const int v0 = rec_variant(i, j - 1), v1 = rec_variant(i, j), v2 = rec_variant(i, j + 1);
-          S = source_at(sc, W.r(0, v0, 0, j - 1), W.r(0, v1, 0, j), W.r(0, v1, 1, j), W.r(0, v2, 1, j + 1));
-        }
         const int wr = flux_variant(i, m, j + 1), wl = flux_variant(i, m, j);
         const T P0 = W.f(wr, 0, j + 1) - W.f(wl, 0, j);
-        const T P1 = W.f(wr, 1, j + 1) - W.f(wl, 1, j) - S;
-        T v0 = (P0 - R0) * ieps, v1 = (P1 - R1) * ieps;
+        T P1 = W.f(wr, 1, j + 1) - W.f(wl, 1, j);
+        if (m == 0) {
+          const int v0 = rec_variant(i, j - 1), v1 = rec_variant(i, j), v2 = rec_variant(i, j + 1);
+          P1 = less_source(
+              sc, P1, source_at(sc, W.r(0, v0, 0, j - 1), W.r(0, v1, 0, j), W.r(0, v1, 1, j), W.r(0, v2, 1, j + 1)));
+        } else {
+          P1 = P1 - Sb;
+        }
+        T v0 = mul_r(P0 - R0, ieps), v1 = mul_r(P1 - R1, ieps);
         if (i == j) {
-          if (m == 0) v0 += reg;
-          else v1 += reg;
+          if (m == 0) v0 = regularised(v0);
+          else v1 = regularised(v1);
         }
         J[(k * 4 + 0 * 2 + m) * N + j] = v0;
         J[(k * 4 + 1 * 2 + m) * N + j] = v1;
@@ -741,8 +779,8 @@ __device__ void res_pass_b(const Geo &G, const RW &W, int first, int stride) {
   for (int f = first; f <= G.N; f += stride) {
     double F0, F1;
     const Face<double> fc = face(G.isf[f], G.cgf[f], G.g);
-    num_flux<FLUX>(fstate(W.r(0, 1, f - 1), W.r(1, 1, f - 1), fc), fstate(W.r(0, 0, f), W.r(1, 0, f), fc), G.flux, F0,
-                   F1);
+    num_flux<FLUX>(fstate<Sum::kRounded>(W.r(0, 1, f - 1), W.r(1, 1, f - 1), fc),
+                   fstate<Sum::kRounded>(W.r(0, 0, f), W.r(1, 0, f), fc), G.flux, F0, F1);
     W.f(0, f) = F0;
     W.f(1, f) = F1;
   }
@@ -1664,8 +1702,8 @@ __global__ void __launch_bounds__(THREADS) k_residual(const ProbDev *P, int leve
       if (it <= cells) {
         const int f = t0 + it;
         const Face<double> fc = face(G.isf[f], G.cgf[f], G.g);
-        num_flux<-1>(fstate(rec[0][1][it], rec[1][1][it], fc), fstate(rec[0][0][it + 1], rec[1][0][it + 1], fc), G.flux,
-                     flx[0][it], flx[1][it]);
+        num_flux<-1>(fstate<Sum::kRounded>(rec[0][1][it], rec[1][1][it], fc),
+                     fstate<Sum::kRounded>(rec[0][0][it + 1], rec[1][0][it + 1], fc), G.flux, flx[0][it], flx[1][it]);
       } else if (it >= first_src) {
         const int i = it - first_src;
         src[i] = source_at(src_cell<double>(G, t0 + i), rec[0][0][i], rec[0][0][i + 1], rec[0][1][i + 1],
@@ -1986,9 +2024,9 @@ __global__ void __launch_bounds__(THREADS, MINB)
       }
       bool bad = false;
       for (int j = team.tid(); j < N; j += team.size()) {
-        double h = Lv.U[j] + prm.tau * double(x[j]);
+        double h = fma(prm.tau, double(x[j]), Lv.U[j]);
         Lv.U[j] = h;
-        Lv.U[N + j] += prm.tau * double(x[N + j]);
+        Lv.U[N + j] = fma(prm.tau, double(x[N + j]), Lv.U[N + j]);
         if constexpr (kMixed) {
           U32[j] = float(h);
           U32[N + j] = float(Lv.U[N + j]);
