@@ -457,8 +457,11 @@ nswe_status nswe_newton_solve_batch_each(nswe_ctx ctx, int count,
  * problem): shape i has nswe_solve_shape_info(i) threads per block and is
  * built for that many resident blocks per SM. Which shape is fastest depends
  * on the precision, the problem sizes and the batch size; the context keeps
- * one shape per precision (shape 0 until changed), used by
- * nswe_newton_solve and nswe_newton_solve_batch on 1D problems. */
+ * one shape per precision, used by nswe_newton_solve and
+ * nswe_newton_solve_batch on 1D problems. Until one is set or tuned, batches
+ * of at most two problems per SM run in shape 2 and larger ones in shape 0,
+ * and nswe_ctx_get_solve_shape reports 0. Results are the same bits in every
+ * shape. */
 int nswe_solve_shape_count(void);
 nswe_status nswe_solve_shape_info(int shape, int *threads, int *blocks_per_sm);
 nswe_status nswe_ctx_set_solve_shape(nswe_ctx ctx, int precision, int shape);
@@ -608,7 +611,7 @@ size_t nswe_server_footprint_2d(int Nx, int Ny, int levels, int nest_start);
  * EINVAL for a bad config, ENOMEM if an arena cannot be allocated. A 1D
  * launch gives each request one thread block of 128 threads (FP64; the
  * launch shape 128 x 4 of nswe_solve_shape_info) or 256 threads (mixed
- * precision; 256 x 4), or a cluster (nswe_server_set_cluster). */
+ * precision; 256 x 2), or a cluster (nswe_server_set_cluster). */
 nswe_status nswe_server_create(nswe_server *out, int device,
                                const nswe_server_config *cfg);
 

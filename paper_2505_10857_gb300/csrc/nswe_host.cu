@@ -1335,7 +1335,8 @@ nswe_status nswe_ctx_get_solve_cluster(nswe_ctx ctx, int *ctas, int *team_cells)
 
 nswe_status nswe_ctx_get_solve_shape(nswe_ctx ctx, int precision, int *shape) {
   if (!ctx || !shape || (precision != NSWE_PREC_FP64 && precision != NSWE_PREC_MIXED)) return NSWE_EINVAL;
-  *shape = ctx->solve_shape[precision == NSWE_PREC_MIXED ? 1 : 0];
+  const int set = ctx->solve_shape[precision == NSWE_PREC_MIXED ? 1 : 0];
+  *shape = set == kShapeAuto ? 0 : set;
   return NSWE_OK;
 }
 

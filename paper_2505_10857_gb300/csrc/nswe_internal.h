@@ -21,16 +21,24 @@ constexpr int kThreads = NSWE_THREADS;
 constexpr int kSolveShapes = 6;
 constexpr int kSolveShapeThreads[kSolveShapes] = {256, 128, 256, 128, 160, 192};
 constexpr int kSolveShapeBlocks[kSolveShapes] = {4, 8, 2, 4, 4, 4};
+// A context's shape until one is set or tuned: taken by the size of the batch.
+// Up to two problems per SM run the 256 threads with 128 registers each (shape
+// 2) instead of the 64, with spills, that four blocks per SM allow (shape 0):
+// 304 uneven mixed problems 185 -> 114 ms, 100 of 2048 cells 91 -> 56, one of
+// 4096 108 -> 68 (FP64 219 -> 191).
+constexpr int kShapeAuto = -1;
 constexpr int kMaxCoarse = 128;    // max cells of the coarsest level (direct solve)
-// Launch shapes of the serving server's 1D block launches, per precision:
-// 128 x 4 in FP64 (128 registers a thread, no spills), 256 x 4 in mixed
-// precision (the faster of the two there).
+// Launch shapes of the serving server's 1D block launches, per precision, one
+// for launches of every size: 128 x 4 in FP64 and 256 x 2 in mixed precision
+// (128 registers a thread, no spills). Mixed, 1024 requests of 256 to 16384
+// cells, 256 x 4 / 256 x 2: all at once 2220 / 2750 solves/s, at 4000 a second
+// 1680 / 2310, at 500 a second p50 57 / 39 ms.
 constexpr int kServerShapeFp64 = 3;
-constexpr int kServerShapeMixed = 0;
+constexpr int kServerShapeMixed = 2;
 static_assert(kSolveShapeThreads[kServerShapeFp64] == 128 && kSolveShapeBlocks[kServerShapeFp64] == 4,
               "FP64 server shape is 128 x 4");
-static_assert(kSolveShapeThreads[kServerShapeMixed] == 256 && kSolveShapeBlocks[kServerShapeMixed] == 4,
-              "mixed server shape is 256 x 4");
+static_assert(kSolveShapeThreads[kServerShapeMixed] == 256 && kSolveShapeBlocks[kServerShapeMixed] == 2,
+              "mixed server shape is 256 x 2");
 // The latency form of the solve kernel: one problem per thread-block cluster
 // of up to kMaxClusterCtas CTAs of kClusterThreads threads.
 constexpr int kClusterThreads = 128;
@@ -313,7 +321,7 @@ cudaError_t launch_solve(const SolveTask *tasks, int count, const nswe_params &p
                          cudaStream_t s);
 // The same with the coarsest band sized for max_nb (3 or 5) whatever prm
 // says (for batches whose tasks carry their own parameters), in launch shape
-// `shape` (0 .. kSolveShapes-1).
+// `shape` (0 .. kSolveShapes-1, or kShapeAuto).
 // flux: the numerical flux of every task (NSWE_FLUX_HLL, or NSWE_FLUX_LLF,
 // which runs in the default shape).
 cudaError_t launch_solve_sized(const SolveTask *tasks, int count, const nswe_params &prm, int max_coarse_cells,
@@ -349,7 +357,7 @@ struct nswe_ctx_s {
   nswe_info *infos;      // device info records
   nswe_params *prms;     // device per-task parameters (nswe_newton_solve_batch_each)
   int cap;               // capacity of tasks / infos / prms
-  int solve_shape[2];    // launch shape of the 1D solve kernel per precision
+  int solve_shape[2] = {nswe::kShapeAuto, nswe::kShapeAuto};  // launch shape of the 1D solve kernel per precision
   int solve_ctas = 1;    // 1D solves: CTAs per problem (1: a block per problem; 2..16: a cluster)
   int team_cells = 1024; // cluster form: multigrid levels with at least this many cells on every CTA
   int batch2d_lockstep = 1;  // 2D batches: 1 lockstep batched launches (default), 0 concurrent solves

@@ -2219,7 +2219,7 @@ cudaError_t launch_vcycle_f32(const ProbDev *p, int level, int levels, int N, in
 
 cudaError_t launch_solve(const SolveTask *tasks, int count, const nswe_params &prm, int max_coarse_cells,
                          cudaStream_t s) {
-  return launch_solve_sized(tasks, count, prm, max_coarse_cells, prm.jacobian == NSWE_JAC_FULL ? 5 : 3, 0, s);
+  return launch_solve_sized(tasks, count, prm, max_coarse_cells, prm.jacobian == NSWE_JAC_FULL ? 5 : 3, kShapeAuto, s);
 }
 
 namespace {
@@ -2267,12 +2267,7 @@ cudaError_t launch_solve_sized(const SolveTask *tasks, int count, const nswe_par
     launch_shape<0, NSWE_FLUX_LLF>(tasks, count, prm, n_cap, ldab_cap, smem, s);
     return cudaGetLastError();
   }
-  // Up to two problems per SM take the default 256 threads with 128 registers
-  // each (shape 2) instead of the 64, with spills, that four blocks per SM
-  // allow. With the legs of the mixed block form: 304 uneven mixed problems
-  // 185 -> 114 ms, 100 of 2048 cells 91 -> 56, one of 4096 108 -> 68 (FP64 219
-  // -> 191); beyond two per SM the legs alone, 608 of 4096 cells 195 -> 159.
-  if (shape == 0 && count <= 2 * kSmCount) shape = 2;
+  if (shape == kShapeAuto) shape = count <= 2 * kSmCount ? 2 : 0;
   switch (shape) {
   case 1: launch_shape<1>(tasks, count, prm, n_cap, ldab_cap, smem, s); break;
   case 2: launch_shape<2>(tasks, count, prm, n_cap, ldab_cap, smem, s); break;
