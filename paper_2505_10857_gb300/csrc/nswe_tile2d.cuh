@@ -241,14 +241,14 @@ template <int SIDE, bool FROZEN>
 __device__ __forceinline__ double weno2_value(double a, double b, double c, double s0, double s1, double w) {
   if (SIDE == 0) {
     const double q0 = fma(0.5, b, 0.5 * c), q1 = fma(1.5, b, -0.5 * a);
-    return (FROZEN ? fma(s0, q1, __dmul_rn(2.0 * s1, q0)) : fma(2.0 * s1, q0, __dmul_rn(s0, q1))) * w;
+    return __dmul_rn(FROZEN ? fma(s0, q1, __dmul_rn(2.0 * s1, q0)) : fma(2.0 * s1, q0, __dmul_rn(s0, q1)), w);
   }
   const double p0 = fma(1.5, b, -0.5 * c), p1 = fma(0.5, a, 0.5 * b);
-  return fma(s1, p0, __dmul_rn(2.0 * s0, p1)) * w;
+  return __dmul_rn(fma(s1, p0, __dmul_rn(2.0 * s0, p1)), w);
 }
 
 __device__ __forceinline__ void from_char2(const Eig2 &e, const double Wr[3], double out[3]) {
-  out[0] = Wr[0] + Wr[2];
+  out[0] = __dadd_rn(Wr[0], Wr[2]);
   out[1] = fma(e.un - e.c, Wr[0], __dmul_rn(e.un + e.c, Wr[2]));
   out[2] = fma(e.ut, Wr[2], fma(e.ut, Wr[0], Wr[1]));
 }
