@@ -15,9 +15,11 @@
 //   sqrt(x): two steps of Heron's iteration s + (x - s^2) / (2 s) with 1/(2 s)
 //            from the seed, the residual x - s^2 formed exactly by an FMA;
 //   a / b:   q = a (1/b) and one correction by the exact residual a - b q.
-// Against the correctly rounded operations, over 4e7 random arguments: the
-// reciprocal differs (in the last bit) in 0.03 % of cases, the square root in
-// 0.04 %, the division in none.
+// Against the correctly rounded operations, 2e6 random arguments each: the
+// reciprocal differs (by one in the last place) in 0.03 % of cases, the square
+// root in 0.04 %, the division in none for exponents near zero and in 0.01 %
+// over all exponents (subnormal residuals); the reciprocal square root is
+// within 0.99 ulp of the exact value (tests/test_gpu_fp64.py).
 //
 // Arguments outside the normal range, whose result would not be a normal
 // number, take the ordinary operation (an integer test of the exponent), so
@@ -48,12 +50,14 @@ __device__ __forceinline__ double fast_sqrt(double x) {
   return fma(fma(-s, s, x), h, s);
 }
 
-// a / b with rb = 1.0 / b given; b and rb normal.
+__device__ __forceinline__ bool fp64_zero(double x) { return ((__double2hiint(x) << 1) | __double2loint(x)) == 0; }
+
+// a / b with rb = 1.0 / b given.
 __device__ __forceinline__ double fast_div(double a, double b, double rb) {
   const double q = a * rb;
   const unsigned eq = fp64_exponent(q);
-  if (eq - 64u > 1919u)  // a quotient that is tiny, huge or not finite; a zero is already right
-    return ((__double2hiint(a) << 1) | __double2loint(a)) == 0 ? q : a / b;
+  if (eq - 64u > 1919u)  // a quotient that is tiny, huge or not finite; zero over a finite rb is already right
+    return fp64_zero(a) && fp64_zero(q) ? q : a / b;
   return fma(fma(-b, q, a), rb, q);
 }
 
