@@ -224,7 +224,7 @@ nswe_status lockstep_t(nswe_ctx ctx, int count, const nswe_prob *probs, const do
     // V-cycles run at once on nine clusters' worth of SMs
     int nvc = 0;
     for (size_t a = 0; a < act.size(); ++a) nvc += lev[a] < probs[act[a]]->levels - 1 ? 1 : 0;
-    int tail_ctas = kTail2MaxCtas;
+    int tail_ctas = ctx->max_cluster;
     while (tail_ctas > 2 && tail_ctas * nvc > 144) tail_ctas /= 2;
     int used_ctas = 1, tail_threads = 0;
     size_t tail_smem = 0;

@@ -289,7 +289,7 @@ Tail2<T> tail2_of(const nswe_prob_s *p, const MG2<T> &m, long tail) {
   }
   t.A = reinterpret_cast<const T *>(p->dense);
   t.piv = p->piv;
-  plan_tail2<T>(t, m.l0, m.lv[m.l0].cm, tail, kTail2MaxCtas);
+  plan_tail2<T>(t, m.l0, m.lv[m.l0].cm, tail, p->ctx->max_cluster);
   return t;
 }
 
@@ -374,7 +374,7 @@ nswe_status solve2d_t(nswe_prob_s *p, const double *U0, double *U, const nswe_pa
     // the tail's levels, nor on the coarsest, whose J the dense LU reads).
     const int minc = p->ctx->cm2d_min_cells;
     const int cm = (l < L && st0 == ST_J9 && minc >= 0 && n >= minc &&
-                    tail2_first<T>(p, l, st0, tail, kTail2MaxCtas) > l)
+                    tail2_first<T>(p, l, st0, tail, p->ctx->max_cluster) > l)
                        ? 1
                        : 0;
     T *const J = reinterpret_cast<T *>(Lv.J);
@@ -552,7 +552,7 @@ nswe_status vcycle2d_entry(nswe_ctx ctx, nswe_prob prob, int level, int nb, cons
   // first: a colour pass then reads a third of it instead of every sector
   // (512 x 256: 12.6 us instead of 14.2, the V-cycle 6.51 -> 6.16 ms).
   const bool cm = level < prob->levels - 1 && st == ST_J9 && minc >= 0 && (long)Nx * Ny >= minc &&
-                  tail2_first<T>(prob, level, st, tail, kTail2MaxCtas) > level;
+                  tail2_first<T>(prob, level, st, tail, ctx->max_cluster) > level;
   if (cm) {
     T *const Jcm = reinterpret_cast<T *>(prob->host2.lev[level].J);
     if (launch2_colour_major<T>(Nx, Ny, J, Jcm, ctx->stream) != cudaSuccess) return NSWE_ECUDA;
@@ -633,6 +633,7 @@ nswe_status nswe_ctx_create(nswe_ctx *out, int device, void *stream) {
   if (!c) return NSWE_ENOMEM;
   c->device = device;
   c->stream = (cudaStream_t)stream;
+  c->max_cluster = max_cluster_ctas();
   if (cudaMalloc(&c->partials, sizeof(double) * 1024) != cudaSuccess ||
       cudaMalloc(&c->status, sizeof(int) * 4) != cudaSuccess) {
     cudaFree(c->partials);
@@ -974,7 +975,7 @@ nswe_status nswe_residual(nswe_ctx ctx, nswe_prob prob, int level, const double 
                ? NSWE_OK
                : NSWE_ECUDA;
   int N = prob->N >> level;
-  return launch_residual(prob->dev, level, N, U, R, res_l1, ctx->partials, ctx->stream) == cudaSuccess
+  return launch_residual(prob->dev, level, N, U, R, res_l1, ctx->partials, ctx->max_cluster, ctx->stream) == cudaSuccess
              ? NSWE_OK
              : NSWE_ECUDA;
 }
@@ -1031,7 +1032,8 @@ nswe_status nswe_jacobian_f32(nswe_ctx ctx, nswe_prob prob, int level, int nb, c
   }
   if (nb != 3 && nb != 5) return NSWE_EINVAL;
   const int N = prob->N >> level;
-  return launch_jacobian_f32(prob->dev, level, N, nb, U, eps, alpha, R, J, res_l1, ctx->partials, ctx->stream) ==
+  return launch_jacobian_f32(prob->dev, level, N, nb, U, eps, alpha, R, J, res_l1, ctx->partials, ctx->max_cluster,
+                             ctx->stream) ==
                  cudaSuccess
              ? NSWE_OK
              : NSWE_ECUDA;
@@ -1046,7 +1048,7 @@ nswe_status nswe_mg_vcycle_f32(nswe_ctx ctx, nswe_prob prob, int level, int nb, 
   if (prob->dim == 2) return vcycle2d_entry<float>(ctx, prob, level, nb, J, R, dU, *params);
   if (nb != 3 && nb != 5) return NSWE_EINVAL;
   return launch_vcycle_f32(prob->dev, level, prob->levels, prob->N >> level, nb, J, R, dU, *params, ctx->status,
-                           ctx->stream) == cudaSuccess
+                           ctx->max_cluster, ctx->stream) == cudaSuccess
              ? NSWE_OK
              : NSWE_ECUDA;
 }
@@ -1060,7 +1062,7 @@ nswe_status nswe_mg_vcycle(nswe_ctx ctx, nswe_prob prob, int level, int nb, cons
   if (prob->dim == 2) return vcycle2d_entry<double>(ctx, prob, level, nb, J, R, dU, *params);
   if (nb != 3 && nb != 5) return NSWE_EINVAL;
   return launch_vcycle(prob->dev, level, prob->levels, prob->N >> level, nb, J, R, dU, *params, ctx->status,
-                       ctx->stream) == cudaSuccess
+                       ctx->max_cluster, ctx->stream) == cudaSuccess
              ? NSWE_OK
              : NSWE_ECUDA;
 }

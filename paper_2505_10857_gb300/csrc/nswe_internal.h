@@ -44,6 +44,10 @@ static_assert(kSolveShapeThreads[kServerShapeMixed] == 256 && kSolveShapeBlocks[
 constexpr int kClusterThreads = 128;
 constexpr int kMaxClusterCtas = 16;
 
+// The largest cluster (16, 8, 4, 2 or 1) that the current device can hold of
+// CTAs that take an SM each.
+int max_cluster_ctas();
+
 // One nested / multigrid level of a 1D problem. Geometry is read-only input;
 // the rest is solver workspace owned by the problem.
 struct LevelDev {
@@ -160,7 +164,7 @@ cudaError_t launch2_to_f32(long count, const double *src, float *dst, cudaStream
 
 // The levels ls..L of a 2D V-cycle (down-leg, coarsest solve with the dense
 // factors A/piv, up-leg) run by one thread-block cluster (nswe_cluster2d.cuh).
-constexpr int kTail2Threads = 512, kTail2MaxCtas = 16;
+constexpr int kTail2Threads = 512;
 // Levels of at most this many cells go to the cluster unless a threshold was
 // set (and if their bands fit its shared memory). FP32 levels gain whatever
 // their size; in FP64 the arithmetic of a larger level wants more than the 16
@@ -301,20 +305,21 @@ struct SolveTask {
 cudaError_t launch_geom_derive(const ProbDev *p, int finest_cells, cudaStream_t s);
 // The derived geometry of tasks[0..count).prob, one block each.
 cudaError_t launch_geom_derive_batch(const SolveTask *tasks, int count, cudaStream_t s);
+// max_ctas (here and below): the largest cluster a launch may take (the context's max_cluster).
 cudaError_t launch_residual(const ProbDev *p, int level, int N, const double *U, double *R, double *res,
-                            double *partials, cudaStream_t s);
+                            double *partials, int max_ctas, cudaStream_t s);
 cudaError_t launch_jacobian(const ProbDev *p, int level, int N, int nb, const double *U, double eps,
                             double alpha, double *R, double *J, double *res, double *partials,
                             cudaStream_t s);
 // FP64 residual (R, res) then the FP32 Jacobian regularised with that R.
 cudaError_t launch_jacobian_f32(const ProbDev *p, int level, int N, int nb, const double *U, double eps,
-                                double alpha, double *R, float *J, double *res, double *partials,
+                                double alpha, double *R, float *J, double *res, double *partials, int max_ctas,
                                 cudaStream_t s);
 // One V-cycle from `level` (N cells) of a problem of `levels` levels.
 cudaError_t launch_vcycle(const ProbDev *p, int level, int levels, int N, int nb, const double *J, const double *R,
-                          double *dU, const nswe_params &prm, int *status, cudaStream_t s);
+                          double *dU, const nswe_params &prm, int *status, int max_ctas, cudaStream_t s);
 cudaError_t launch_vcycle_f32(const ProbDev *p, int level, int levels, int N, int nb, const float *J, const float *R,
-                              float *dU, const nswe_params &prm, int *status, cudaStream_t s);
+                              float *dU, const nswe_params &prm, int *status, int max_ctas, cudaStream_t s);
 // max_coarse_cells: largest coarsest level over the tasks; prm.precision
 // selects the FP64 or the mixed-precision solve kernel.
 cudaError_t launch_solve(const SolveTask *tasks, int count, const nswe_params &prm, int max_coarse_cells,
@@ -359,6 +364,7 @@ struct nswe_ctx_s {
   int cap;               // capacity of tasks / infos / prms
   int solve_shape[2] = {nswe::kShapeAuto, nswe::kShapeAuto};  // launch shape of the 1D solve kernel per precision
   int solve_ctas = 1;    // 1D solves: CTAs per problem (1: a block per problem; 2..16: a cluster)
+  int max_cluster = nswe::kMaxClusterCtas;  // max_cluster_ctas() of the device
   int team_cells = 1024; // cluster form: multigrid levels with at least this many cells on every CTA
   int batch2d_lockstep = 1;  // 2D batches: 1 lockstep batched launches (default), 0 concurrent solves
   int cm2d_min_cells = 131072;  // 2D Newton levels of at least this many cells store J9 colour-major

@@ -2122,7 +2122,7 @@ cudaError_t launch_geom_derive_batch(const SolveTask *tasks, int count, cudaStre
 }
 
 cudaError_t launch_residual(const ProbDev *p, int level, int N, const double *U, double *R, double *res,
-                            double *partials, cudaStream_t s) {
+                            double *partials, int max_ctas, cudaStream_t s) {
   const int small = (N + kResTileSmall - 1) / kResTileSmall;
   if (small > 4 * kSmCount) {
     const int tiles = (N + kResTile - 1) / kResTile, grid = tiles < kResMaxBlocks ? tiles : kResMaxBlocks;
@@ -2131,7 +2131,7 @@ cudaError_t launch_residual(const ProbDev *p, int level, int N, const double *U,
     return cudaGetLastError();
   }
   auto kern = k_residual<kResTileSmall, kResThreadsSmall>;
-  if (!res || small > kMaxClusterCtas) {
+  if (!res || small > max_ctas) {
     kern<<<small, kResThreadsSmall, 0, s>>>(p, level, U, R, partials, nullptr);
     if (res) k_finish_res<<<1, kThreads, 0, s>>>(partials, small, N, res);
     return cudaGetLastError();
@@ -2156,10 +2156,11 @@ cudaError_t launch_jacobian(const ProbDev *p, int level, int N, int nb, const do
 }
 
 cudaError_t launch_jacobian_f32(const ProbDev *p, int level, int N, int nb, const double *U, double eps,
-                                double alpha, double *R, float *J, double *res, double *partials, cudaStream_t s) {
+                                double alpha, double *R, float *J, double *res, double *partials, int max_ctas,
+                                cudaStream_t s) {
   // The residual's reduction has consumed `partials` (stream order) before
   // the FP32 pass C reuses it (it writes zeros there).
-  cudaError_t e = launch_residual(p, level, N, U, R, res, partials, s);
+  cudaError_t e = launch_residual(p, level, N, U, R, res, partials, max_ctas, s);
   if (e != cudaSuccess) return e;
   k_jac_a<float><<<grid_for((N + 2) * 2), kThreads, 0, s>>>(p, level, U, eps);
   k_jac_b<float><<<grid_for(N + 1), kThreads, 0, s>>>(p, level);
@@ -2174,7 +2175,7 @@ size_t band_smem_bytes(int n_cap, int ldab_cap) {
 namespace {
 template <typename T>
 cudaError_t vcycle_t(const ProbDev *p, int level, int levels, int N, int nb, const T *J, const T *R, T *dU,
-                     const nswe_params &prm, int *status, cudaStream_t s) {
+                     const nswe_params &prm, int *status, int max_ctas, cudaStream_t s) {
   const int L = levels - 1, NL = N >> (L - level), n_cap = 2 * NL;
   const int ldab_cap = 3 * (level == L && nb == 5 ? 5 : 3) + 1;
   const size_t smem = band_smem_bytes(n_cap, ldab_cap);
@@ -2194,7 +2195,7 @@ cudaError_t vcycle_t(const ProbDev *p, int level, int levels, int N, int nb, con
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute at[2];
-  cudaLaunchConfig_t cfg = cluster_config(kMaxClusterCtas, kMaxClusterCtas, kVcThreads, smem, s, at);
+  cudaLaunchConfig_t cfg = cluster_config(max_ctas, max_ctas, kVcThreads, smem, s, at);
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -2208,13 +2209,13 @@ cudaError_t vcycle_t(const ProbDev *p, int level, int levels, int N, int nb, con
 }  // namespace
 
 cudaError_t launch_vcycle(const ProbDev *p, int level, int levels, int N, int nb, const double *J, const double *R,
-                          double *dU, const nswe_params &prm, int *status, cudaStream_t s) {
-  return vcycle_t<double>(p, level, levels, N, nb, J, R, dU, prm, status, s);
+                          double *dU, const nswe_params &prm, int *status, int max_ctas, cudaStream_t s) {
+  return vcycle_t<double>(p, level, levels, N, nb, J, R, dU, prm, status, max_ctas, s);
 }
 
 cudaError_t launch_vcycle_f32(const ProbDev *p, int level, int levels, int N, int nb, const float *J, const float *R,
-                              float *dU, const nswe_params &prm, int *status, cudaStream_t s) {
-  return vcycle_t<float>(p, level, levels, N, nb, J, R, dU, prm, status, s);
+                              float *dU, const nswe_params &prm, int *status, int max_ctas, cudaStream_t s) {
+  return vcycle_t<float>(p, level, levels, N, nb, J, R, dU, prm, status, max_ctas, s);
 }
 
 cudaError_t launch_solve(const SolveTask *tasks, int count, const nswe_params &prm, int max_coarse_cells,

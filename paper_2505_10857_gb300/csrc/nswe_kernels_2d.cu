@@ -1060,6 +1060,36 @@ cudaError_t launch_clusters2(std::atomic<unsigned> &raised, void (*kern)(KArgs..
 }
 }  // namespace
 
+int max_cluster_ctas() {
+  static std::atomic<unsigned> raised{0};
+  static std::atomic<int> known[32];  // per device; 0: not asked yet
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  std::atomic<int> *slot = dev < 32 ? known + dev : nullptr;
+  int n = slot ? slot->load(std::memory_order_relaxed) : 0;
+  if (n) return n;
+  auto kern = k2_vcycle_tail<double>;
+  n = raise_smem(raised, kern, true) == cudaSuccess ? kMaxClusterCtas : 1;
+  for (; n > 1; n /= 2) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)n, 1, 1);
+    cfg.blockDim = dim3(kTail2Threads, 1, 1);
+    cfg.dynamicSmemBytes = kTile2MaxSmem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)n;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters > 0) break;
+    (void)cudaGetLastError();
+  }
+  if (slot) slot->store(n, std::memory_order_relaxed);
+  return n;
+}
+
 template <typename T>
 cudaError_t launch2_vcycle_tail(const Tail2<T> &t, int nu1, int nu2, double omega, int Kc, int cycles,
                                 bool after_factor, cudaStream_t s) {
