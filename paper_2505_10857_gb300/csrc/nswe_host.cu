@@ -69,7 +69,7 @@ size_t nswe::prob2d_arena_doubles(int Nx, int Ny, int levels) {
     nk += 2 * (size_t)((Nx >> l) + (Ny >> l));
   }
   const size_t N3 = 3 * (size_t)(Nx >> (levels - 1)) * (Ny >> (levels - 1));
-  return doubles + round_up(N3 * N3) + round_up(N3) + 2 * round_up(nk);
+  return doubles + round_up(N3 * N3) + 2 * round_up(nk);
 }
 
 // All device bytes nswe_prob_create_2d requests for such a problem.
@@ -955,7 +955,6 @@ nswe_status nswe_prob_create_2d(nswe_ctx ctx, nswe_prob *out, int Nx, int Ny, in
   }
   p->dense = a;
   a += round_up(N3 * N3);
-  a += round_up(N3);
   if (cudaMemcpyAsync(kind_dev, kinds.data(), sizeof(int) * nk, cudaMemcpyHostToDevice, ctx->stream)) ok = false;
   if (cudaMemcpyAsync(p->dev2, &p->host2, sizeof(ProbDev2), cudaMemcpyHostToDevice, ctx->stream)) ok = false;
   if (!ok || cudaStreamSynchronize(ctx->stream) != cudaSuccess) {
@@ -1083,7 +1082,7 @@ nswe_status nswe_mg_smooth(nswe_ctx ctx, nswe_prob prob, int level, int nb, cons
   resolve2d(prob, *params, prm, tail);
   Lev2<double> Lv{L.Nx, L.Ny, const_cast<double *>(J), L.Dinv, const_cast<double *>(R), dU, colour_major};
   int count = 0;
-  if (launch2_dinv<double>(L.Nx, L.Ny, stc, J, L.Dinv, colour_major, ctx->stream) != cudaSuccess ||
+  if (launch2_dinv(L.Nx, L.Ny, stc, J, L.Dinv, colour_major, ctx->stream) != cudaSuccess ||
       smooth2<double>(Lv, stc, prm.nu1, prm.omega, prm.colours2d, ctx->stream, &count) != cudaSuccess)
     return NSWE_ECUDA;
   if (launches) *launches = count;

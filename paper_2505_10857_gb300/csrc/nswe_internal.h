@@ -138,8 +138,7 @@ cudaError_t launch2_jacobian(const ProbDev2 *p, int level, int Nx, int Ny, int s
                              double alpha, const double *R, TJ *J, bool frozen, int cm, cudaStream_t s);
 template <typename T>
 cudaError_t launch2_coarse_op(int Nx, int Ny, int st, const T *Jf, T *Jc, int cm, cudaStream_t s);
-template <typename T>
-cudaError_t launch2_dinv(int Nx, int Ny, int st, const T *J, T *Dinv, int cm, cudaStream_t s);
+cudaError_t launch2_dinv(int Nx, int Ny, int st, const double *J, double *Dinv, int cm, cudaStream_t s);
 // mode 0: cells of colour col of the stencil's colouring; mode 1 / 2: of the
 // diagonal colourings (i + j) mod Kc / (j - i + Nx - 1) mod Kc. early: the
 // launch before it on the stream is a pass of the same smoothing.

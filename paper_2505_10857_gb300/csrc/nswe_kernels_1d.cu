@@ -419,8 +419,6 @@ struct BlockTeam {
   // the same sum in every thread (fixed order)
   __device__ __forceinline__ double sum(double v, double *red) const { return block_sum(v, red); }
   __device__ __forceinline__ bool any(bool b) const { return __syncthreads_or(b) != 0; }
-  // the leader's value of a flag in every thread (after the leader wrote it)
-  __device__ __forceinline__ int lead_value(const int *flag) const { return *flag; }
 };
 
 struct ClusterTeam {
@@ -453,6 +451,7 @@ struct ClusterTeam {
     sync();
     return a != 0;
   }
+  // the leader's value of a flag in every thread (after the leader wrote it)
   __device__ int lead_value(const int *flag) const {
     const int v = *cooperative_groups::this_cluster().map_shared_rank(const_cast<int *>(flag), 0);
     sync();
@@ -1015,9 +1014,6 @@ struct Band {
 // to 0, so a NaN never wins a pivot search).
 __device__ __forceinline__ unsigned long long abs_key(double a) {
   return a == a ? (unsigned long long)(__double_as_longlong(a) & 0x7fffffffffffffffLL) : 0ull;
-}
-__device__ __forceinline__ unsigned long long abs_key(float a) {
-  return a == a ? (unsigned long long)(__float_as_uint(a) & 0x7fffffffu) : 0ull;
 }
 
 // Pivot steps k0 .. k1 - 1 of the factorisation by warp 0 (lanes 0..31, all of

@@ -243,10 +243,9 @@ __device__ __forceinline__ void dinv_cells2(int Nx, int Ny, int st, const T *J, 
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k2_dinv(int Nx, int Ny, int st, const T *J, T *Dinv, int cm) {
+__global__ void __launch_bounds__(kThreads) k2_dinv(int Nx, int Ny, int st, const double *J, double *Dinv, int cm) {
   pdl_enter();
-  dinv_cells2<T>(Nx, Ny, st, J, Dinv, cm, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  dinv_cells2<double>(Nx, Ny, st, J, Dinv, cm, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 // The inverse diagonal blocks of the levels l0 .. L - 1 of a hierarchy in one
@@ -450,8 +449,6 @@ __global__ void __launch_bounds__(kThreads) k2_prolong(int Nx, int Ny, T *dU, co
   prolong_cells2<T>(Nx, Ny, dU, dUc, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
-// Dense system A (row-major, unknown 3c+m) assembled from a block operator:
-// zero it, then scatter the blocks.
 // A cell-contiguous J9 (81 planes) in colour-major storage. Items run along
 // the destination's rows (plane, colour, row j, slot), so writes coalesce; the
 // reads of a row's three colours share their sectors through L2.
@@ -468,6 +465,8 @@ __global__ void __launch_bounds__(kThreads) k2_colour_major(int Nx, int Ny, cons
   }
 }
 
+// Dense system A (row-major, unknown 3c+m) assembled from a block operator:
+// zero it, then scatter the blocks.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k2_zero(long count, T *A) {
   pdl_enter();
@@ -884,9 +883,8 @@ cudaError_t launch2_coarse_op(int Nx, int Ny, int st, const T *Jf, T *Jc, int cm
   return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch2_dinv(int Nx, int Ny, int st, const T *J, T *Dinv, int cm, cudaStream_t s) {
-  launchk2(k2_dinv<T>, grid2((long)Nx * Ny), kThreads, s, Nx, Ny, st, J, Dinv, cm);
+cudaError_t launch2_dinv(int Nx, int Ny, int st, const double *J, double *Dinv, int cm, cudaStream_t s) {
+  launchk2(k2_dinv, grid2((long)Nx * Ny), kThreads, s, Nx, Ny, st, J, Dinv, cm);
   return cudaGetLastError();
 }
 
@@ -1107,7 +1105,6 @@ cudaError_t launch2_to_f32(long count, const double *src, float *dst, cudaStream
   template cudaError_t launch2_jacobian<T>(const ProbDev2 *, int, int, int, int, const double *, double, double, \
                                            const double *, T *, bool, int, cudaStream_t);                        \
   template cudaError_t launch2_coarse_op<T>(int, int, int, const T *, T *, int, cudaStream_t);                   \
-  template cudaError_t launch2_dinv<T>(int, int, int, const T *, T *, int, cudaStream_t);                        \
   template cudaError_t launch2_sor<T>(int, int, int, const T *, const T *, const T *, T *, double, int, int, int, \
                                       int, int, bool, cudaStream_t);                                             \
   template cudaError_t launch2_restrict<T>(int, int, int, const T *, const T *, const T *, T *, T *, int,        \
