@@ -677,16 +677,15 @@ __device__ double jac_pass_c(const Geo &G, int nb, double eps, double alpha, con
       }
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
-        const int wr = flux_variant(i, m, j + 1), wl = flux_variant(i, m, j);
-        const T P0 = W.f(wr, 0, j + 1) - W.f(wl, 0, j);
-        T P1 = W.f(wr, 1, j + 1) - W.f(wl, 1, j);
+        T S = Sb;
         if (m == 0) {
           const int v0 = rec_variant(i, j - 1), v1 = rec_variant(i, j), v2 = rec_variant(i, j + 1);
-          P1 = less_source(
-              sc, P1, source_at(sc, W.r(0, v0, 0, j - 1), W.r(0, v1, 0, j), W.r(0, v1, 1, j), W.r(0, v2, 1, j + 1)));
-        } else {
-          P1 = P1 - Sb;
+          S = source_at(sc, W.r(0, v0, 0, j - 1), W.r(0, v1, 0, j), W.r(0, v1, 1, j), W.r(0, v2, 1, j + 1));
         }
+        const int wr = flux_variant(i, m, j + 1), wl = flux_variant(i, m, j);
+        const T P0 = W.f(wr, 0, j + 1) - W.f(wl, 0, j);
+        const T d1 = W.f(wr, 1, j + 1) - W.f(wl, 1, j);
+        const T P1 = m == 0 ? less_source(sc, d1, S) : d1 - S;
         T v0 = mul_r(P0 - R0, ieps), v1 = mul_r(P1 - R1, ieps);
         if (i == j) {
           if (m == 0) v0 = regularised(v0);
