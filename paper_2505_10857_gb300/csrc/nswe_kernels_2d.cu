@@ -1067,8 +1067,9 @@ int max_cluster_ctas() {
   int n = slot ? slot->load(std::memory_order_relaxed) : 0;
   if (n) return n;
   auto kern = k2_vcycle_tail<double>;
-  n = raise_smem(raised, kern, true) == cudaSuccess ? kMaxClusterCtas : 1;
-  for (; n > 1; n /= 2) {
+  const bool raisable = raise_smem(raised, kern, true) == cudaSuccess;
+  if (!raisable) (void)cudaGetLastError();
+  for (n = raisable ? kMaxClusterCtas : 1; n > 1; n /= 2) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)n, 1, 1);
     cfg.blockDim = dim3(kTail2Threads, 1, 1);
