@@ -1778,7 +1778,7 @@ __global__ void __launch_bounds__(kThreads) k_jac_c(const ProbDev *P, int level,
 // the Jacobian workspace), then k_vc_cluster with the levels that one cluster
 // of 16 blocks takes, started beside the factorisation; larger levels are
 // launches of their own before and after it (k_vc_leg). One block for all of
-// it took 513 us for 4096 cells, this 146.
+// it took 513 us for 4096 cells, this 121.
 // The factors lie at the front of the workspace: ab, rinv, piv of Band.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_vc_setup(const ProbDev *P, int level, int nb, const T *J,
