@@ -434,7 +434,7 @@ def run_gpu(args, rank, world, local_rank):
 
     # Launch-shape autotuning on this batch (before the warm-up; not timed).
     tune = None
-    shape = 0
+    shape = None  # the context's own choice by the batch's size
     if args.shape is not None:
         shape = args.shape
         nswe.nswe_ctx_set_solve_shape(ctx, prm.precision, shape)
@@ -444,8 +444,9 @@ def run_gpu(args, rank, world, local_rank):
                 "chosen": "%dx%d" % nswe.solve_shapes()[best],
                 "what": "threads per block x resident blocks per SM of k_solve, one timed batch each"}
         shape = best
-    shape_name = "%dx%d" % nswe.solve_shapes()[shape]
-    if pipelined:
+    default = 2 if len(inps) <= 304 else 0
+    shape_name = "%dx%d" % nswe.solve_shapes()[default if shape is None else shape]
+    if pipelined and shape is not None:
         nswe.nswe_ctx_set_solve_shape(ctx_b, prm.precision, shape)
 
     def barrier():
